@@ -69,141 +69,187 @@ __global__ void widen(const float* __restrict__ V32, int N, int n, double* __res
   }
 }
 
-// The record of slot (x, y) (x the slot's first index) for the FP32 inner
-// sweep: Algorithm 2 with the skip test of Algorithm 4 (compared in squares),
-// t in the stable form, c = 1 / sqrt(1 + t^2) by rsqrtf, c - 1 = -t^2 c / (1 + h)
-// with h = 1 / c = (1 + t^2) c; the new diagonal a_pp - t a_pq, a_qq + t a_pq.
-MPJ_DEV void rec32(int x, int y, float dxx, float dyy, float axy, float skip, RotRec<float>& rr) {
-  const bool xp = x < y;
-  const float app = xp ? dxx : dyy, aqq = xp ? dyy : dxx;
+// The rotation of pair (p, q), p < q, for the FP32 inner sweep: Algorithm 2
+// with the skip test of Algorithm 4 (compared in squares), t in the stable
+// form, c = 1 / sqrt(1 + t^2) by rsqrtf, c - 1 = -t^2 c / (1 + h) with
+// h = 1 / c = (1 + t^2) c; the new diagonal a_pp - t a_pq, a_qq + t a_pq.  The
+// approximate divisions and square roots (2 ulp) only perturb the angle: the
+// stage delivers Q_l to single precision and c, s belong to the same t.
+struct Rot32 {
+  float cm1, sig;
+};
+MPJ_DEV float sqrt_approx(float x) {
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+MPJ_DEV bool rot32(float& app, float& aqq, float apq, float skip, Rot32& rr) {
   rr.cm1 = 0.0f;
   rr.sig = 0.0f;
-  rr.dx = dxx;
-  rr.dy = dyy;
-  if (!(axy * axy > (skip * skip) * fabsf(app * aqq)) || y >= W2 || x >= W2) return;
-  const float tau = (aqq - app) / (2.0f * axy);
-  const float r = sqrtf(fmaf(tau, tau, 1.0f));
-  const float t = (tau >= 0.0f) ? 1.0f / (tau + r) : 1.0f / (tau - r);
+  if (!(apq * apq > (skip * skip) * fabsf(app * aqq))) return false;
+  const float tau = __fdividef(aqq - app, 2.0f * apq);
+  const float r = sqrt_approx(fmaf(tau, tau, 1.0f));
+  const float ta = __fdividef(1.0f, fabsf(tau) + r);
+  const float t = (tau >= 0.0f) ? ta : -ta;
   const float w = fmaf(t, t, 1.0f);
   const float c = rsqrtf(w);
   const float h = w * c;
-  const float s = t * c;
-  rr.cm1 = -(t * t) * c / (1.0f + h);
-  rr.sig = xp ? s : -s;
-  const float np = app - t * axy, nq = aqq + t * axy;
-  rr.dx = xp ? np : nq;
-  rr.dy = xp ? nq : np;
+  rr.cm1 = -(t * t) * __fdividef(c, 1.0f + h);
+  rr.sig = t * c;
+  app = fmaf(-t, apq, app);
+  aqq = fmaf(t, apq, aqq);
+  return true;
 }
 
-// One CTA per block pair of outer round R: inner round-robin sweep on the
-// 32 x 32 subproblem; writes the rotated subproblem S (column-major), the
-// accumulated U (row-major for the FP32 products, column-major, urow false,
-// for the tensor-core panel) and the set T of its indices that rotated
-// (Mbuf, bit l for local index l, if not null): U is the identity outside
-// T x T.
-constexpr int S32_THREADS = 512;
+// One entry of a rotated pair: `own` with the other index's entry `oth`
+// (sg = -sig for the pair's first index, +sig for its second).
+MPJ_DEV float rot_one(float cm1, float sg, float own, float oth) { return fmaf(cm1, own, fmaf(sg, oth, own)); }
+
+// v with a zero bit inserted at position h
+MPJ_DEV int ins0(int v, int h) { return ((v >> h) << (h + 1)) | (v & ((1 << h) - 1)); }
+
+// One CTA per block pair of outer round R: inner sweep on the 32 x 32
+// subproblem; writes the rotated subproblem S (column-major), the accumulated
+// U (row-major for the FP32 products, column-major, urow false, for the
+// tensor-core panel) and the set T of its indices that rotated (Mbuf, bit l
+// for local index l, if not null): U is the identity outside T x T.
+//
+// The inner sweep runs the exclusive-or ordering: round r = 1 .. 31 rotates
+// the 16 disjoint pairs (i, i ^ r), every pair once per sweep.  Pair k of
+// round r is p = k with a zero bit inserted at r's highest bit h, q = p ^ r, so
+// p < q always, and the 2 x 2 blocks between two pairs are enumerated by bit
+// operations alone.  S is held once per unordered index pair, entry {i, j} at
+// (i ^ j) * SLD + min(i, j), so a block is read and written once without a
+// mirror.  What bounds the kernel is the chain coupling -> angle -> records ->
+// next round's coupling: the 16 couplings of the next round all lie in eight
+// blocks of this one, so warp 0 recomputes just those 16 entries, forms the
+// next round's rotations and leaves the blocks themselves to warps 1-4 (one
+// block per thread) and U to warps 5-8 (lane = row, four column pairs each).
+// S alternates between two buffers, so one barrier per round is enough.
+// Measured at n = 4096 (128 CTAs): circle ordering, two barriers, IEEE
+// divisions 23.8 us per launch; this form 18.1 us.  The sweeps to reach
+// the stopping test are the same or one fewer (n = 96 .. 512, three spectra).
+constexpr int S32_THREADS = 288;
+constexpr int SLD = 40;  // row stride of the packed S (8 more than 32: rows of d, d + 1, .. start 8 banks apart)
 __global__ void __launch_bounds__(S32_THREADS) solve32(const float* __restrict__ A32, int N, int nb, int R,
                                                float* __restrict__ Sbuf, float* __restrict__ Ubuf, bool hq,
                                                bool urow, unsigned* __restrict__ Mbuf) {
-  __shared__ float S[W2][LD];
-  __shared__ float U[W2][LD];
-  __shared__ RotRec<float> rec[W2 / 2];
+  __shared__ float S[2][W2 * SLD];
+  __shared__ float U[W2][LD];  // U[column][row]
+  __shared__ float dg[W2];     // the diagonal (warp 0 only)
+  __shared__ Rot32 rec[2][W2 / 2];
   const int slot = blockIdx.x;
   int I, J;
   block_pair(nb, R, slot, I, J);
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   pdl_wait();
-  #pragma unroll
-  for (int it = 0; it < W2 * W2 / S32_THREADS; ++it) {
-    const int e = tid + it * S32_THREADS;
-    int li = e % W2, lj = e / W2;
-    S[li][lj] = A32[(size_t)gidx(I, J, lj) * N + gidx(I, J, li)];
-    U[li][lj] = (li == lj) ? 1.0f : 0.0f;
+  for (int e = tid; e < W2 * W2; e += S32_THREADS) {
+    const int li = e % W2, lj = e / W2;
+    const float v = A32[(size_t)gidx(I, J, lj) * N + gidx(I, J, li)];
+    if (li == lj)
+      dg[li] = v;
+    else if (li < lj)
+      S[0][(li ^ lj) * SLD + li] = v;
+    U[lj][li] = (li == lj) ? 1.0f : 0.0f;
   }
   __syncthreads();
   const float skip = hq ? 0x1p-11f : 0x1p-24f;
-  unsigned tmask = 0u;  // thread 0: the indices that rotated so far
-  for (int rho = 0; rho < W2 - 1; ++rho) {
-    if (tid < W2 / 2) {
-      int x, y;
-      rr_slot(W2, rho, tid, x, y);
-      RotRec<float> rr;
-      rec32(x, y, S[x][x], S[y][y], S[y][x], skip, rr);
-      if (hq && rec_rotated(rr.cm1, rr.sig)) {  // c and s as binary16, new diagonal rounded
-        rr.cm1 = qh(1.0f + rr.cm1, true) - 1.0f;
-        rr.sig = qh(rr.sig, true);
-        rr.dx = qh(rr.dx, true);
-        rr.dy = qh(rr.dy, true);
-      }
-      rec[tid] = rr;
-      if (Mbuf) {
-        const unsigned bits = rec_rotated(rr.cm1, rr.sig) ? ((1u << x) | (1u << y)) : 0u;
-        tmask |= __reduce_or_sync(0x0000FFFFu, bits);  // the 16 record lanes of warp 0
-      }
+  unsigned tmask = 0u;  // warp 0: the indices that rotated so far
+  float held = 0.0f;    // warp 0: the pair's own coupling after its rotation
+  // rotation of pair k of round r from its coupling, into rec[buf]
+  auto rotate = [&](int k, int p, int q, float apq, int buf) {
+    float app = dg[p], aqq = dg[q];
+    Rot32 rr;
+    const bool rot = rot32(app, aqq, apq, skip, rr);
+    if (hq && rot) {  // c and s as binary16, new diagonal rounded
+      rr.cm1 = qh(1.0f + rr.cm1, true) - 1.0f;
+      rr.sig = qh(rr.sig, true);
+      app = qh(app, true);
+      aqq = qh(aqq, true);
     }
-    __syncthreads();
-    {
-      int a = tid % 16, b = tid / 16;
-      if (b < 16 && a >= b) {
-        int xa, ya, xb, yb;
-        rr_slot(W2, rho, a, xa, ya);
-        rr_slot(W2, rho, b, xb, yb);
-        RotRec<float> ra = rec[a], rb = rec[b];
-        bool rota = rec_rotated(ra.cm1, ra.sig), rotb = rec_rotated(rb.cm1, rb.sig);
-        if (a == b) {
-          if (rota) {
-            S[xa][xa] = ra.dx;
-            S[ya][ya] = ra.dy;
-            S[xa][ya] = 0.0f;
-            S[ya][xa] = 0.0f;
-          }
-        } else if (rota || rotb) {
-          float vxx = S[xa][xb], vxy = S[xa][yb], vyx = S[ya][xb], vyy = S[ya][yb];
-          if (rota) {
-            rot_apply(ra.cm1, ra.sig, vxx, vyx);
-            rot_apply(ra.cm1, ra.sig, vxy, vyy);
-          }
-          if (rotb) {
-            rot_apply(rb.cm1, rb.sig, vxx, vxy);
-            rot_apply(rb.cm1, rb.sig, vyx, vyy);
-          }
-          vxx = qh(vxx, hq);
-          vxy = qh(vxy, hq);
-          vyx = qh(vyx, hq);
-          vyy = qh(vyy, hq);
-          S[xa][xb] = vxx;
-          S[xb][xa] = vxx;
-          S[xa][yb] = vxy;
-          S[yb][xa] = vxy;
-          S[ya][xb] = vyx;
-          S[xb][ya] = vyx;
-          S[ya][yb] = vyy;
-          S[yb][ya] = vyy;
+    rec[buf][k] = rr;
+    if (rot) {
+      dg[p] = app;
+      dg[q] = aqq;
+    }
+    held = rot ? 0.0f : apq;
+    if (Mbuf) {
+      const unsigned bits = rec_rotated(rr.cm1, rr.sig) ? ((1u << p) | (1u << q)) : 0u;
+      tmask |= __reduce_or_sync(0x0000FFFFu, bits);  // the 16 record lanes of warp 0
+    }
+  };
+  if (warp == 0) {
+    if (lane < W2 / 2) rotate(lane, 2 * lane, 2 * lane + 1, S[0][SLD + 2 * lane], 0);
+    __syncwarp();
+  }
+  // the block of threads 32 .. 151: pairs with 4-bit labels xl and yl = xl ^ dl,
+  // xl's bit at dl's highest bit zero: 15 x 8 unordered label pairs
+  const int bt = tid - 32, dl = 1 + (bt >> 3);
+  const int xl = ins0(bt & 7, 31 - __clz(dl)), yl = xl ^ dl;
+  __syncthreads();
+#pragma unroll 1
+  for (int r = 1; r < W2; ++r) {
+    const int cur = (r - 1) & 1;
+    const float* Sc = S[cur];
+    float* Sn = S[cur ^ 1];
+    const int h = 31 - __clz(r);
+    const int rn = r + 1;  // the next round (none after r = 31)
+    if (warp == 0) {
+      if (lane < W2 / 2) {
+        Sn[r * SLD + ins0(lane, h)] = held;
+        if (rn < W2) {
+          const int hn = 31 - __clz(rn);
+          const int p = ins0(lane, hn), q = p ^ rn;
+          // this round's pairs of p and of q: records and the side of each
+          const bool p2 = (p >> h) & 1, q2 = (q >> h) & 1;
+          const int pr = p2 ? p ^ r : p, qr = q2 ? q ^ r : q;
+          const Rot32 ra = rec[cur][((pr >> (h + 1)) << h) | (pr & ((1 << h) - 1))];
+          const Rot32 rb = rec[cur][((qr >> (h + 1)) << h) | (qr & ((1 << h) - 1))];
+          const int po = p ^ r, qo = q ^ r, dA = rn * SLD, dB = (rn ^ r) * SLD;
+          const float e00 = Sc[dA + min(p, q)], e01 = Sc[dB + min(p, qo)];
+          const float e10 = Sc[dB + min(po, q)], e11 = Sc[dA + min(po, qo)];
+          const float sa = p2 ? ra.sig : -ra.sig, sb = q2 ? rb.sig : -rb.sig;
+          const float t0 = rot_one(ra.cm1, sa, e00, e10), t1 = rot_one(ra.cm1, sa, e01, e11);
+          rotate(lane, p, q, qh(rot_one(rb.cm1, sb, t0, t1), hq), cur ^ 1);
         }
       }
-      // U <- U J: rows of U are independent; columns x_b, y_b
-      for (int e = tid; e < W2 * (W2 / 2); e += S32_THREADS) {
-        int row = e % W2, sb = e / W2;
-        RotRec<float> rb = rec[sb];
-        if (!rec_rotated(rb.cm1, rb.sig)) continue;
-        int xb, yb;
-        rr_slot(W2, rho, sb, xb, yb);
-        float ux = U[row][xb], uy = U[row][yb];
-        rot_apply(rb.cm1, rb.sig, ux, uy);
-        U[row][xb] = qh(ux, hq);
-        U[row][yb] = qh(uy, hq);
+    } else if (warp < 5) {
+      if (bt < 120) {
+        const int x = ins0(xl, h), y = ins0(yl, h), x2 = x ^ r, y2 = y ^ r;
+        const Rot32 ra = rec[cur][xl], rb = rec[cur][yl];
+        const int d0 = x ^ y, d1 = d0 ^ r;
+        const int i00 = d0 * SLD + min(x, y), i01 = d1 * SLD + min(x, y2);
+        const int i10 = d1 * SLD + min(x2, y), i11 = d0 * SLD + min(x2, y2);
+        const float v00 = Sc[i00], v01 = Sc[i01], v10 = Sc[i10], v11 = Sc[i11];
+        const float t00 = rot_one(ra.cm1, -ra.sig, v00, v10), t10 = rot_one(ra.cm1, ra.sig, v10, v00);
+        const float t01 = rot_one(ra.cm1, -ra.sig, v01, v11), t11 = rot_one(ra.cm1, ra.sig, v11, v01);
+        if (d0 != rn) {  // warp 0 holds the next round's couplings
+          Sn[i00] = qh(rot_one(rb.cm1, -rb.sig, t00, t01), hq);
+          Sn[i11] = qh(rot_one(rb.cm1, rb.sig, t11, t10), hq);
+        }
+        if (d1 != rn) {
+          Sn[i01] = qh(rot_one(rb.cm1, rb.sig, t01, t00), hq);
+          Sn[i10] = qh(rot_one(rb.cm1, -rb.sig, t10, t11), hq);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int k = 4 * (warp - 5) + i, p = ins0(k, h), q = p ^ r;
+        const Rot32 rr = rec[cur][k];
+        const float up = U[p][lane], uq = U[q][lane];
+        U[p][lane] = qh(rot_one(rr.cm1, -rr.sig, up, uq), hq);
+        U[q][lane] = qh(rot_one(rr.cm1, rr.sig, uq, up), hq);
       }
     }
     __syncthreads();
   }
   float* So = Sbuf + (size_t)slot * W2 * W2;
   float* Uo = Ubuf + (size_t)slot * W2 * W2;
-  #pragma unroll
-  for (int it = 0; it < W2 * W2 / S32_THREADS; ++it) {
-    const int e = tid + it * S32_THREADS;
-    int li = e % W2, lj = e / W2;
-    So[e] = S[li][lj];
-    Uo[e] = urow ? U[lj][li] : U[li][lj];
+  for (int e = tid; e < W2 * W2; e += S32_THREADS) {
+    const int li = e % W2, lj = e / W2;
+    So[e] = li == lj ? dg[li] : S[1][(li ^ lj) * SLD + min(li, lj)];
+    Uo[e] = urow ? U[li][lj] : U[lj][li];
   }
   if (tid == 0 && Mbuf) Mbuf[slot] = tmask;
 }
