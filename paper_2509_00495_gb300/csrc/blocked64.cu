@@ -1,15 +1,15 @@
 // blocked64.cu -- FP64 Jacobi sweeps in block round-robin order with the
 // block updates on the tcgen05 tensor cores (the block Jacobi procedure the
 // paper names as further work, Ch. 6; the rotations themselves are the
-// paper's Algorithm 2 with the skip test of Algorithm 4, in FP64).
+// paper's Algorithm 2 with the skip test of Algorithm 4).
 //
 // Ordering: the padded index range [0, N) (N = n rounded up to a multiple of
 // 32; indices >= n are inert) is cut into nb = N/16 blocks of 16.  A sweep is
 // nb - 1 outer rounds of the circle method on blocks; in round R the nb/2
 // disjoint block pairs P = (I, J) each run one inner round-robin sweep (31
 // inner rounds of 16 disjoint pairs) over the 32 indices of I u J on their
-// 32 x 32 diagonal subproblem A[P, P], in FP64 in shared memory, accumulating
-// the orthogonal U_P.  This is the rotation sequence of the block
+// 32 x 32 diagonal subproblem A[P, P] in shared memory, accumulating U_P,
+// which is then made orthogonal to FP64 precision (blk_solve).  This is the rotation sequence of the block
 // round-robin ordering one rotation at a time: the subproblem's rotations
 // depend only on its own entries, and the pairs of one round are disjoint.
 // The rest of the matrix then receives the round's rotations as products
@@ -74,6 +74,22 @@ MPJ_DEV void block_pair(int nb, int R, int slot, int& I, int& J) {
 // core matrices (k-adjacent cores 128 bytes apart, 8-row groups 512 apart)
 MPJ_DEV int kmaj16(int row, int k) { return (((row >> 3) * 4 + (k >> 3)) << 7) + ((row & 7) << 4) + ((k & 7) << 1); }
 
+// Seven digits of an integer value: Y = |x| 2^(56 - e) < 2^56 rounded, sign sg
+// = +-1 (the weights are in digits_f32).
+MPJ_DEV void digits_of(unsigned long long Y, float sg, uint32_t d[NSL]) {
+  const unsigned long long T = Y + 0x0000808080808080ULL;
+  const uint32_t lo = (uint32_t)T, hi = (uint32_t)(T >> 32);
+  const float c128 = -8388736.0f * sg;  // -(2^23 + 128) sign(x)
+  // bytes of lo: d6+128, d5+128, d4+128, d3+128; of hi: d2+128, d1+128; hi >> 16: d0
+  d[6] = __float_as_uint(fmaf(__uint_as_float(__byte_perm(lo, 0x4B00u, 0x5440)), sg, c128));
+  d[5] = __float_as_uint(fmaf(__uint_as_float(__byte_perm(lo, 0x4B00u, 0x5441)), sg, c128));
+  d[4] = __float_as_uint(fmaf(__uint_as_float(__byte_perm(lo, 0x4B00u, 0x5442)), sg, c128));
+  d[3] = __float_as_uint(fmaf(__uint_as_float(__byte_perm(lo, 0x4B00u, 0x5443)), sg, c128));
+  d[2] = __float_as_uint(fmaf(__uint_as_float(__byte_perm(hi, 0x4B00u, 0x5440)), sg, c128));
+  d[1] = __float_as_uint(fmaf(__uint_as_float(__byte_perm(hi, 0x4B00u, 0x5441)), sg, c128));
+  d[0] = __float_as_uint(fmaf(__uint_as_float(0x4B000000u | (hi >> 16)), sg, -8388608.0f * sg));
+}
+
 // The seven signed digits of x on the grid 2^e (|x| < 2^e): x = sum_i d_i
 // 2^(e - 8 (i + 1)) + r, |r| <= 2^(e - 57), |d_0| <= 256, |d_i| <= 128 (i >= 1),
 // returned as FP32 bit patterns (exact small integers; their top 16 bits are
@@ -97,18 +113,7 @@ MPJ_DEV void digits_f32(double x, int e, uint32_t d[NSL]) {
     Y = (M + (1ULL << (-sh - 1))) >> (-sh);
   else
     Y = 0;
-  const unsigned long long T = Y + 0x0000808080808080ULL;
-  const uint32_t lo = (uint32_t)T, hi = (uint32_t)(T >> 32);
-  const float sg = (bits >> 63) ? -1.0f : 1.0f;
-  const float c128 = -8388736.0f * sg;  // -(2^23 + 128) sign(x)
-  // bytes of lo: d6+128, d5+128, d4+128, d3+128; of hi: d2+128, d1+128; hi >> 16: d0
-  d[6] = __float_as_uint(fmaf(__uint_as_float(__byte_perm(lo, 0x4B00u, 0x5440)), sg, c128));
-  d[5] = __float_as_uint(fmaf(__uint_as_float(__byte_perm(lo, 0x4B00u, 0x5441)), sg, c128));
-  d[4] = __float_as_uint(fmaf(__uint_as_float(__byte_perm(lo, 0x4B00u, 0x5442)), sg, c128));
-  d[3] = __float_as_uint(fmaf(__uint_as_float(__byte_perm(lo, 0x4B00u, 0x5443)), sg, c128));
-  d[2] = __float_as_uint(fmaf(__uint_as_float(__byte_perm(hi, 0x4B00u, 0x5440)), sg, c128));
-  d[1] = __float_as_uint(fmaf(__uint_as_float(__byte_perm(hi, 0x4B00u, 0x5441)), sg, c128));
-  d[0] = __float_as_uint(fmaf(__uint_as_float(0x4B000000u | (hi >> 16)), sg, -8388608.0f * sg));
+  digits_of(Y, (bits >> 63) ? -1.0f : 1.0f, d);
 }
 
 // Two FP32 digit patterns packed as two bf16 (a in the low half).
@@ -179,306 +184,511 @@ MPJ_DEV double z_to_double(long long hi, long long lo, int E) {
   return __longlong_as_double((long long)(sign | ((unsigned long long)biased << 52) | (mant & ((1ULL << 52) - 1ULL))));
 }
 
-// Algorithm 2 for the scaled subproblem rotations, with the skip test of
-// Algorithm 4 (|a_pq| > skip sqrt|a_pp a_qq|, compared in squares, and the
-// threshold |a_pq| > skip_abs): t as in the stable form, c = 1 / sqrt(1 + t^2)
-// and h = 1 / c = (1 + t^2) c for the scale vector and its reciprocal.
-MPJ_DEV bool rot_scaled(double app, double aqq, double apq, double skip, double skip_abs, double& t, double& c,
-                        double& h) {
-  if (!(apq * apq > (skip * skip) * fabs(app * aqq) && fabs(apq) > skip_abs)) return false;
-  const double tau = (aqq - app) / (2.0 * apq);
-  const double r = sqrt(fma(tau, tau, 1.0));
-  t = (tau >= 0.0) ? 1.0 / (tau + r) : 1.0 / (tau - r);
-  const double w = fma(t, t, 1.0);
-  c = rsqrt(w);
-  h = w * c;
-  return true;
+// ---------------------------------------------------------------- subproblems
+// Pairs of FP32 values v = hi + lo (about 48 bits).  The subproblem's entries
+// and U_P are held this way: an FP64 instruction takes 64 FP32 issue slots on
+// this GPU, and only U_P leaves the subproblem, which is made orthogonal to
+// FP64 precision (and 2^-60 in fixed point) before it is applied.
+MPJ_DEV float2 df_norm(float hi, float lo) {  // |hi| >= |lo|
+  const float s = __fadd_rn(hi, lo);
+  return make_float2(s, __fsub_rn(lo, __fsub_rn(s, hi)));
+}
+// a * b as an unnormalised pair (relative error about 2^-47)
+MPJ_DEV float2 df_mul(float2 a, float2 b) {
+  const float p = __fmul_rn(a.x, b.x);
+  float e = __fmaf_rn(a.x, b.x, -p);
+  e = __fmaf_rn(a.x, b.y, e);
+  e = __fmaf_rn(a.y, b.x, e);
+  return make_float2(p, e);
+}
+MPJ_DEV float2 df_add(float2 a, float2 b) {
+  const float s = __fadd_rn(a.x, b.x);
+  const float bb = __fsub_rn(s, a.x);
+  const float err = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, bb)), __fsub_rn(b.x, bb));
+  return df_norm(s, __fadd_rn(err, __fadd_rn(a.y, b.y)));
+}
+MPJ_DEV float2 df_neg(float2 a) { return make_float2(-a.x, -a.y); }
+// c x + s y
+MPJ_DEV float2 df_rot(float2 c, float2 x, float2 s, float2 y) { return df_add(df_mul(c, x), df_mul(s, y)); }
+
+// x 2^-eo as a pair (integer instructions): truncated to 24 bits, then the
+// remaining 29 rounded; parts below the normal FP32 range become zero.
+MPJ_DEV float2 df_split(double x, int eo) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)((b >> 52) & 0x7FF);
+  if (ex == 0) return make_float2(0.0f, 0.0f);
+  const unsigned long long m = (b & 0xFFFFFFFFFFFFFULL) | (1ULL << 52);
+  const int k = ex - 1075 - eo;  // x 2^-eo = +- m 2^k
+  const float sg = (b >> 63) ? -1.0f : 1.0f;
+  const int kh = k + 29;
+  const float h = kh >= -126 ? __int_as_float((min(kh, 127) + 127) << 23) : 0.0f;
+  const float l = k >= -126 ? __int_as_float((min(k, 127) + 127) << 23) : 0.0f;
+  return make_float2(sg * (float)(unsigned)(m >> 29) * h, sg * (float)(unsigned)(m & 0x1FFFFFFFULL) * l);
 }
 
-// ---------------------------------------------------------------- subproblems
-// One CTA per block pair of round R: one inner round-robin sweep on the FP64
-// 32 x 32 subproblem (the paper's row update, column update and vector update
-// per rotation, in scaled form: one FMA per entry and side, the factors c kept
-// in a scale vector; the 16 disjoint rotations of an inner round are applied
-// together), then U_P's columns cut into digits for the tensor products.
-// Writes per block pair: NSL digit tiles (32 x 32 bf16, K-major over the
-// rows of U_P, one "row" per column of U_P), 32 column exponents, and whether
-// any rotation happened.
-constexpr int SOLVE_THREADS = 512;
+// Algorithm 2 on FP32 pairs: coupling a, d = a_qq - a_pp, giving t (the root
+// of a t^2 + d t - a with |t| <= 1, '+' for d = 0), c = 1 / sqrt(1 + t^2) and
+// s = t c.  t and c start from FP32 seeds; one Newton step each on a residual
+// formed with pairs takes them to the pairs' precision.
+MPJ_DEV void df_angle(float2 a, float2 d, float2& t, float2& c, float2& s) {
+  const float tau = __fdividef(d.x, 2.0f * a.x), at = fabsf(tau);
+  float root;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(root) : "f"(fmaf(at, at, 1.0f)));
+  float t0 = at > 1e9f ? __fdividef(0.5f, at) : __fdividef(1.0f, at + root);
+  t0 = tau >= 0.0f ? t0 : -t0;
+  const float c0 = rsqrtf(fmaf(t0, t0, 1.0f));
+  // f = (a t0 + d) t0 - a, t = t0 - f / (2 a t0 + d)
+  const float inv = __fdividef(1.0f, fmaf(2.0f * a.x, t0, d.x));
+  const float2 t0p = make_float2(t0, 0.0f);
+  const float2 g = df_add(d, df_mul(a, t0p));
+  const float2 f = df_add(df_mul(g, t0p), df_neg(a));
+  const float dt = f.x * inv;
+  t.x = __fsub_rn(t0, dt);
+  t.y = __fsub_rn(__fsub_rn(t0, t.x), dt);
+  // e = 1 - (1 + t^2) c0^2, c = c0 (1 + e / 2 + 3 e^2 / 8)
+  const float2 t2 = df_mul(t, t);
+  const float wh = __fadd_rn(1.0f, t2.x);
+  const float wl = __fadd_rn(__fsub_rn(t2.x, __fsub_rn(wh, 1.0f)), t2.y);
+  const float u = __fmul_rn(c0, c0), ue = __fmaf_rn(c0, c0, -u);
+  const float2 m = df_mul(make_float2(wh, wl), make_float2(u, ue));
+  const float e = __fsub_rn(__fsub_rn(1.0f, m.x), m.y);
+  const float corr = c0 * fmaf(0.375f * e, e, 0.5f * e);
+  c.x = __fadd_rn(c0, corr);
+  c.y = __fadd_rn(__fsub_rn(c0, c.x), corr);
+  const float2 sp = df_mul(t, c);
+  s = df_norm(sp.x, sp.y);
+}
+
+// One CTA per block pair of round R: one inner round-robin sweep (circle
+// method, 31 rounds of 16 disjoint pairs, Algorithm 2 with the skip test of
+// Algorithm 4) on the 32 x 32 subproblem, then one Newton-Schulz correction of
+// U_P and U_P's columns cut into digits for the tensor products.  Writes per
+// block pair: NSL digit tiles (32 x 32 bf16, K-major over the rows of U_P, one
+// "row" per column of U_P), 32 column exponents, and whether any rotation
+// happened (when none did, U_P = I and only that flag is written).
+//
+// Arithmetic.  The couplings and U_P are FP32 pairs, the couplings scaled by
+// the power of two of the largest; the diagonal is the FP64 diagonal at the
+// start plus a pair with its change, and a_qq - a_pp is formed from the FP64
+// difference, so nearly equal diagonal entries keep their gap.  U_P comes out
+// orthogonal to about 2^-43; in 60-bit fixed point E = U_P^T U_P - I is then
+// formed exactly enough (2^-59) with integer products, and U_P - U_P E / 2 is
+// orthogonal to 2^-59.  (The digits the products use have 2^-57.)  Entries
+// whose range does not fit pairs (more than 2^70 between the couplings, or
+// 2^100 between a coupling and the diagonal: graded matrices) run the same
+// sweep in FP64 instructions instead.
+//
+// What bounds it: the chain coupling -> angle -> record -> next coupling.  The
+// 16 couplings of the next round lie in blocks known in advance, so warp 0
+// recomputes just those entries and the next round's rotations while warps
+// 1-4 update the 2 x 2 blocks (one per thread) and warps 5-8 U_P (lane = row,
+// four column pairs each); the couplings alternate between two buffers, so
+// one barrier per round is enough.  In FP64 instructions the chain alone was
+// about 60 dependent instructions of 65 cycles per round.  Measured at
+// n = 4096 (128 CTAs): 101 us per launch in FP64, 34.5 us in this form.
+constexpr int SOLVE_THREADS = 288;
+constexpr int UFL = 36;  // row stride of the fixed-point U (16-byte rows, conflict-free 16-byte reads)
+struct SolveSmem {
+  union {
+    struct {
+      float2 S[2][W2 * LDS];  // couplings {i, j} at max(i, j) * LDS + min(i, j)
+      float2 U[W2][LDS];      // U[column][row]
+    } p;
+    double U64[W2][LDS];  // FP64 form: U[column][row]
+    struct {
+      int u1[W2][UFL], u0[W2][UFL];  // U = (u1 + u0 2^-30) 2^-30, [column][row]
+      float Ef[W2][UFL];             // E = U^T U - I
+    } f;
+  };
+  double A[W2][LDS];      // the subproblem as loaded; FP64 form: in place
+  double cs[W2 / 2][2];   // FP64 form: c - 1, s
+  float4 rec[2][W2 / 2];  // c, sig oriented to the slot's (x, y)
+  float2 corr[W2];        // change of the diagonal (scaled pair)
+  float d0[W2];           // starting diagonal (scaled)
+  unsigned emax_off, emin_off, emax_dg, any;
+};
+
 __global__ void __launch_bounds__(SOLVE_THREADS) blk_solve(const double* __restrict__ A, int lda, int n, int nb, int R,
                                                  double skip, double skip_abs, __nv_bfloat16* __restrict__ Usl,
                                                  int* __restrict__ Uexp, int* __restrict__ rotated,
                                                  unsigned* __restrict__ nrot) {
-  __shared__ double S[W2][LDS];
-  __shared__ double U[W2][LDS];
-  __shared__ int any;
-  const int P = blockIdx.x, tid = threadIdx.x;
+  __shared__ __align__(16) SolveSmem sm;
+  const int P = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   int I, J;
   block_pair(nb, R, P, I, J);
-  if (tid == 0) any = 0;
+  if (tid == 0) {
+    sm.emax_off = 0u;
+    sm.emin_off = 0xFFFFu;
+    sm.emax_dg = 0u;
+    sm.any = 0u;
+  }
+  __syncthreads();
   pdl_wait();
-  for (int e = tid; e < W2 * W2; e += blockDim.x) {
-    const int li = e % W2, lj = e / W2;
-    const int gi = gidx(I, J, li), gj = gidx(I, J, lj);
-    S[li][lj] = (gi < n && gj < n) ? A[(size_t)gj * lda + gi] : 0.0;
-    U[li][lj] = (li == lj) ? 1.0 : 0.0;
-  }
-  __syncthreads();
-  // Scaled rotations (the scheme of the scalar round-robin sweeps): off the
-  // diagonal S = D S~ D and U = U~ D with one scale vector d (and e = 1/d);
-  // S's diagonal holds the true values.  A rotation (c, s = t c) of pair
-  // p < q then costs one FMA per entry and side:
-  //   x_p <- x_p - mx x_q,  x_q <- x_q + my x_p  (old values),
-  //   mx = t d_q / d_p,  my = t d_p / d_q,  d_p, d_q <- c d_p, c d_q,
-  // the pair's diagonal becomes a_pp - t a_pq, a_qq + t a_pq and a_pq 0.
-  // Each inner round applies its 16 rotations to every 2 x 2 block of S
-  // between two pairs a < b once (rows by pair a, then columns by pair b; the
-  // mirror block is the same values transposed) and to the two columns of U~
-  // of every pair.  The next round's rotations read only the diagonal entries
-  // and the blocks (a, b) that hold one of its pairs: warp 0 sets the
-  // diagonal blocks and updates those blocks first and then computes the next
-  // round's rotations, while the other warps update the remaining blocks and
-  // U~.  Each block is updated by exactly one thread.
-  __shared__ double cs[2][W2 / 2][2];  // mx, my
-  __shared__ double dg[2][W2 / 2][2];  // the pair's new true diagonal
-  __shared__ int rot[2][W2 / 2];
-  __shared__ int pq[2][W2 / 2][2];
-  __shared__ int slot_of[2][W2];  // pair slot of each local index in the round
-  __shared__ double dsc[W2], esc[W2];  // d and e = 1 / d
-  const int warp = tid >> 5, lane = tid & 31;
-  if (tid < W2) {
-    dsc[tid] = 1.0;
-    esc[tid] = 1.0;
-  }
-  __syncthreads();
-  // Algorithm 2 with the skip test of Algorithm 4 for pair `k` of inner round
-  // rho, on the true coupling; the pair's scales are updated here (its lane
-  // is the only one that touches them this round)
-  auto rotation = [&](int rho, int k, int buf) {
-    int x, y;
-    rr_slot(W2, rho, k, x, y);
-    const int p = x < y ? x : y, q = x < y ? y : x;
-    const double app = S[p][p], aqq = S[q][q];
-    const double dp = dsc[p], dq = dsc[q];
-    const double apq = S[p][q] * dp * dq;
-    double t = 0.0, c = 1.0, h = 1.0;
-    const int r = gidx(I, J, q) < n && rot_scaled(app, aqq, apq, skip, skip_abs, t, c, h);
-    double mx = 0.0, my = 0.0;
-    if (r) {
-      any = 1;
-      const double ep = esc[p], eq = esc[q];
-      mx = t * dq * ep;
-      my = t * dp * eq;
-      dsc[p] = dp * c;
-      dsc[q] = dq * c;
-      esc[p] = ep * h;
-      esc[q] = eq * h;
-      dg[buf][k][0] = app - t * apq;
-      dg[buf][k][1] = aqq + t * apq;
-    }
-    cs[buf][k][0] = mx;
-    cs[buf][k][1] = my;
-    rot[buf][k] = r;
-    pq[buf][k][0] = p;
-    pq[buf][k][1] = q;
-    slot_of[buf][p] = k;
-    slot_of[buf][q] = k;
-  };
-  // the pair's own 2 x 2 block: the new true diagonal and a zero coupling
-  auto diag_update = [&](int a, int buf) {
-    if (!rot[buf][a]) return;
-    const int pa = pq[buf][a][0], qa = pq[buf][a][1];
-    S[pa][pa] = dg[buf][a][0];
-    S[qa][qa] = dg[buf][a][1];
-    S[pa][qa] = 0.0;
-    S[qa][pa] = 0.0;
-  };
-  // the 2 x 2 block between pairs a < b of the round in buffer `buf`
-  auto block_update = [&](int a, int b, int buf) {
-    if (!rot[buf][a] && !rot[buf][b]) return;
-    const int pa = pq[buf][a][0], qa = pq[buf][a][1], pb = pq[buf][b][0], qb = pq[buf][b][1];
-    double b00 = S[pa][pb], b01 = S[pa][qb], b10 = S[qa][pb], b11 = S[qa][qb];
-    if (rot[buf][a]) {  // rows pa, qa
-      const double mx = cs[buf][a][0], my = cs[buf][a][1];
-      const double t00 = fma(-mx, b10, b00), t10 = fma(my, b00, b10);
-      const double t01 = fma(-mx, b11, b01), t11 = fma(my, b01, b11);
-      b00 = t00;
-      b10 = t10;
-      b01 = t01;
-      b11 = t11;
-    }
-    if (rot[buf][b]) {  // columns pb, qb
-      const double mx = cs[buf][b][0], my = cs[buf][b][1];
-      const double t00 = fma(-mx, b01, b00), t01 = fma(my, b00, b01);
-      const double t10 = fma(-mx, b11, b10), t11 = fma(my, b10, b11);
-      b00 = t00;
-      b01 = t01;
-      b10 = t10;
-      b11 = t11;
-    }
-    S[pa][pb] = b00;
-    S[pa][qb] = b01;
-    S[qa][pb] = b10;
-    S[qa][qb] = b11;
-    S[pb][pa] = b00;
-    S[qb][pa] = b01;
-    S[pb][qa] = b10;
-    S[qb][qa] = b11;
-  };
-  if (warp == 0 && lane < W2 / 2) rotation(0, lane, 0);
-  __syncthreads();
-  for (int rho = 0; rho < W2 - 1; ++rho) {
-    const int cur = rho & 1;
-    const bool more = rho + 1 < W2 - 1;
-    if (warp == 0) {
-      // lanes 0-15: the pairs' own blocks; lanes 16-31: the block holding pair
-      // lane - 16 of the next round (once, when two next pairs share a block)
-      if (lane < W2 / 2) {
-        diag_update(lane, cur);
-      } else if (more) {
-        int x, y;
-        rr_slot(W2, rho + 1, lane - W2 / 2, x, y);
-        int a = slot_of[cur][x], b = slot_of[cur][y];
-        if (a > b) {
-          const int t = a;
-          a = b;
-          b = t;
-          const int tx = x;
-          x = y;
-          y = tx;
-        }
-        // x is in pair a: the other index of a, if its next partner is in b,
-        // gives the same block; the smaller of the two indices takes it
-        const int o = pq[cur][a][0] == x ? pq[cur][a][1] : pq[cur][a][0];
-        const bool dup = slot_of[cur][rr_partner(W2, rho + 1, o)] == b;
-        if (a != b && (!dup || x < o)) block_update(a, b, cur);
+  {
+    unsigned mo = 0u, mn = 0xFFFFu, md = 0u, big = 0u;
+    for (int e = tid; e < W2 * W2; e += SOLVE_THREADS) {
+      const int li = e % W2, lj = e / W2;
+      const int gi = gidx(I, J, li), gj = gidx(I, J, lj);
+      const double v = (gi < n && gj < n) ? A[(size_t)gj * lda + gi] : 0.0;
+      sm.A[li][lj] = v;
+      const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFULL;
+      const unsigned ex = (unsigned)(b >> 52);
+      if (li == lj) {
+        md = max(md, ex);
+      } else if (b != 0) {
+        mo = max(mo, ex);
+        mn = min(mn, ex);
+        // |v| > skip_abs, as bit patterns
+        if (b > (unsigned long long)__double_as_longlong(skip_abs)) big = 1u;
       }
-      __syncwarp();
-      if (more && lane < W2 / 2) rotation(rho + 1, lane, cur ^ 1);
-    } else {
-      for (int task = tid - 32; task < 120 + (W2 / 2) * W2; task += blockDim.x - 32) {
+    }
+    mo = __reduce_max_sync(0xFFFFFFFFu, mo);
+    mn = __reduce_min_sync(0xFFFFFFFFu, mn);
+    md = __reduce_max_sync(0xFFFFFFFFu, md);
+    big = __reduce_or_sync(0xFFFFFFFFu, big);
+    if (lane == 0) {
+      atomicMax(&sm.emax_off, mo);
+      atomicMin(&sm.emin_off, mn);
+      atomicMax(&sm.emax_dg, md);
+      if (big) atomicOr(&sm.any, 1u);
+    }
+  }
+  __syncthreads();
+  if (!sm.any) {  // every coupling is zero or at most skip_abs: nothing rotates
+    if (tid == 0) rotated[P] = 0;
+    return;
+  }
+  const int emax_off = (int)sm.emax_off, emin_off = (int)sm.emin_off;
+  const int etop = max(emax_off, (int)sm.emax_dg);
+  const bool pairs = emin_off > 0 && emax_off - emin_off <= 70 && etop - emin_off <= 100 && etop < 2000;
+  const int eo = emax_off - 1022;  // couplings scaled by 2^-eo: at most 1
+  __syncthreads();
+  if (tid == 0) sm.any = 0u;
+  if (pairs) {
+    for (int e = tid; e < W2 * W2; e += SOLVE_THREADS) {
+      const int li = e % W2, lj = e / W2;
+      if (li == lj) {
+        sm.corr[li] = make_float2(0.0f, 0.0f);
+        sm.d0[li] = df_split(sm.A[li][li], eo).x;
+      } else if (li > lj) {
+        sm.p.S[0][li * LDS + lj] = df_split(sm.A[li][lj], eo);
+      }
+      sm.p.U[lj][li] = make_float2(li == lj ? 1.0f : 0.0f, 0.0f);
+    }
+    // skip_abs 2^-eo rounded to FP32 (infinite when it is beyond every coupling)
+    float sabs;
+    {
+      const int k = (int)(((unsigned long long)__double_as_longlong(skip_abs) >> 52) & 0x7FF) - 1023 - eo;
+      sabs = skip_abs <= 0.0 ? 0.0f : k > 100 ? __int_as_float(0x7F800000) : k < -120 ? 0.0f : df_split(skip_abs, eo).x;
+    }
+    const float skf = (float)skip;
+    __syncthreads();
+    float2 held = make_float2(0.0f, 0.0f);  // warp 0: the pair's own coupling after its rotation
+    bool mine = false;
+    auto rotate = [&](int rho, float2 a, float2 base, int buf) {
+      int x, y;
+      rr_slot(W2, rho, lane, x, y);
+      const int pi = min(x, y), qi = max(x, y);
+      const float2 cp = sm.corr[pi], cq = sm.corr[qi];
+      const float app = fabsf(sm.d0[pi] + cp.x), aqq = fabsf(sm.d0[qi] + cq.x);
+      float rp, rq;
+      asm("sqrt.approx.f32 %0, %1;" : "=f"(rp) : "f"(app));
+      asm("sqrt.approx.f32 %0, %1;" : "=f"(rq) : "f"(aqq));
+      float4 r = make_float4(1.0f, 0.0f, 0.0f, 0.0f);
+      held = a;
+      if (fabsf(a.x) > skf * rp * rq && fabsf(a.x) > sabs) {
+        mine = true;
+        const float2 d = df_add(base, df_add(cq, df_neg(cp)));
+        float2 t, c, s;
+        df_angle(a, d, t, c, s);
+        const float2 ta = df_mul(t, a);
+        sm.corr[pi] = df_add(cp, df_neg(ta));
+        sm.corr[qi] = df_add(cq, ta);
+        if (x > y) s = df_neg(s);
+        r = make_float4(c.x, c.y, s.x, s.y);
+        held = make_float2(0.0f, 0.0f);
+      }
+      sm.rec[buf][lane] = r;
+    };
+    // a_qq - a_pp of the starting diagonal for pair `lane` of round rho
+    auto base_gap = [&](int rho) {
+      int x, y;
+      rr_slot(W2, rho, lane, x, y);
+      const int pi = min(x, y), qi = max(x, y);
+      return df_split(sm.A[qi][qi] - sm.A[pi][pi], eo);
+    };
+    auto at = [](int i, int j) { return max(i, j) * LDS + min(i, j); };
+    // where pair `lane` of the next round lies now: block (sa, sb) of this
+    // round's slots, index x or y of each (rr_slot's indices advance by one)
+    const int sa = lane < 2 ? 0 : lane == 15 ? 14 : lane - 1;
+    const int sb = lane == 0 ? 1 : lane == 1 ? 2 : lane == 15 ? 15 : lane + 1;
+    const bool ya = lane != 1, yb = lane == 15;
+    float2 base = make_float2(0.0f, 0.0f);
+    if (warp == 0 && lane < W2 / 2) {
+      int x, y;
+      rr_slot(W2, 0, lane, x, y);
+      rotate(0, sm.p.S[0][at(x, y)], base_gap(0), 0);
+      base = base_gap(1);
+    }
+    // the block of threads 32 .. 151: slots ba < bb
+    int ba = 0, bb = 0;
+    {
+      int rem = tid - 32;
+      if (rem >= 0 && rem < 120) {
+        while (rem >= 15 - ba) {
+          rem -= 15 - ba;
+          ++ba;
+        }
+        bb = ba + 1 + rem;
+      }
+    }
+    // entries of the block that are couplings of the next round (left to warp 0)
+    const bool skip00 = ba == 0 && bb == 2;
+    const bool skip10 = ba == 0 ? bb == 1 : bb == ba + 2;
+    const bool skip11 = ba == 14 && bb == 15;
+    __syncthreads();
+#pragma unroll 1
+    for (int rho = 0; rho < W2 - 1; ++rho) {
+      const int cur = rho & 1;
+      const float2* Sc = sm.p.S[cur];
+      float2* Sn = sm.p.S[cur ^ 1];
+      if (warp == 0) {
+        if (lane < W2 / 2) {
+          int x, y;
+          rr_slot(W2, rho, lane, x, y);
+          Sn[at(x, y)] = held;
+          if (rho + 1 < W2 - 1) {
+            int xa, yaa, xb, ybb;
+            rr_slot(W2, rho, sa, xa, yaa);
+            rr_slot(W2, rho, sb, xb, ybb);
+            const int i = ya ? yaa : xa, io = ya ? xa : yaa, j = yb ? ybb : xb, jo = yb ? xb : ybb;
+            const float4 ra = sm.rec[cur][sa], rb = sm.rec[cur][sb];
+            const float2 ca = make_float2(ra.x, ra.y), cb = make_float2(rb.x, rb.y);
+            float2 ga = make_float2(ra.z, ra.w), gb = make_float2(rb.z, rb.w);
+            if (!ya) ga = df_neg(ga);
+            if (!yb) gb = df_neg(gb);
+            const float2 t0 = df_rot(ca, Sc[at(i, j)], ga, Sc[at(io, j)]);
+            const float2 t1 = df_rot(ca, Sc[at(i, jo)], ga, Sc[at(io, jo)]);
+            rotate(rho + 1, df_rot(cb, t0, gb, t1), base, cur ^ 1);
+            if (rho + 2 < W2 - 1) base = base_gap(rho + 2);
+          }
+        }
+      } else if (warp < 5) {
+        if (bb > 0) {
+          int xa, yaa, xb, ybb;
+          rr_slot(W2, rho, ba, xa, yaa);
+          rr_slot(W2, rho, bb, xb, ybb);
+          const float4 ra = sm.rec[cur][ba], rb = sm.rec[cur][bb];
+          const float2 ca = make_float2(ra.x, ra.y), ga = make_float2(ra.z, ra.w), na = df_neg(ga);
+          const float2 cb = make_float2(rb.x, rb.y), gb = make_float2(rb.z, rb.w), nbg = df_neg(gb);
+          const int i00 = at(xa, xb), i01 = at(xa, ybb), i10 = at(yaa, xb), i11 = at(yaa, ybb);
+          const float2 v00 = Sc[i00], v01 = Sc[i01], v10 = Sc[i10], v11 = Sc[i11];
+          const float2 t00 = df_rot(ca, v00, na, v10), t10 = df_rot(ca, v10, ga, v00);
+          const float2 t01 = df_rot(ca, v01, na, v11), t11 = df_rot(ca, v11, ga, v01);
+          if (!skip00) Sn[i00] = df_rot(cb, t00, nbg, t01);
+          Sn[i01] = df_rot(cb, t01, gb, t00);
+          if (!skip10) Sn[i10] = df_rot(cb, t10, nbg, t11);
+          if (!skip11) Sn[i11] = df_rot(cb, t11, gb, t10);
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int k = 4 * (warp - 5) + i;
+          int x, y;
+          rr_slot(W2, rho, k, x, y);
+          const float4 r = sm.rec[cur][k];
+          const float2 c = make_float2(r.x, r.y), g = make_float2(r.z, r.w);
+          const float2 ux = sm.p.U[x][lane], uy = sm.p.U[y][lane];
+          sm.p.U[x][lane] = df_rot(c, ux, df_neg(g), uy);
+          sm.p.U[y][lane] = df_rot(c, uy, g, ux);
+        }
+      }
+      __syncthreads();
+    }
+    if (warp == 0 && mine) sm.any = 1u;
+  } else {
+    // the same sweep in FP64 instructions (c - 1 carried separately)
+    for (int e = tid; e < W2 * W2; e += SOLVE_THREADS) sm.U64[e / W2][e % W2] = (e / W2 == e % W2) ? 1.0 : 0.0;
+    __syncthreads();
+#pragma unroll 1
+    for (int rho = 0; rho < W2 - 1; ++rho) {
+      if (tid < W2 / 2) {
+        int x, y;
+        rr_slot(W2, rho, tid, x, y);
+        double t, cm1, s;
+        const int pi = min(x, y), qi = max(x, y);
+        const double apq = sm.A[pi][qi];
+        const bool rot = jacobi_pair<double>(sm.A[pi][pi], sm.A[qi][qi], apq, skip, t, cm1, s, skip_abs);
+        if (rot) {
+          sm.any = 1u;
+          sm.A[pi][pi] -= t * apq;
+          sm.A[qi][qi] += t * apq;
+          sm.A[pi][qi] = 0.0;
+          sm.A[qi][pi] = 0.0;
+        }
+        sm.cs[tid][0] = cm1;
+        sm.cs[tid][1] = x < y ? s : -s;
+      }
+      __syncthreads();
+      for (int task = tid; task < 120 + (W2 / 2) * W2; task += SOLVE_THREADS) {
         if (task < 120) {
-          // pair indices a < b from the triangular task number
           int a = 0, rem = task;
           while (rem >= 15 - a) {
             rem -= 15 - a;
             ++a;
           }
           const int b = a + 1 + rem;
-          if (more) {  // a block that holds a pair of the next round: warp 0
-            const int na = rr_partner(W2, rho + 1, pq[cur][a][0]), nq = rr_partner(W2, rho + 1, pq[cur][a][1]);
-            if (slot_of[cur][na] == b || slot_of[cur][nq] == b) continue;
-          }
-          block_update(a, b, cur);
+          int xa, ya, xb, yb;
+          rr_slot(W2, rho, a, xa, ya);
+          rr_slot(W2, rho, b, xb, yb);
+          double v00 = sm.A[xa][xb], v01 = sm.A[xa][yb], v10 = sm.A[ya][xb], v11 = sm.A[ya][yb];
+          rot_apply(sm.cs[a][0], sm.cs[a][1], v00, v10);
+          rot_apply(sm.cs[a][0], sm.cs[a][1], v01, v11);
+          rot_apply(sm.cs[b][0], sm.cs[b][1], v00, v01);
+          rot_apply(sm.cs[b][0], sm.cs[b][1], v10, v11);
+          sm.A[xa][xb] = sm.A[xb][xa] = v00;
+          sm.A[xa][yb] = sm.A[yb][xa] = v01;
+          sm.A[ya][xb] = sm.A[xb][ya] = v10;
+          sm.A[ya][yb] = sm.A[yb][ya] = v11;
         } else {
           const int e = task - 120, k = e / W2, j = e % W2;
-          if (!rot[cur][k]) continue;
-          const int p = pq[cur][k][0], q = pq[cur][k][1];
-          const double up = U[j][p], uq = U[j][q];
-          U[j][p] = fma(-cs[cur][k][0], uq, up);
-          U[j][q] = fma(cs[cur][k][1], up, uq);
+          int x, y;
+          rr_slot(W2, rho, k, x, y);
+          rot_apply(sm.cs[k][0], sm.cs[k][1], sm.U64[x][j], sm.U64[y][j]);
         }
       }
+      __syncthreads();
     }
-    __syncthreads();
   }
-  // U = U~ D
-  for (int e = tid; e < W2 * W2; e += blockDim.x) {
-    const int i = e % W2, j = e / W2;
-    U[i][j] *= dsc[j];
+  __syncthreads();
+  if (!sm.any) {
+    if (tid == 0) rotated[P] = 0;
+    return;
+  }
+  // U_P in fixed point, F = U 2^60 (|U| <= 1 up to rounding)
+  constexpr int NE = (W2 * W2 + SOLVE_THREADS - 1) / SOLVE_THREADS;
+  long long F[NE];
+#pragma unroll
+  for (int i = 0; i < NE; ++i) {
+    const int e = tid + i * SOLVE_THREADS;
+    F[i] = 0;
+    if (e < W2 * W2) {
+      const int row = e % W2, col = e / W2;
+      if (pairs) {
+        const float2 v = sm.p.U[col][row];
+        F[i] = __float2ll_rn(v.x * 0x1p60f) + __float2ll_rn(v.y * 0x1p60f);
+      } else {
+        F[i] = __double2ll_rn(sm.U64[col][row] * 0x1p60);
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < NE; ++i) {
+    const int e = tid + i * SOLVE_THREADS;
+    if (e < W2 * W2) {
+      const int row = e % W2, col = e / W2;
+      const long long u1 = (F[i] + (1LL << 29)) >> 30;
+      sm.f.u1[col][row] = (int)u1;
+      sm.f.u0[col][row] = (int)(F[i] - (u1 << 30));  // in [-2^29, 2^29)
+    }
   }
   __syncthreads();
   // One Newton-Schulz step on U_P (Sec. 4.3.4): U <- U - U E / 2, E = U^T U - I.
   // U_P carries the rounding of its 496 rotations; applied to all of A and V
   // every round, that departure from orthogonality would accumulate over the
-  // sweeps, so each U_P is made orthogonal to working precision first.
+  // sweeps, so each U_P is made orthogonal first.  E (symmetric: the 528
+  // entries i <= j, mirrored) from sums of integer products: u1 v1 exactly
+  // (at most 2^60 by Cauchy-Schwarz), the cross terms at weight 2^-30 (below
+  // 2^62.5), u0 v0 (below 2^-59 in all) left out.
+  for (int idx = tid; idx < 528; idx += SOLVE_THREADS) {
+    int i = 0, rem = idx;
+    while (rem >= W2 - i) {
+      rem -= W2 - i;
+      ++i;
+    }
+    const int j = i + rem;
+    long long g = (i == j) ? -(1LL << 60) : 0LL, x = 0;
+#pragma unroll
+    for (int k = 0; k < W2; k += 4) {
+      const int4 a1 = *reinterpret_cast<const int4*>(&sm.f.u1[i][k]), b1 = *reinterpret_cast<const int4*>(&sm.f.u1[j][k]);
+      const int4 a0 = *reinterpret_cast<const int4*>(&sm.f.u0[i][k]), b0 = *reinterpret_cast<const int4*>(&sm.f.u0[j][k]);
+      g += (long long)a1.x * b1.x + (long long)a1.y * b1.y + (long long)a1.z * b1.z + (long long)a1.w * b1.w;
+      x += (long long)a1.x * b0.x + (long long)a1.y * b0.y + (long long)a1.z * b0.z + (long long)a1.w * b0.w;
+      x += (long long)a0.x * b1.x + (long long)a0.y * b1.y + (long long)a0.z * b1.z + (long long)a0.w * b1.w;
+    }
+    const float ev = fmaf((float)x, 0x1p-90f, (float)g * 0x1p-60f);
+    sm.f.Ef[i][j] = ev;
+    sm.f.Ef[j][i] = ev;
+  }
+  __syncthreads();
+  // U E / 2 in FP32: |E| is about 2^-43, so its error is below 2^-65.  Warp w
+  // takes columns w, w + 9, ..; lane = row.
   {
-    // E is symmetric: the 528 entries i <= j, mirrored (S is free now: it holds E)
-    constexpr int NE = (528 + SOLVE_THREADS - 1) / SOLVE_THREADS;
-    double e3[NE];
-    int ij[NE];
+    float ur[W2];
 #pragma unroll
-    for (int t = 0; t < NE; ++t) {
-      const int idx = tid + t * SOLVE_THREADS;
-      e3[t] = 0.0;
-      ij[t] = -1;
-      if (idx < 528) {
-        int i = 0, rem = idx;
-        while (rem >= W2 - i) {
-          rem -= W2 - i;
-          ++i;
+    for (int k = 0; k < W2; ++k) ur[k] = (float)sm.f.u1[k][lane];  // U(lane, k) 2^30
+    long long Fn[4];
+#pragma unroll
+    for (int jj = 0; jj < 4; ++jj) {
+      const int j = warp + 9 * jj;
+      Fn[jj] = 0;
+      if (j < W2) {
+        float acc = 0.0f;
+#pragma unroll
+        for (int k = 0; k < W2; k += 4) {
+          const float4 ev = *reinterpret_cast<const float4*>(&sm.f.Ef[j][k]);
+          acc = fmaf(ur[k], ev.x, acc);
+          acc = fmaf(ur[k + 1], ev.y, acc);
+          acc = fmaf(ur[k + 2], ev.z, acc);
+          acc = fmaf(ur[k + 3], ev.w, acc);
         }
-        const int j = i + rem;
-        double acc = (i == j) ? -1.0 : 0.0;
-        for (int k = 0; k < W2; ++k) acc = fma(U[k][i], U[k][j], acc);
-        e3[t] = acc;
-        ij[t] = i * W2 + j;
+        Fn[jj] = ((long long)sm.f.u1[j][lane] << 30) + sm.f.u0[j][lane] - __float2ll_rn(acc * 0x1p29f);
       }
     }
     __syncthreads();
+    long long* Fs = reinterpret_cast<long long*>(&sm.f);  // [column][row], row stride LDS
 #pragma unroll
-    for (int t = 0; t < NE; ++t)
-      if (ij[t] >= 0) {
-        const int i = ij[t] / W2, j = ij[t] % W2;
-        S[i][j] = e3[t];
-        S[j][i] = e3[t];
-      }
-    __syncthreads();
-    // |E| is at the rounding level, so U E is formed in FP32 (its relative
-    // error 2^-24 of a 1e-15 correction is far below FP64 rounding); U and E
-    // are rounded to FP32 once (FP64 conversions issue on the slow FP64 pipe)
-    __shared__ float Uf[W2][W2 + 1], Ef[W2][W2 + 1];
-    for (int e = tid; e < W2 * W2; e += SOLVE_THREADS) {
-      const int i = e % W2, j = e / W2;
-      Uf[i][j] = (float)U[i][j];
-      Ef[i][j] = (float)S[i][j];
-    }
-    __syncthreads();
-    constexpr int NU = W2 * W2 / SOLVE_THREADS;
-    double u4[NU];
-#pragma unroll
-    for (int t = 0; t < NU; ++t) {
-      const int idx = tid + t * SOLVE_THREADS, i = idx % W2, j = idx / W2;
-      float acc = 0.0f;
-      for (int k = 0; k < W2; ++k) acc = fmaf(Uf[i][k], Ef[k][j], acc);
-      u4[t] = fma(-0.5, (double)acc, U[i][j]);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int t = 0; t < NU; ++t) {
-      const int idx = tid + t * SOLVE_THREADS, i = idx % W2, j = idx / W2;
-      U[i][j] = u4[t];
-    }
+    for (int jj = 0; jj < 4; ++jj)
+      if (warp + 9 * jj < W2) Fs[(warp + 9 * jj) * LDS + lane] = Fn[jj];
     __syncthreads();
   }
   // digits of U_P's columns: column c is "row" c of the right operand, over
-  // k = row of U_P; four threads per column, eight values each
+  // k = row of U_P; eight threads per column, four values each
   __nv_bfloat16* dst = Usl + (size_t)P * NSL * (USL_BYTES / 2);
-  if (tid < 4 * W2) {
-    const int c = tid >> 2, k0 = (tid & 3) * 8;
-    unsigned long long maxbits = 0;
-    for (int k = 0; k < W2; ++k) {
-      const unsigned long long b = (unsigned long long)__double_as_longlong(U[k][c]) & 0x7FFFFFFFFFFFFFFFULL;
-      maxbits = b > maxbits ? b : maxbits;
-    }
-    const int e = exp_of_maxbits(maxbits);
-    if ((tid & 3) == 0) Uexp[P * W2 + c] = e;
-    uint32_t d[8][NSL];
+  if (tid < 8 * W2) {
+    const long long* Fs = reinterpret_cast<const long long*>(&sm.f);
+    const int c = tid >> 3, k0 = (tid & 7) * 4;
+    long long v[4];
+    unsigned long long top = 0;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) digits_f32(U[k0 + j][c], e, d[j]);
+    for (int j = 0; j < 4; ++j) {
+      v[j] = Fs[c * LDS + k0 + j];
+      top |= (unsigned long long)(v[j] < 0 ? -v[j] : v[j]);  // same leading bit as the largest
+    }
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) top |= __shfl_xor_sync(0xffffffffu, top, o);
+    const int bits = 64 - __clzll((long long)top);  // max|F| < 2^bits
+    if ((tid & 7) == 0) Uexp[P * W2 + c] = bits - 60;
+    const int sh = bits - 56;  // Y = |F| 2^-sh rounded
+    uint32_t d[4][NSL];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const unsigned long long m = (unsigned long long)(v[j] < 0 ? -v[j] : v[j]);
+      const unsigned long long Y = sh > 0 ? (m + (1ULL << (sh - 1))) >> sh : m << -sh;
+      digits_of(Y, v[j] < 0 ? -1.0f : 1.0f, d[j]);
+    }
 #pragma unroll
     for (int sl = 0; sl < NSL; ++sl) {
-      uint4 q;
+      uint2 q;
       q.x = pack_bf16x2(d[0][sl], d[1][sl]);
       q.y = pack_bf16x2(d[2][sl], d[3][sl]);
-      q.z = pack_bf16x2(d[4][sl], d[5][sl]);
-      q.w = pack_bf16x2(d[6][sl], d[7][sl]);
-      *reinterpret_cast<uint4*>(reinterpret_cast<char*>(dst + (size_t)sl * (USL_BYTES / 2)) + kmaj16(c, k0)) = q;
+      *reinterpret_cast<uint2*>(reinterpret_cast<char*>(dst + (size_t)sl * (USL_BYTES / 2)) + kmaj16(c, k0)) = q;
     }
   }
   if (tid == 0) {
-    rotated[P] = any;
-    if (any && nrot) atomicAdd(nrot, 1u);
+    rotated[P] = 1;
+    if (nrot) atomicAdd(nrot, 1u);
   }
 }
 
