@@ -70,43 +70,51 @@ __global__ void widen(const float* __restrict__ V32, int N, int n, double* __res
 }
 
 // The rotation of pair (p, q), p < q, for the FP32 inner sweep: Algorithm 2
-// with the skip test of Algorithm 4 (compared in squares), t in the stable
-// form, c = 1 / sqrt(1 + t^2) by rsqrtf, c - 1 = -t^2 c / (1 + h) with
-// h = 1 / c = (1 + t^2) c; the new diagonal a_pp - t a_pq, a_qq + t a_pq.  The
-// approximate divisions and square roots (2 ulp) only perturb the angle: the
-// stage delivers Q_l to single precision and c, s belong to the same t.
+// with the skip test of Algorithm 4 (compared in squares) in half-angle form,
+// which has the shortest chain of special functions: z = |sin 2 theta| =
+// 1 / sqrt(1 + tau^2), c^2 = (1 + |tau| z) / 2, s = z / (2 c) with tau's sign
+// ('+' for 0), c - 1 = -s^2 / (1 + c), and t a_pq = s a_pq / c for the diagonal
+// a_pp - t a_pq, a_qq + t a_pq.  c - 1 comes from s, so an error of c enters
+// (1 + cm1)^2 + s^2 - 1 by less than a quarter.  |tau| is capped at 1e18: s
+// is then below FP32 resolution.  The flush-to-zero forms take half the latency
+// (19 against 41 cycles); their operands are normal numbers whenever apq^2 > 0
+// passes the skip test.  No branch: lanes that skip select zeros.
 struct Rot32 {
   float cm1, sig;
 };
-MPJ_DEV float sqrt_approx(float x) {
+MPJ_DEV float rcp_ftz(float x) {
   float r;
-  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+MPJ_DEV float rsqrt_ftz(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
 MPJ_DEV bool rot32(float& app, float& aqq, float apq, float skip, Rot32& rr) {
-  rr.cm1 = 0.0f;
-  rr.sig = 0.0f;
-  if (!(apq * apq > (skip * skip) * fabsf(app * aqq))) return false;
-  const float tau = __fdividef(aqq - app, 2.0f * apq);
-  const float r = sqrt_approx(fmaf(tau, tau, 1.0f));
-  const float ta = __fdividef(1.0f, fabsf(tau) + r);
-  const float t = (tau >= 0.0f) ? ta : -ta;
-  const float w = fmaf(t, t, 1.0f);
-  const float c = rsqrtf(w);
-  const float h = w * c;
-  rr.cm1 = -(t * t) * __fdividef(c, 1.0f + h);
-  rr.sig = t * c;
-  app = fmaf(-t, apq, app);
-  aqq = fmaf(t, apq, aqq);
-  return true;
+  const bool rot = apq * apq > (skip * skip) * fabsf(app * aqq);
+  const float tau = (aqq - app) * rcp_ftz(2.0f * apq), at = fminf(fabsf(tau), 1e18f);
+  const float z = rsqrt_ftz(fmaf(at, at, 1.0f));
+  const float c2 = fmaf(0.5f * at, z, 0.5f);
+  const float ic = rsqrt_ftz(c2);
+  const float sa = 0.5f * z * ic, s = tau >= 0.0f ? sa : -sa;
+  const float c1 = fmaf(c2, ic, 1.0f);  // 1 + c
+  const float ta = rot ? s * ic * apq : 0.0f;
+  rr.cm1 = rot ? -(s * s) * rcp_ftz(c1) : 0.0f;
+  rr.sig = rot ? s : 0.0f;
+  app -= ta;
+  aqq += ta;
+  return rot;
 }
 
 // One entry of a rotated pair: `own` with the other index's entry `oth`
 // (sg = -sig for the pair's first index, +sig for its second).
 MPJ_DEV float rot_one(float cm1, float sg, float own, float oth) { return fmaf(cm1, own, fmaf(sg, oth, own)); }
 
-// v with a zero bit inserted at position h
+// v with a zero bit inserted at position h, and with bit h taken out
 MPJ_DEV int ins0(int v, int h) { return ((v >> h) << (h + 1)) | (v & ((1 << h) - 1)); }
+MPJ_DEV int del0(int v, int h) { return ((v >> (h + 1)) << h) | (v & ((1 << h) - 1)); }
 
 // One CTA per block pair of outer round R: inner sweep on the 32 x 32
 // subproblem; writes the rotated subproblem S (column-major), the accumulated
@@ -122,18 +130,24 @@ MPJ_DEV int ins0(int v, int h) { return ((v >> h) << (h + 1)) | (v & ((1 << h) -
 // (i ^ j) * SLD + min(i, j), so a block is read and written once without a
 // mirror.  What bounds the kernel is the chain coupling -> angle -> records ->
 // next round's coupling: the 16 couplings of the next round all lie in eight
-// blocks of this one, so warp 0 recomputes just those 16 entries, forms the
-// next round's rotations and leaves the blocks themselves to warps 1-4 (one
-// block per thread) and U to warps 5-8 (lane = row, four column pairs each).
+// blocks of this one, so warp 0 recomputes just those 16 entries and forms the
+// next round's rotations, with every address of the round computed before the
+// barrier that opens it; the blocks are left to warps 1-8 (half a block, one
+// row, per thread) and U to warps 9-16 (lane = row, two column pairs each).
 // S alternates between two buffers, so one barrier per round is enough.
 // Measured at n = 4096 (128 CTAs): circle ordering, two barriers, IEEE
-// divisions 23.8 us per launch; this form 18.1 us.  The sweeps to reach
+// divisions 23.8 us per launch; two index sets per thread and four-task warps
+// 18.4 us; this form 12.3 us.  The sweeps to reach
 // the stopping test are the same or one fewer (n = 96 .. 512, three spectra).
-constexpr int S32_THREADS = 288;
+constexpr int S32_THREADS = 544;
 constexpr int SLD = 40;  // row stride of the packed S (8 more than 32: rows of d, d + 1, .. start 8 banks apart)
-__global__ void __launch_bounds__(S32_THREADS) solve32(const float* __restrict__ A32, int N, int nb, int R,
-                                               float* __restrict__ Sbuf, float* __restrict__ Ubuf, bool hq,
-                                               bool urow, unsigned* __restrict__ Mbuf) {
+// The CTA's barrier from the three roles' own code paths.
+MPJ_DEV void s32_barrier() { asm volatile("bar.sync 0, %0;\n" ::"n"(S32_THREADS) : "memory"); }
+
+template <bool HQ>
+__global__ void __launch_bounds__(S32_THREADS, 1) solve32(const float* __restrict__ A32, int N, int nb, int R,
+                                               float* __restrict__ Sbuf, float* __restrict__ Ubuf, bool urow,
+                                               unsigned* __restrict__ Mbuf) {
   __shared__ float S[2][W2 * SLD];
   __shared__ float U[W2][LD];  // U[column][row]
   __shared__ float dg[W2];     // the diagonal (warp 0 only)
@@ -153,97 +167,113 @@ __global__ void __launch_bounds__(S32_THREADS) solve32(const float* __restrict__
     U[lj][li] = (li == lj) ? 1.0f : 0.0f;
   }
   __syncthreads();
-  const float skip = hq ? 0x1p-11f : 0x1p-24f;
-  unsigned tmask = 0u;  // warp 0: the indices that rotated so far
-  float held = 0.0f;    // warp 0: the pair's own coupling after its rotation
-  // rotation of pair k of round r from its coupling, into rec[buf]
-  auto rotate = [&](int k, int p, int q, float apq, int buf) {
-    float app = dg[p], aqq = dg[q];
-    Rot32 rr;
-    const bool rot = rot32(app, aqq, apq, skip, rr);
-    if (hq && rot) {  // c and s as binary16, new diagonal rounded
-      rr.cm1 = qh(1.0f + rr.cm1, true) - 1.0f;
-      rr.sig = qh(rr.sig, true);
-      app = qh(app, true);
-      aqq = qh(aqq, true);
-    }
-    rec[buf][k] = rr;
-    if (rot) {
-      dg[p] = app;
-      dg[q] = aqq;
-    }
-    held = rot ? 0.0f : apq;
-    if (Mbuf) {
-      const unsigned bits = rec_rotated(rr.cm1, rr.sig) ? ((1u << p) | (1u << q)) : 0u;
-      tmask |= __reduce_or_sync(0x0000FFFFu, bits);  // the 16 record lanes of warp 0
-    }
-  };
+  const float skip = HQ ? 0x1p-11f : 0x1p-24f;
   if (warp == 0) {
-    if (lane < W2 / 2) rotate(lane, 2 * lane, 2 * lane + 1, S[0][SLD + 2 * lane], 0);
-    __syncwarp();
-  }
-  // the block of threads 32 .. 151: pairs with 4-bit labels xl and yl = xl ^ dl,
-  // xl's bit at dl's highest bit zero: 15 x 8 unordered label pairs
-  const int bt = tid - 32, dl = 1 + (bt >> 3);
-  const int xl = ins0(bt & 7, 31 - __clz(dl)), yl = xl ^ dl;
-  __syncthreads();
-#pragma unroll 1
-  for (int r = 1; r < W2; ++r) {
-    const int cur = (r - 1) & 1;
-    const float* Sc = S[cur];
-    float* Sn = S[cur ^ 1];
-    const int h = 31 - __clz(r);
-    const int rn = r + 1;  // the next round (none after r = 31)
-    if (warp == 0) {
+    unsigned tmask = 0u;  // the indices that rotated so far
+    float held = 0.0f;    // the pair's own coupling after its rotation
+    const int k = lane & 15;
+    // rotation of pair (p, q), record k, from its coupling, into rec[buf]
+    auto rotate = [&](int p, int q, float app, float aqq, float apq, int buf) {
+      Rot32 rr;
+      const bool rot = rot32(app, aqq, apq, skip, rr);
+      if (HQ) {  // c and s as binary16, new diagonal rounded
+        rr.cm1 = qh(1.0f + rr.cm1, true) - 1.0f;
+        rr.sig = qh(rr.sig, true);
+        app = rot ? qh(app, true) : app;
+        aqq = rot ? qh(aqq, true) : aqq;
+      }
+      __syncwarp();  // every lane has read the diagonal
       if (lane < W2 / 2) {
-        Sn[r * SLD + ins0(lane, h)] = held;
-        if (rn < W2) {
-          const int hn = 31 - __clz(rn);
-          const int p = ins0(lane, hn), q = p ^ rn;
-          // this round's pairs of p and of q: records and the side of each
-          const bool p2 = (p >> h) & 1, q2 = (q >> h) & 1;
-          const int pr = p2 ? p ^ r : p, qr = q2 ? q ^ r : q;
-          const Rot32 ra = rec[cur][((pr >> (h + 1)) << h) | (pr & ((1 << h) - 1))];
-          const Rot32 rb = rec[cur][((qr >> (h + 1)) << h) | (qr & ((1 << h) - 1))];
-          const int po = p ^ r, qo = q ^ r, dA = rn * SLD, dB = (rn ^ r) * SLD;
-          const float e00 = Sc[dA + min(p, q)], e01 = Sc[dB + min(p, qo)];
-          const float e10 = Sc[dB + min(po, q)], e11 = Sc[dA + min(po, qo)];
-          const float sa = p2 ? ra.sig : -ra.sig, sb = q2 ? rb.sig : -rb.sig;
-          const float t0 = rot_one(ra.cm1, sa, e00, e10), t1 = rot_one(ra.cm1, sa, e01, e11);
-          rotate(lane, p, q, qh(rot_one(rb.cm1, sb, t0, t1), hq), cur ^ 1);
-        }
+        rec[buf][k] = rr;
+        dg[p] = app;
+        dg[q] = aqq;
       }
-    } else if (warp < 5) {
-      if (bt < 120) {
-        const int x = ins0(xl, h), y = ins0(yl, h), x2 = x ^ r, y2 = y ^ r;
-        const Rot32 ra = rec[cur][xl], rb = rec[cur][yl];
-        const int d0 = x ^ y, d1 = d0 ^ r;
-        const int i00 = d0 * SLD + min(x, y), i01 = d1 * SLD + min(x, y2);
-        const int i10 = d1 * SLD + min(x2, y), i11 = d0 * SLD + min(x2, y2);
-        const float v00 = Sc[i00], v01 = Sc[i01], v10 = Sc[i10], v11 = Sc[i11];
-        const float t00 = rot_one(ra.cm1, -ra.sig, v00, v10), t10 = rot_one(ra.cm1, ra.sig, v10, v00);
-        const float t01 = rot_one(ra.cm1, -ra.sig, v01, v11), t11 = rot_one(ra.cm1, ra.sig, v11, v01);
-        if (d0 != rn) {  // warp 0 holds the next round's couplings
-          Sn[i00] = qh(rot_one(rb.cm1, -rb.sig, t00, t01), hq);
-          Sn[i11] = qh(rot_one(rb.cm1, rb.sig, t11, t10), hq);
-        }
-        if (d1 != rn) {
-          Sn[i01] = qh(rot_one(rb.cm1, rb.sig, t01, t00), hq);
-          Sn[i10] = qh(rot_one(rb.cm1, -rb.sig, t10, t11), hq);
-        }
+      held = rot ? 0.0f : apq;
+      if (Mbuf) {
+        const unsigned bits = rec_rotated(rr.cm1, rr.sig) ? ((1u << p) | (1u << q)) : 0u;
+        tmask |= __reduce_or_sync(0xFFFFFFFFu, bits);
       }
-    } else {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int k = 4 * (warp - 5) + i, p = ins0(k, h), q = p ^ r;
-        const Rot32 rr = rec[cur][k];
-        const float up = U[p][lane], uq = U[q][lane];
-        U[p][lane] = qh(rot_one(rr.cm1, -rr.sig, up, uq), hq);
-        U[q][lane] = qh(rot_one(rr.cm1, rr.sig, uq, up), hq);
+    };
+    rotate(2 * k, 2 * k + 1, dg[2 * k], dg[2 * k + 1], S[0][SLD + 2 * k], 0);
+    int p_cur = 2 * k;
+#pragma unroll 1
+    for (int r = 1; r < W2; ++r) {
+      const int cur = (r - 1) & 1;
+      const int h = 31 - __clz(r), rn = r + 1, hn = 31 - __clz(rn);
+      const int p = ins0(k, hn), q = p ^ rn, po = p ^ r, qo = q ^ r;
+      // this round's pairs of p and of q: records and the side of each
+      const bool p2 = (p >> h) & 1, q2 = (q >> h) & 1;
+      const Rot32* pa = &rec[cur][del0(p2 ? po : p, h)];
+      const Rot32* pb = &rec[cur][del0(q2 ? qo : q, h)];
+      const int dA = (rn & 31) * SLD, dB = ((rn ^ r) & 31) * SLD;
+      const int i00 = dA + min(p, q), i11 = dA + min(po, qo);
+      const int i01 = dB + min(p, qo), i10 = dB + min(po, q);
+      float* Sh = &S[cur ^ 1][r * SLD + p_cur];
+      const float* Sc = S[cur];
+      s32_barrier();
+      if (lane < W2 / 2) *Sh = held;
+      if (rn < W2) {
+        const Rot32 ra = *pa, rb = *pb;
+        const float app = dg[p], aqq = dg[q];
+        const float e00 = Sc[i00], e01 = Sc[i01], e10 = Sc[i10], e11 = Sc[i11];
+        const float sa = p2 ? ra.sig : -ra.sig, sb = q2 ? rb.sig : -rb.sig;
+        const float t0 = rot_one(ra.cm1, sa, e00, e10), t1 = rot_one(ra.cm1, sa, e01, e11);
+        rotate(p, q, app, aqq, qh(rot_one(rb.cm1, sb, t0, t1), HQ), cur ^ 1);
+        p_cur = p;
       }
     }
-    __syncthreads();
+    if (lane == 0 && Mbuf) Mbuf[slot] = tmask;
+  } else if (warp < 9) {
+    // half a block: pairs with 4-bit labels xl and yl = xl ^ dl, xl's bit at
+    // dl's highest bit zero (15 x 8 unordered label pairs), and the row of
+    // xl's first (side 0) or second index
+    const int bt = (tid - 32) >> 1, side = tid & 1, dl = 1 + (bt >> 3);
+    const int xl = ins0(bt & 7, 31 - __clz(dl)), yl = xl ^ dl;
+    const bool on = bt < 120;
+#pragma unroll 1
+    for (int h = 0; h < 5; ++h) {
+      const int x = ins0(xl, h), y = ins0(yl, h), d0 = x ^ y;
+#pragma unroll 1
+      for (int r = 1 << h; r < (2 << h); ++r) {
+        const int cur = (r - 1) & 1, rn = r + 1;
+        const int i = side ? x ^ r : x, io = i ^ r, y2 = y ^ r, d1 = d0 ^ r;
+        const int ds = side ? d1 : d0, dt = side ? d0 : d1;  // i ^ y and i ^ y2
+        const int i0 = ds * SLD + min(i, y), i1 = dt * SLD + min(i, y2);
+        const int o0 = dt * SLD + min(io, y), o1 = ds * SLD + min(io, y2);
+        const float* Sc = S[cur];
+        float* Sn = S[cur ^ 1];
+        s32_barrier();
+        if (on) {
+          const Rot32 ra = rec[cur][xl], rb = rec[cur][yl];
+          const float v0 = Sc[i0], v1 = Sc[i1], w0 = Sc[o0], w1 = Sc[o1];
+          const float sg = side ? ra.sig : -ra.sig;
+          const float t0 = rot_one(ra.cm1, sg, v0, w0), t1 = rot_one(ra.cm1, sg, v1, w1);
+          // warp 0 holds the next round's couplings
+          if (ds != rn) Sn[i0] = qh(rot_one(rb.cm1, -rb.sig, t0, t1), HQ);
+          if (dt != rn) Sn[i1] = qh(rot_one(rb.cm1, rb.sig, t1, t0), HQ);
+        }
+      }
+    }
+  } else {
+    const int k0 = 2 * (warp - 9);
+#pragma unroll 1
+    for (int h = 0; h < 5; ++h) {
+      const int pa = ins0(k0, h), pb = ins0(k0 + 1, h);
+#pragma unroll 1
+      for (int r = 1 << h; r < (2 << h); ++r) {
+        const int cur = (r - 1) & 1;
+        float *u0 = &U[pa][lane], *u1 = &U[pa ^ r][lane], *w0 = &U[pb][lane], *w1 = &U[pb ^ r][lane];
+        s32_barrier();
+        const Rot32 ra = rec[cur][k0], rb = rec[cur][k0 + 1];
+        const float a0 = *u0, a1 = *u1, b0 = *w0, b1 = *w1;
+        *u0 = qh(rot_one(ra.cm1, -ra.sig, a0, a1), HQ);
+        *u1 = qh(rot_one(ra.cm1, ra.sig, a1, a0), HQ);
+        *w0 = qh(rot_one(rb.cm1, -rb.sig, b0, b1), HQ);
+        *w1 = qh(rot_one(rb.cm1, rb.sig, b1, b0), HQ);
+      }
+    }
   }
+  s32_barrier();
   float* So = Sbuf + (size_t)slot * W2 * W2;
   float* Uo = Ubuf + (size_t)slot * W2 * W2;
   for (int e = tid; e < W2 * W2; e += S32_THREADS) {
@@ -251,7 +281,6 @@ __global__ void __launch_bounds__(S32_THREADS) solve32(const float* __restrict__
     So[e] = li == lj ? dg[li] : S[1][(li ^ lj) * SLD + min(li, lj)];
     Uo[e] = urow ? U[li][lj] : U[lj][li];
   }
-  if (tid == 0 && Mbuf) Mbuf[slot] = tmask;
 }
 
 
@@ -557,8 +586,8 @@ cudaError_t stage1_sweep(const Stage1Bufs& b, cudaStream_t s, SideStream* side) 
     float* Ubuf = b.Ub[par];
     if (side && vpending[par]) S1_TRY(cudaStreamWaitEvent(s, side->done[par], 0));
     unsigned* Mbuf = b.sparse ? b.Mb[par] : nullptr;
-    S1_TRY(mpj_launch_pdl(solve32, dim3(npairs), dim3(S32_THREADS), 0, s, (const float*)b.A32, N, nb, R, Sbuf, Ubuf,
-                          b.half, b.tc != 1, Mbuf));
+    S1_TRY(mpj_launch_pdl(b.half ? solve32<true> : solve32<false>, dim3(npairs), dim3(S32_THREADS), 0, s,
+                          (const float*)b.A32, N, nb, R, Sbuf, Ubuf, b.tc != 1, Mbuf));
     auto vmul = b.sparse ? rmul32<R32_ALL, true> : rmul32<R32_ALL, false>;
     // V <- V U~
     if (side) {
