@@ -226,37 +226,112 @@ MPJ_DEV float2 df_split(double x, int eo) {
   return make_float2(sg * (float)(unsigned)(m >> 29) * h, sg * (float)(unsigned)(m & 0x1FFFFFFFULL) * l);
 }
 
-// Algorithm 2 on FP32 pairs: coupling a, d = a_qq - a_pp, giving t (the root
-// of a t^2 + d t - a with |t| <= 1, '+' for d = 0), c = 1 / sqrt(1 + t^2) and
-// s = t c.  t and c start from FP32 seeds; one Newton step each on a residual
-// formed with pairs takes them to the pairs' precision.
-MPJ_DEV void df_angle(float2 a, float2 d, float2& t, float2& c, float2& s) {
-  const float tau = __fdividef(d.x, 2.0f * a.x), at = fabsf(tau);
-  float root;
-  asm("sqrt.approx.f32 %0, %1;" : "=f"(root) : "f"(fmaf(at, at, 1.0f)));
-  float t0 = at > 1e9f ? __fdividef(0.5f, at) : __fdividef(1.0f, at + root);
-  t0 = tau >= 0.0f ? t0 : -t0;
-  const float c0 = rsqrtf(fmaf(t0, t0, 1.0f));
-  // f = (a t0 + d) t0 - a, t = t0 - f / (2 a t0 + d)
-  const float inv = __fdividef(1.0f, fmaf(2.0f * a.x, t0, d.x));
-  const float2 t0p = make_float2(t0, 0.0f);
-  const float2 g = df_add(d, df_mul(a, t0p));
-  const float2 f = df_add(df_mul(g, t0p), df_neg(a));
-  const float dt = f.x * inv;
-  t.x = __fsub_rn(t0, dt);
-  t.y = __fsub_rn(__fsub_rn(t0, t.x), dt);
-  // e = 1 - (1 + t^2) c0^2, c = c0 (1 + e / 2 + 3 e^2 / 8)
-  const float2 t2 = df_mul(t, t);
-  const float wh = __fadd_rn(1.0f, t2.x);
-  const float wl = __fadd_rn(__fsub_rn(t2.x, __fsub_rn(wh, 1.0f)), t2.y);
+// Two values held as pairs (hi and lo parts packed two and two): the packed
+// FP32 instructions do both with one issue slot.
+struct Df2 {
+  unsigned long long h, l;
+};
+MPJ_DEV unsigned long long pk(float a, float b) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+MPJ_DEV void unpk(unsigned long long v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+MPJ_DEV unsigned long long mul2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+MPJ_DEV unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+MPJ_DEV unsigned long long add2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+MPJ_DEV unsigned long long sub2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+// Two rotations' coefficients for df2_rot: c, s and their negatives.
+struct RotC {
+  unsigned long long ch, cl, nch, sh, sl, nsh, nsl;
+};
+// c x + s y for two (x, y) (NEG: c x - s y); the products' errors are exact and
+// enter the low parts, the leading parts are added with their error.
+template <bool NEG>
+MPJ_DEV Df2 df2_rot(const RotC& r, const Df2& x, const Df2& y) {
+  const unsigned long long sh = NEG ? r.nsh : r.sh, nsh = NEG ? r.sh : r.nsh, sl = NEG ? r.nsl : r.sl;
+  const unsigned long long np = mul2(r.nch, x.h), nq = mul2(nsh, y.h);  // minus the products
+  const unsigned long long e = fma2(r.cl, x.h, fma2(r.ch, x.l, fma2(r.ch, x.h, np)));
+  const unsigned long long f = fma2(sl, y.h, fma2(sh, y.l, fma2(sh, y.h, nq)));
+  const unsigned long long n = add2(np, nq), bb = sub2(n, np);
+  const unsigned long long er = add2(sub2(np, sub2(n, bb)), sub2(nq, bb));
+  const unsigned long long lo = sub2(add2(e, f), er);
+  Df2 o;
+  o.h = sub2(lo, n);
+  o.l = sub2(lo, add2(o.h, n));
+  return o;
+}
+
+MPJ_DEV float rcp_ftz(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+MPJ_DEV float rsqrt_ftz(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+MPJ_DEV float sqrt_ftz(float x) {
+  float r;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// Algorithm 2 on FP32 pairs for the slot's indices (x, y): coupling a, d =
+// a_yy - a_xx, giving t (the root of a t^2 + d t - a with |t| <= 1, the sign of
+// `tie` for d = 0), c = 1 / sqrt(1 + t^2) and s = t c.  From an FP32 seed t0,
+// one Newton step with the residual formed in pairs gives t = t0 - dt to about
+// 2^-44; c and s are formed at t0 in pairs beside it (c by one step from its
+// own FP32 seed) and moved to t by their derivatives -t c^3 and c^3, which
+// leaves dt^2.  (|a| < 2^-110 gives values that the caller does not use.)
+MPJ_DEV void df_angle(float2 a, float2 d, float tie, float2& t, float2& c, float2& s) {
+  const float tau = d.x * rcp_ftz(2.0f * a.x), at = fabsf(tau);
+  const float den = at > 1e9f ? 2.0f * at : at + sqrt_ftz(fmaf(at, at, 1.0f));
+  const float t0 = copysignf(rcp_ftz(den), tau == 0.0f ? tie : tau);
+  // f = (a t0 + d) t0 - a, dt = f / (2 a t0 + d); the leading parts of f
+  // cancel exactly (they agree to the seed's 2^-21)
+  const float inv = rcp_ftz(fmaf(2.0f * a.x, t0, d.x));
+  const float p = __fmul_rn(a.x, t0);
+  const float pe = __fmaf_rn(a.y, t0, __fmaf_rn(a.x, t0, -p));
+  const float g = __fadd_rn(p, d.x), bb = __fsub_rn(g, p);
+  const float q = __fmul_rn(g, t0);
+  const float ge = __fadd_rn(__fadd_rn(__fsub_rn(p, __fsub_rn(g, bb)), __fsub_rn(d.x, bb)), __fadd_rn(pe, d.y));
+  const float qe = __fmaf_rn(ge, t0, __fmaf_rn(g, t0, -q));
+  const float dt = __fadd_rn(__fsub_rn(q, a.x), __fsub_rn(qe, a.y)) * inv;
+  // c at t0: e = 1 - (1 + t0^2) c0^2, c0 (1 + e / 2 + 3 e^2 / 8)
+  const float c0 = rsqrt_ftz(fmaf(t0, t0, 1.0f));
   const float u = __fmul_rn(c0, c0), ue = __fmaf_rn(c0, c0, -u);
+  const float t2 = __fmul_rn(t0, t0), wh = __fadd_rn(1.0f, t2);
+  const float wl = __fadd_rn(__fsub_rn(t2, __fsub_rn(wh, 1.0f)), __fmaf_rn(t0, t0, -t2));
   const float2 m = df_mul(make_float2(wh, wl), make_float2(u, ue));
   const float e = __fsub_rn(__fsub_rn(1.0f, m.x), m.y);
-  const float corr = c0 * fmaf(0.375f * e, e, 0.5f * e);
-  c.x = __fadd_rn(c0, corr);
-  c.y = __fadd_rn(__fsub_rn(c0, c.x), corr);
-  const float2 sp = df_mul(t, c);
-  s = df_norm(sp.x, sp.y);
+  const float cc = c0 * fmaf(0.375f * e, e, 0.5f * e), c3 = c0 * u;
+  // s at t0: t0 (c0 + cc)
+  const float sp = __fmul_rn(t0, c0);
+  const float se = __fmaf_rn(t0, cc, __fmaf_rn(t0, c0, -sp));
+  const float co = __fmaf_rn(t0 * c3, dt, cc), so = __fmaf_rn(-c3, dt, se);
+  c.x = __fadd_rn(c0, co);
+  c.y = __fadd_rn(__fsub_rn(c0, c.x), co);
+  s = df_norm(sp, so);
+  t.x = __fsub_rn(t0, dt);
+  t.y = __fsub_rn(__fsub_rn(t0, t.x), dt);
 }
 
 // One CTA per block pair of round R: one inner round-robin sweep (circle
@@ -278,21 +353,31 @@ MPJ_DEV void df_angle(float2 a, float2 d, float2& t, float2& c, float2& s) {
 // 2^100 between a coupling and the diagonal: graded matrices) run the same
 // sweep in FP64 instructions instead.
 //
-// What bounds it: the chain coupling -> angle -> record -> next coupling.  The
-// 16 couplings of the next round lie in blocks known in advance, so warp 0
-// recomputes just those entries and the next round's rotations while warps
-// 1-4 update the 2 x 2 blocks (one per thread) and warps 5-8 U_P (lane = row,
-// four column pairs each); the couplings alternate between two buffers, so
-// one barrier per round is enough.  In FP64 instructions the chain alone was
-// about 60 dependent instructions of 65 cycles per round.  Measured at
-// n = 4096 (128 CTAs): 101 us per launch in FP64, 34.5 us in this form.
-constexpr int SOLVE_THREADS = 288;
+// What bounds it: the chain coupling -> angle -> record -> next coupling, and
+// beside it the number of instructions a warp has to get through per round.
+// Positions instead of indices: slot k's x is at position k, its y at 31 - k,
+// so a round rotates (k, 31 - k) and every address is a constant of the thread;
+// moving on to the next round takes position p to p - 1 (0 to 30, 31 stays),
+// done by writing the new values where they belong next.  The 16 couplings of
+// the next round lie in blocks known in advance: warp 0 recomputes just those
+// entries and the next round's rotations, eight warps update the 2 x 2 blocks
+// (one row of a block per thread) and eight U_P (in registers, eight lanes per
+// row).  The couplings alternate between two buffers, so one barrier per round
+// is enough.  Three warps rest: they share warp 0's scheduler, and its
+// instructions should not queue behind theirs.  In FP64 instructions the chain
+// alone was about 60 dependent instructions of 65 cycles per round.  Measured
+// at n = 4096 (128 CTAs): 101 us per launch in FP64, 34.8 us in pairs with two
+// 288-thread roles and index arithmetic per round, 24.6 us in this form.
+constexpr int SOLVE_THREADS = 640;
+constexpr int SWEEP_THREADS = 17 * 32;  // warps 0 - 7, 9 - 11, 13 - 15, 17 - 19
+constexpr int SSTR = 136;  // stride of the four entries' arrays (120 blocks; 64 bytes off a multiple of 128)
 constexpr int UFL = 36;  // row stride of the fixed-point U (16-byte rows, conflict-free 16-byte reads)
 struct SolveSmem {
   union {
     struct {
-      float2 S[2][W2 * LDS];  // couplings {i, j} at max(i, j) * LDS + min(i, j)
-      float2 U[W2][LDS];      // U[column][row]
+      float2 S[2][4 * SSTR];       // couplings by block, see pos_at
+      float2 U[W2][LDS];           // U[column][row]
+      float2 gap[W2 - 1][W2 / 2];  // starting a_yy - a_xx of each round's slots
     } p;
     double U64[W2][LDS];  // FP64 form: U[column][row]
     struct {
@@ -302,13 +387,36 @@ struct SolveSmem {
   };
   double A[W2][LDS];      // the subproblem as loaded; FP64 form: in place
   double cs[W2 / 2][2];   // FP64 form: c - 1, s
-  float4 rec[2][W2 / 2];  // c, sig oriented to the slot's (x, y)
-  float2 corr[W2];        // change of the diagonal (scaled pair)
-  float d0[W2];           // starting diagonal (scaled)
+  float4 rec[2][W2 / 2];  // c, s oriented to the slot's (x, y)
   unsigned emax_off, emin_off, emax_dg, any;
 };
 
-__global__ void __launch_bounds__(SOLVE_THREADS) blk_solve(const double* __restrict__ A, int lda, int n, int nb, int R,
+// The packed coefficients of two rotations from their records (c, s as pairs).
+MPJ_DEV RotC rot_coef(const float4& a, const float4& b) {
+  return RotC{pk(a.x, b.x), pk(a.y, b.y), pk(-a.x, -b.x), pk(a.z, b.z), pk(a.w, b.w), pk(-a.z, -b.z), pk(-a.w, -b.w)};
+}
+
+// The barrier of the sweep's 17 warps.
+MPJ_DEV void solve_barrier() { asm volatile("bar.sync 1, %0;\n" ::"n"(SWEEP_THREADS) : "memory"); }
+
+// Position p of this round in the next one, and the position it came from.
+MPJ_DEV int pos_next(int p) { return p == 31 ? 31 : p == 0 ? 30 : p - 1; }
+MPJ_DEV int pos_prev(int p) { return p == 31 ? 31 : p == 30 ? 0 : p + 1; }
+// Where the coupling of positions i and j (of different slots) is kept: one
+// array per place in the 2 x 2 block (row x or y, column x or y), one element
+// per block of slots a < b, so a warp reads its blocks without bank conflicts.
+MPJ_DEV int pos_at(int i, int j) {
+  const int si = i < 16 ? i : 31 - i, sj = j < 16 ? j : 31 - j;
+  const int a = min(si, sj), b = max(si, sj), ea = si < sj ? i > 15 : j > 15, eb = si < sj ? j > 15 : i > 15;
+  return (2 * ea + eb) * SSTR + (a * (31 - a)) / 2 + (b - a - 1);
+}
+
+// CTAS: resident CTAs per SM the registers are limited for.  One (78 registers)
+// has the shorter latency and is taken when every subproblem of a round finds
+// its own SM; beyond that two (48 registers) have the higher rate: 16 against 21
+// us per subproblem and SM.
+template <int CTAS>
+__global__ void __launch_bounds__(SOLVE_THREADS, CTAS) blk_solve(const double* __restrict__ A, int lda, int n, int nb, int R,
                                                  double skip, double skip_abs, __nv_bfloat16* __restrict__ Usl,
                                                  int* __restrict__ Uexp, int* __restrict__ rotated,
                                                  unsigned* __restrict__ nrot) {
@@ -324,12 +432,18 @@ __global__ void __launch_bounds__(SOLVE_THREADS) blk_solve(const double* __restr
   }
   __syncthreads();
   pdl_wait();
+  constexpr int NE = (W2 * W2 + SOLVE_THREADS - 1) / SOLVE_THREADS;
+  double v0[NE];
   {
     unsigned mo = 0u, mn = 0xFFFFu, md = 0u, big = 0u;
-    for (int e = tid; e < W2 * W2; e += SOLVE_THREADS) {
-      const int li = e % W2, lj = e / W2;
+#pragma unroll
+    for (int it = 0; it < NE; ++it) {
+      const int e = tid + it * SOLVE_THREADS, li = e % W2, lj = e / W2;
+      v0[it] = 0.0;
+      if (e >= W2 * W2) continue;
       const int gi = gidx(I, J, li), gj = gidx(I, J, lj);
       const double v = (gi < n && gj < n) ? A[(size_t)gj * lda + gi] : 0.0;
+      v0[it] = v;
       sm.A[li][lj] = v;
       const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFULL;
       const unsigned ex = (unsigned)(b >> 52);
@@ -362,151 +476,172 @@ __global__ void __launch_bounds__(SOLVE_THREADS) blk_solve(const double* __restr
   const int etop = max(emax_off, (int)sm.emax_dg);
   const bool pairs = emin_off > 0 && emax_off - emin_off <= 70 && etop - emin_off <= 100 && etop < 2000;
   const int eo = emax_off - 1022;  // couplings scaled by 2^-eo: at most 1
-  __syncthreads();
-  if (tid == 0) sm.any = 0u;
   if (pairs) {
-    for (int e = tid; e < W2 * W2; e += SOLVE_THREADS) {
-      const int li = e % W2, lj = e / W2;
-      if (li == lj) {
-        sm.corr[li] = make_float2(0.0f, 0.0f);
-        sm.d0[li] = df_split(sm.A[li][li], eo).x;
-      } else if (li > lj) {
-        sm.p.S[0][li * LDS + lj] = df_split(sm.A[li][lj], eo);
-      }
-      sm.p.U[lj][li] = make_float2(li == lj ? 1.0f : 0.0f, 0.0f);
-    }
-    // skip_abs 2^-eo rounded to FP32 (infinite when it is beyond every coupling)
-    float sabs;
-    {
-      const int k = (int)(((unsigned long long)__double_as_longlong(skip_abs) >> 52) & 0x7FF) - 1023 - eo;
-      sabs = skip_abs <= 0.0 ? 0.0f : k > 100 ? __int_as_float(0x7F800000) : k < -120 ? 0.0f : df_split(skip_abs, eo).x;
-    }
-    const float skf = (float)skip;
-    __syncthreads();
-    float2 held = make_float2(0.0f, 0.0f);  // warp 0: the pair's own coupling after its rotation
-    bool mine = false;
-    auto rotate = [&](int rho, float2 a, float2 base, int buf) {
-      int x, y;
-      rr_slot(W2, rho, lane, x, y);
-      const int pi = min(x, y), qi = max(x, y);
-      const float2 cp = sm.corr[pi], cq = sm.corr[qi];
-      const float app = fabsf(sm.d0[pi] + cp.x), aqq = fabsf(sm.d0[qi] + cq.x);
-      float rp, rq;
-      asm("sqrt.approx.f32 %0, %1;" : "=f"(rp) : "f"(app));
-      asm("sqrt.approx.f32 %0, %1;" : "=f"(rq) : "f"(aqq));
-      float4 r = make_float4(1.0f, 0.0f, 0.0f, 0.0f);
-      held = a;
-      if (fabsf(a.x) > skf * rp * rq && fabsf(a.x) > sabs) {
-        mine = true;
-        const float2 d = df_add(base, df_add(cq, df_neg(cp)));
-        float2 t, c, s;
-        df_angle(a, d, t, c, s);
-        const float2 ta = df_mul(t, a);
-        sm.corr[pi] = df_add(cp, df_neg(ta));
-        sm.corr[qi] = df_add(cq, ta);
-        if (x > y) s = df_neg(s);
-        r = make_float4(c.x, c.y, s.x, s.y);
-        held = make_float2(0.0f, 0.0f);
-      }
-      sm.rec[buf][lane] = r;
-    };
-    // a_qq - a_pp of the starting diagonal for pair `lane` of round rho
-    auto base_gap = [&](int rho) {
-      int x, y;
-      rr_slot(W2, rho, lane, x, y);
-      const int pi = min(x, y), qi = max(x, y);
-      return df_split(sm.A[qi][qi] - sm.A[pi][pi], eo);
-    };
-    auto at = [](int i, int j) { return max(i, j) * LDS + min(i, j); };
-    // where pair `lane` of the next round lies now: block (sa, sb) of this
-    // round's slots, index x or y of each (rr_slot's indices advance by one)
-    const int sa = lane < 2 ? 0 : lane == 15 ? 14 : lane - 1;
-    const int sb = lane == 0 ? 1 : lane == 1 ? 2 : lane == 15 ? 15 : lane + 1;
-    const bool ya = lane != 1, yb = lane == 15;
-    float2 base = make_float2(0.0f, 0.0f);
-    if (warp == 0 && lane < W2 / 2) {
-      int x, y;
-      rr_slot(W2, 0, lane, x, y);
-      rotate(0, sm.p.S[0][at(x, y)], base_gap(0), 0);
-      base = base_gap(1);
-    }
-    // the block of threads 32 .. 151: slots ba < bb
-    int ba = 0, bb = 0;
-    {
-      int rem = tid - 32;
-      if (rem >= 0 && rem < 120) {
-        while (rem >= 15 - ba) {
-          rem -= 15 - ba;
-          ++ba;
-        }
-        bb = ba + 1 + rem;
-      }
-    }
-    // entries of the block that are couplings of the next round (left to warp 0)
-    const bool skip00 = ba == 0 && bb == 2;
-    const bool skip10 = ba == 0 ? bb == 1 : bb == ba + 2;
-    const bool skip11 = ba == 14 && bb == 15;
-    __syncthreads();
-#pragma unroll 1
-    for (int rho = 0; rho < W2 - 1; ++rho) {
-      const int cur = rho & 1;
-      const float2* Sc = sm.p.S[cur];
-      float2* Sn = sm.p.S[cur ^ 1];
-      if (warp == 0) {
-        if (lane < W2 / 2) {
-          int x, y;
-          rr_slot(W2, rho, lane, x, y);
-          Sn[at(x, y)] = held;
-          if (rho + 1 < W2 - 1) {
-            int xa, yaa, xb, ybb;
-            rr_slot(W2, rho, sa, xa, yaa);
-            rr_slot(W2, rho, sb, xb, ybb);
-            const int i = ya ? yaa : xa, io = ya ? xa : yaa, j = yb ? ybb : xb, jo = yb ? xb : ybb;
-            const float4 ra = sm.rec[cur][sa], rb = sm.rec[cur][sb];
-            const float2 ca = make_float2(ra.x, ra.y), cb = make_float2(rb.x, rb.y);
-            float2 ga = make_float2(ra.z, ra.w), gb = make_float2(rb.z, rb.w);
-            if (!ya) ga = df_neg(ga);
-            if (!yb) gb = df_neg(gb);
-            const float2 t0 = df_rot(ca, Sc[at(i, j)], ga, Sc[at(io, j)]);
-            const float2 t1 = df_rot(ca, Sc[at(i, jo)], ga, Sc[at(io, jo)]);
-            rotate(rho + 1, df_rot(cb, t0, gb, t1), base, cur ^ 1);
-            if (rho + 2 < W2 - 1) base = base_gap(rho + 2);
-          }
-        }
-      } else if (warp < 5) {
-        if (bb > 0) {
-          int xa, yaa, xb, ybb;
-          rr_slot(W2, rho, ba, xa, yaa);
-          rr_slot(W2, rho, bb, xb, ybb);
-          const float4 ra = sm.rec[cur][ba], rb = sm.rec[cur][bb];
-          const float2 ca = make_float2(ra.x, ra.y), ga = make_float2(ra.z, ra.w), na = df_neg(ga);
-          const float2 cb = make_float2(rb.x, rb.y), gb = make_float2(rb.z, rb.w), nbg = df_neg(gb);
-          const int i00 = at(xa, xb), i01 = at(xa, ybb), i10 = at(yaa, xb), i11 = at(yaa, ybb);
-          const float2 v00 = Sc[i00], v01 = Sc[i01], v10 = Sc[i10], v11 = Sc[i11];
-          const float2 t00 = df_rot(ca, v00, na, v10), t10 = df_rot(ca, v10, ga, v00);
-          const float2 t01 = df_rot(ca, v01, na, v11), t11 = df_rot(ca, v11, ga, v01);
-          if (!skip00) Sn[i00] = df_rot(cb, t00, nbg, t01);
-          Sn[i01] = df_rot(cb, t01, gb, t00);
-          if (!skip10) Sn[i10] = df_rot(cb, t10, nbg, t11);
-          if (!skip11) Sn[i11] = df_rot(cb, t11, gb, t10);
-        }
-      } else {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int k = 4 * (warp - 5) + i;
-          int x, y;
-          rr_slot(W2, rho, k, x, y);
-          const float4 r = sm.rec[cur][k];
-          const float2 c = make_float2(r.x, r.y), g = make_float2(r.z, r.w);
-          const float2 ux = sm.p.U[x][lane], uy = sm.p.U[y][lane];
-          sm.p.U[x][lane] = df_rot(c, ux, df_neg(g), uy);
-          sm.p.U[y][lane] = df_rot(c, uy, g, ux);
+    for (int it = 0; it < NE; ++it) {
+      const int e = tid + it * SOLVE_THREADS, li = e % W2, lj = e / W2;
+      if (e >= W2 * W2) continue;
+      if (li > lj && li + lj != 31) sm.p.S[0][pos_at(li, lj)] = df_split(v0[it], eo);
+    }
+    for (int e = tid; e < (W2 - 1) * (W2 / 2); e += SOLVE_THREADS) {
+      int x, y;
+      rr_slot(W2, e / (W2 / 2), e % (W2 / 2), x, y);
+      sm.p.gap[e / (W2 / 2)][e % (W2 / 2)] = df_split(sm.A[y][y] - sm.A[x][x], eo);
+    }
+    __syncthreads();
+    if (tid == 0) sm.any = 0u;  // read by all above; set again by warp 0
+    if (warp == 0) {
+      // skip_abs 2^-eo rounded to FP32 (infinite when it is beyond every
+      // coupling), at least 2^-110: smaller couplings wait for a later sweep
+      float sabs;
+      {
+        const int k = (int)(((unsigned long long)__double_as_longlong(skip_abs) >> 52) & 0x7FF) - 1023 - eo;
+        sabs = skip_abs <= 0.0 ? 0.0f : k > 100 ? __int_as_float(0x7F800000) : k < -110 ? 0.0f : df_split(skip_abs, eo).x;
+        sabs = fmaxf(sabs, 0x1p-110f);
+      }
+      const float skf = (float)skip;
+      const int k = lane & 15;                // slot; lanes 16-31 repeat lanes 0-15
+      float2 held = make_float2(0.0f, 0.0f);  // the slot's own coupling after its rotation
+      float2 cx = held, cy = held;            // change of the slot's diagonal entries (scaled pairs)
+      float dx = df_split(sm.A[k][k], eo).x, dy = df_split(sm.A[31 - k][31 - k], eo).x;  // the entries themselves
+      bool mine = false;
+      // rotation of the slot in round rho from its coupling a, d = a_yy - a_xx and the skip test's bound
+      auto rotate = [&](int rho, float2 a, float2 d, float lim, int buf) {
+        const bool rot = fabsf(a.x) > lim;
+        const float tie = k == 0 || rho < k || rho > 30 - k ? 1.0f : -1.0f;  // x < y: '+'
+        float2 t, c, s;
+        df_angle(a, d, tie, t, c, s);
+        mine |= rot;
+        const float2 z = make_float2(0.0f, 0.0f);
+        held = rot ? z : a;
+        if (lane < W2 / 2) sm.rec[buf][k] = rot ? make_float4(c.x, c.y, s.x, s.y) : make_float4(1.0f, 0.0f, 0.0f, 0.0f);
+        const float2 ta = rot ? df_mul(t, a) : z;
+        cx = df_add(cx, df_neg(ta));
+        cy = df_add(cy, ta);
+        dx -= ta.x;
+        dy += ta.x;
+      };
+      // the skip test's bound max(skip sqrt(|a_xx a_yy|), skip_abs)
+      auto bound = [&]() { return fmaxf(skf * sqrt_ftz(fabsf(dx)) * sqrt_ftz(fabsf(dy)), sabs); };
+      // the next round's slot k lies at positions (i, j) now
+      const int i = pos_prev(k), j = pos_prev(31 - k), io = 31 - i, jo = 31 - j;
+      const int a00 = pos_at(i, j), a01 = pos_at(i, jo), a10 = pos_at(io, j), a11 = pos_at(io, jo);
+      const int own = pos_at(pos_next(k), pos_next(31 - k));
+      const bool iy = i > 15, jy = j > 15;
+      const int sa = iy ? io : i, sb = jy ? jo : j;
+      rotate(0, df_split(sm.A[k][31 - k], eo), sm.p.gap[0][k], bound(), 0);
+#pragma unroll 1
+      for (int rho = 0; rho < W2 - 1; ++rho) {
+        const int cur = rho & 1;
+        const float2* Sc = sm.p.S[cur];
+        // the diagonal entries of the next round's slot (two lanes on either side)
+        {
+          const float2 nx = make_float2(__shfl_down_sync(~0u, cx.x, 1, 16), __shfl_down_sync(~0u, cx.y, 1, 16));
+          const float2 py = make_float2(__shfl_up_sync(~0u, cy.x, 1, 16), __shfl_up_sync(~0u, cy.y, 1, 16));
+          const float2 x0 = make_float2(__shfl_sync(~0u, cx.x, 0, 16), __shfl_sync(~0u, cx.y, 0, 16));
+          const float ndx = __shfl_down_sync(~0u, dx, 1, 16), pdy = __shfl_up_sync(~0u, dy, 1, 16);
+          const float d0 = __shfl_sync(~0u, dx, 0, 16);
+          cx = k == 15 ? cy : nx;
+          dx = k == 15 ? dy : ndx;
+          cy = k == 0 ? cy : k == 1 ? x0 : py;
+          dy = k == 0 ? dy : k == 1 ? d0 : pdy;
+        }
+        const float2 d = df_add(sm.p.gap[min(rho + 1, W2 - 2)][k], df_add(cy, df_neg(cx)));
+        const float lim = bound();
+        const float2 h = held;
+        __syncwarp();
+        const float4 ra = sm.rec[cur][sa], rb = sm.rec[cur][sb];  // this warp's own writes
+        const float2 ca = make_float2(ra.x, ra.y), cb = make_float2(rb.x, rb.y);
+        const float2 ga = iy ? make_float2(ra.z, ra.w) : make_float2(-ra.z, -ra.w);
+        const float2 gb = jy ? make_float2(rb.z, rb.w) : make_float2(-rb.z, -rb.w);
+        solve_barrier();
+        if (rho + 1 < W2 - 1) {
+          const float2 t0 = df_rot(ca, Sc[a00], ga, Sc[a10]), t1 = df_rot(ca, Sc[a01], ga, Sc[a11]);
+          rotate(rho + 1, df_rot(cb, t0, gb, t1), d, lim, cur ^ 1);
+        }
+        if (lane < W2 / 2) sm.p.S[cur ^ 1][own] = h;
+      }
+      if (mine) sm.any = 1u;
+    } else if (warp < 4 || (warp > 4 && warp < 8) || warp == 9 || warp == 10) {
+      // one row of the 2 x 2 block of slots ba < bb: position i (its other one io)
+      const int w = warp < 4 ? warp - 1 : warp < 8 ? warp - 2 : warp - 3, side = lane & 1;
+      int ba = 0, rem = w * 16 + (lane >> 1);
+      const bool on = rem < 120;
+      while (on && rem >= 15 - ba) {
+        rem -= 15 - ba;
+        ++ba;
+      }
+      const int bb = on ? ba + 1 + rem : 1;
+      const int i = side ? 31 - ba : ba, io = 31 - i, jx = bb, jy = 31 - bb;
+      const int i0 = pos_at(i, jx), i1 = pos_at(i, jy), o0 = pos_at(io, jx), o1 = pos_at(io, jy);
+      const int w0 = pos_at(pos_next(i), pos_next(jx)), w1 = pos_at(pos_next(i), pos_next(jy));
+      // couplings of the next round are left to warp 0
+      const bool keep0 = on && pos_next(i) + pos_next(jx) != 31, keep1 = on && pos_next(i) + pos_next(jy) != 31;
+#pragma unroll 2
+      for (int rho = 0; rho < W2 - 1; ++rho) {
+        const int cur = rho & 1;
+        const float2* Sc = sm.p.S[cur];
+        float2* Sn = sm.p.S[cur ^ 1];
+        solve_barrier();
+        const float4 ra = sm.rec[cur][ba], rb = sm.rec[cur][bb];
+        const float2 v0 = Sc[i0], u0 = Sc[o0], v1 = Sc[i1], u1 = Sc[o1];
+        const float2 ca = make_float2(ra.x, ra.y), cb = make_float2(rb.x, rb.y), gb = make_float2(rb.z, rb.w);
+        const float2 ga = side ? make_float2(ra.z, ra.w) : make_float2(-ra.z, -ra.w);
+        const float2 t0 = df_rot(ca, v0, ga, u0), t1 = df_rot(ca, v1, ga, u1);
+        if (keep0) Sn[w0] = df_rot(cb, t0, df_neg(gb), t1);
+        if (keep1) Sn[w1] = df_rot(cb, t1, gb, t0);
+      }
+    } else if (warp != 8 && warp != 12 && warp != 16) {
+      // U_P in registers: eight lanes per row, lane e the columns at slots 2 e
+      // and 2 e + 1.  The columns move with the positions: x_k <- x_(k+1), y_k
+      // <- y_(k-1), x_15 <- y_15, y_1 <- x_0, and y_0 (index 31) stays.
+      const int e = lane & 7, w = warp == 4 ? 0 : warp == 11 ? 1 : warp < 16 ? warp - 11 : warp - 12;
+      const int row = w * 4 + (lane >> 3);
+      float xh[2], xl[2], yh[2], yl[2];
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        xh[t] = 2 * e + t == row ? 1.0f : 0.0f;
+        yh[t] = 31 - 2 * e - t == row ? 1.0f : 0.0f;
+        xl[t] = yl[t] = 0.0f;
+      }
+      // one round behind: its records are loaded while the others work, not
+      // in the burst of loads after the barrier
+      solve_barrier();
+      float4 r0 = sm.rec[0][2 * e], r1 = sm.rec[0][2 * e + 1];
+#pragma unroll 2
+      for (int rho = 0; rho < W2 - 1; ++rho) {
+        if (rho + 1 < W2 - 1) solve_barrier();
+        const RotC r = rot_coef(r0, r1);
+        const Df2 ux{pk(xh[0], xh[1]), pk(xl[0], xl[1])}, uy{pk(yh[0], yh[1]), pk(yl[0], yl[1])};
+        const Df2 nx = df2_rot<true>(r, ux, uy), ny = df2_rot<false>(r, uy, ux);
+        float x0h, x0l, y0h, y0l, y1h, y1l;
+        unpk(nx.h, x0h, xh[0]);  // the new x_0 is this round's x_1
+        unpk(nx.l, x0l, xl[0]);
+        unpk(ny.h, y0h, y1h);
+        unpk(ny.l, y0l, y1l);
+        const float nh = __shfl_down_sync(0xFFFFFFFFu, x0h, 1), nl = __shfl_down_sync(0xFFFFFFFFu, x0l, 1);
+        const float ph = __shfl_up_sync(0xFFFFFFFFu, y1h, 1), pl = __shfl_up_sync(0xFFFFFFFFu, y1l, 1);
+        xh[1] = e == 7 ? y1h : nh;
+        xl[1] = e == 7 ? y1l : nl;
+        yh[0] = e == 0 ? y0h : ph;
+        yl[0] = e == 0 ? y0l : pl;
+        yh[1] = e == 0 ? x0h : y0h;
+        yl[1] = e == 0 ? x0l : y0l;
+        if (rho + 1 < W2 - 1) {
+          r0 = sm.rec[(rho + 1) & 1][2 * e];
+          r1 = sm.rec[(rho + 1) & 1][2 * e + 1];
         }
       }
-      __syncthreads();
+      // after 31 rounds the positions are the indices again
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        sm.p.U[2 * e + t][row] = make_float2(xh[t], xl[t]);
+        sm.p.U[31 - 2 * e - t][row] = make_float2(yh[t], yl[t]);
+      }
     }
-    if (warp == 0 && mine) sm.any = 1u;
   } else {
+    __syncthreads();
+    if (tid == 0) sm.any = 0u;  // read by all above
     // the same sweep in FP64 instructions (c - 1 carried separately)
     for (int e = tid; e < W2 * W2; e += SOLVE_THREADS) sm.U64[e / W2][e % W2] = (e / W2 == e % W2) ? 1.0 : 0.0;
     __syncthreads();
@@ -565,32 +700,35 @@ __global__ void __launch_bounds__(SOLVE_THREADS) blk_solve(const double* __restr
     if (tid == 0) rotated[P] = 0;
     return;
   }
-  // U_P in fixed point, F = U 2^60 (|U| <= 1 up to rounding)
-  constexpr int NE = (W2 * W2 + SOLVE_THREADS - 1) / SOLVE_THREADS;
-  long long F[NE];
+  // U_P in fixed point, U = (u1 + u0 2^-30) 2^-30 with u0 in [-2^29, 2^29]
+  int u1[NE], u0[NE];
 #pragma unroll
-  for (int i = 0; i < NE; ++i) {
-    const int e = tid + i * SOLVE_THREADS;
-    F[i] = 0;
-    if (e < W2 * W2) {
-      const int row = e % W2, col = e / W2;
-      if (pairs) {
-        const float2 v = sm.p.U[col][row];
-        F[i] = __float2ll_rn(v.x * 0x1p60f) + __float2ll_rn(v.y * 0x1p60f);
-      } else {
-        F[i] = __double2ll_rn(sm.U64[col][row] * 0x1p60);
-      }
+  for (int it = 0; it < NE; ++it) {
+    const int e = tid + it * SOLVE_THREADS, row = e % W2, col = e / W2;
+    u1[it] = u0[it] = 0;
+    if (e >= W2 * W2) continue;
+    if (pairs) {  // each part on the grid 2^-30, its exact remainder on 2^-60
+      const float2 v = sm.p.U[col][row];
+      const float xh = v.x * 0x1p30f, xl = v.y * 0x1p30f;
+      const int ah = __float2int_rn(xh), al = __float2int_rn(xl);
+      const int b = __float2int_rn((xh - (float)ah) * 0x1p30f) + __float2int_rn((xl - (float)al) * 0x1p30f);
+      const int carry = (b + (1 << 29)) >> 30;  // |b| <= 2^30
+      u1[it] = ah + al + carry;
+      u0[it] = b - (carry << 30);
+    } else {
+      const long long F = __double2ll_rn(sm.U64[col][row] * 0x1p60);
+      const long long t = (F + (1LL << 29)) >> 30;
+      u1[it] = (int)t;
+      u0[it] = (int)(F - (t << 30));
     }
   }
   __syncthreads();
 #pragma unroll
-  for (int i = 0; i < NE; ++i) {
-    const int e = tid + i * SOLVE_THREADS;
+  for (int it = 0; it < NE; ++it) {
+    const int e = tid + it * SOLVE_THREADS;
     if (e < W2 * W2) {
-      const int row = e % W2, col = e / W2;
-      const long long u1 = (F[i] + (1LL << 29)) >> 30;
-      sm.f.u1[col][row] = (int)u1;
-      sm.f.u0[col][row] = (int)(F[i] - (u1 << 30));  // in [-2^29, 2^29)
+      sm.f.u1[e / W2][e % W2] = u1[it];
+      sm.f.u0[e / W2][e % W2] = u0[it];
     }
   }
   __syncthreads();
@@ -598,9 +736,10 @@ __global__ void __launch_bounds__(SOLVE_THREADS) blk_solve(const double* __restr
   // U_P carries the rounding of its 496 rotations; applied to all of A and V
   // every round, that departure from orthogonality would accumulate over the
   // sweeps, so each U_P is made orthogonal first.  E (symmetric: the 528
-  // entries i <= j, mirrored) from sums of integer products: u1 v1 exactly
-  // (at most 2^60 by Cauchy-Schwarz), the cross terms at weight 2^-30 (below
-  // 2^62.5), u0 v0 (below 2^-59 in all) left out.
+  // entries i <= j, mirrored) from sums of integer products on the grid 2^-60:
+  // sum u1 v1 modulo 2^32, which is enough because |E| < 2^-29 (the identity's
+  // 2^60 vanishes), and the cross terms at weight 2^-30 (below 2^62.5); u0 v0
+  // (below 2^-59 in all) is left out.
   for (int idx = tid; idx < 528; idx += SOLVE_THREADS) {
     int i = 0, rem = idx;
     while (rem >= W2 - i) {
@@ -608,30 +747,34 @@ __global__ void __launch_bounds__(SOLVE_THREADS) blk_solve(const double* __restr
       ++i;
     }
     const int j = i + rem;
-    long long g = (i == j) ? -(1LL << 60) : 0LL, x = 0;
+    unsigned g = 0u;
+    long long x = 0;
 #pragma unroll
     for (int k = 0; k < W2; k += 4) {
       const int4 a1 = *reinterpret_cast<const int4*>(&sm.f.u1[i][k]), b1 = *reinterpret_cast<const int4*>(&sm.f.u1[j][k]);
       const int4 a0 = *reinterpret_cast<const int4*>(&sm.f.u0[i][k]), b0 = *reinterpret_cast<const int4*>(&sm.f.u0[j][k]);
-      g += (long long)a1.x * b1.x + (long long)a1.y * b1.y + (long long)a1.z * b1.z + (long long)a1.w * b1.w;
+      g += (unsigned)a1.x * (unsigned)b1.x + (unsigned)a1.y * (unsigned)b1.y + (unsigned)a1.z * (unsigned)b1.z +
+           (unsigned)a1.w * (unsigned)b1.w;
       x += (long long)a1.x * b0.x + (long long)a1.y * b0.y + (long long)a1.z * b0.z + (long long)a1.w * b0.w;
       x += (long long)a0.x * b1.x + (long long)a0.y * b1.y + (long long)a0.z * b1.z + (long long)a0.w * b1.w;
     }
-    const float ev = fmaf((float)x, 0x1p-90f, (float)g * 0x1p-60f);
+    // x 2^-30 taken out of g's grid first, so the small difference is exact
+    const int gx = (int)(g + (unsigned)(x >> 30));
+    const float ev = fmaf((float)(int)(x & 0x3FFFFFFF), 0x1p-90f, (float)gx * 0x1p-60f);
     sm.f.Ef[i][j] = ev;
     sm.f.Ef[j][i] = ev;
   }
   __syncthreads();
   // U E / 2 in FP32: |E| is about 2^-43, so its error is below 2^-65.  Warp w
-  // takes columns w, w + 9, ..; lane = row.
+  // takes columns w and w + 20; lane = row.
   {
     float ur[W2];
 #pragma unroll
     for (int k = 0; k < W2; ++k) ur[k] = (float)sm.f.u1[k][lane];  // U(lane, k) 2^30
-    long long Fn[4];
+    long long Fn[2];
 #pragma unroll
-    for (int jj = 0; jj < 4; ++jj) {
-      const int j = warp + 9 * jj;
+    for (int jj = 0; jj < 2; ++jj) {
+      const int j = warp + 20 * jj;
       Fn[jj] = 0;
       if (j < W2) {
         float acc = 0.0f;
@@ -643,14 +786,14 @@ __global__ void __launch_bounds__(SOLVE_THREADS) blk_solve(const double* __restr
           acc = fmaf(ur[k + 2], ev.z, acc);
           acc = fmaf(ur[k + 3], ev.w, acc);
         }
-        Fn[jj] = ((long long)sm.f.u1[j][lane] << 30) + sm.f.u0[j][lane] - __float2ll_rn(acc * 0x1p29f);
+        Fn[jj] = ((long long)sm.f.u1[j][lane] << 30) + sm.f.u0[j][lane] - __float2int_rn(acc * 0x1p29f);
       }
     }
     __syncthreads();
     long long* Fs = reinterpret_cast<long long*>(&sm.f);  // [column][row], row stride LDS
 #pragma unroll
-    for (int jj = 0; jj < 4; ++jj)
-      if (warp + 9 * jj < W2) Fs[(warp + 9 * jj) * LDS + lane] = Fn[jj];
+    for (int jj = 0; jj < 2; ++jj)
+      if (warp + 20 * jj < W2) Fs[(warp + 20 * jj) * LDS + lane] = Fn[jj];
     __syncthreads();
   }
   // digits of U_P's columns: column c is "row" c of the right operand, over
@@ -1030,6 +1173,13 @@ cudaError_t rmul_attr() {
   if (e == cudaSuccess) done = true;
   return e;
 }
+int sm_count() {
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    (void)cudaGetLastError();
+  return sms;
+}
 }  // namespace
 
 // Round R, step 1: the subproblems of the block pairs, U_P into set R mod 2;
@@ -1039,8 +1189,8 @@ cudaError_t mpj_blocked_solve(const double* A, int lda, int n, int R, double ski
   const int N = (n + 2 * BS - 1) / (2 * BS) * (2 * BS);
   const int nb = N / BS;
   const USet u = uset(scratch, n, R & 1);
-  return mpj_launch_pdl(blk_solve, dim3(nb / 2), dim3(SOLVE_THREADS), 0, s, A, lda, n, nb, R, skip, skip_abs, u.sl,
-                        u.ex, u.rot, nrot);
+  return mpj_launch_pdl(nb / 2 <= sm_count() ? blk_solve<1> : blk_solve<2>, dim3(nb / 2), dim3(SOLVE_THREADS), 0, s, A,
+                        lda, n, nb, R, skip, skip_abs, u.sl, u.ex, u.rot, nrot);
 }
 
 // Round R, step 2: A <- U~^T A U~ through B (two right multiplications).
