@@ -45,8 +45,10 @@
  *                         the FP64 DMMA kernel instead of the tensor cores
  *                         (the exact bf16-slice products of mpj_dgemm_tc, the
  *                         default);
- *   MPJ_AUTOTUNE_CACHE=f  file that keeps the batched group-size choices;
- *   MPJ_BATCHED_GROUP=g   fix the batched group size (256, 512 or 1024).
+ *   MPJ_BATCHED_GROUP=g   batched solve with one thread group per matrix (256,
+ *                         512 or 1024 threads, anything else: autotuned)
+ *                         instead of round by round (read on each call);
+ *   MPJ_AUTOTUNE_CACHE=f  file that keeps the autotuned group-size choices.
  */
 #ifndef MPJACOBI_H
 #define MPJACOBI_H
@@ -165,24 +167,28 @@ int mpj_syev(int n, const double* A_dev, int lda, double* W_dev, double* Q_dev, 
 int mpj_syev_ex(int n, const double* A_dev, int lda, double* W_dev, double* Q_dev, int ldq, const mpj_opts* o,
                 mpj_info* info, void* work_dev, size_t work_bytes, void* stream);
 
-/* Batched solve of `batch` independent matrices (sizes 1 <= n_i <= 256) in one
- * persistent launch (not in the paper; each matrix runs Algorithm 9 in one
- * thread group).  n_host: host array of sizes.  A_dev, W_dev, Q_dev: device
- * arrays of `batch` device pointers (A read only, lda_i = n_i; Q_i is
- * n_i x n_i, ld n_i).  sweeps_host (may be NULL): receives the FP64 sweep count
- * per matrix.  tol <= 0 selects n_i 2^-53 ||A_i||_F per matrix.
- * The first call for a given (sizes, pointer arrays, tol) plans: it allocates
- * a workspace with cudaMalloc, orders the queue by decreasing n, picks the
- * thread-group size (256, 512 or 1024 threads per matrix) by timing each on
- * this batch unless the size histogram was tuned before (choices persist in
- * the file named by the environment variable MPJ_AUTOTUNE_CACHE, if set;
- * MPJ_BATCHED_GROUP=256|512|1024 fixes the size instead), and
- * captures [queue reset, kernel, result copies] in a CUDA graph.  Later calls
- * with the same sizes and pointer arrays only launch that graph on `stream`
- * (the pointed-to data may change); they may themselves be stream-captured,
- * the first one may not.  Up to 4 plans are kept (mpj_release_plans frees
- * them).  Synchronizes `stream`.  Returns MPJ_NOT_CONVERGED if any matrix hit
- * the sweep cap, MPJ_ENONFINITE if any input holds a NaN or an infinity. */
+/* Batched solve of `batch` independent matrices (sizes 1 <= n_i <= 256; not in
+ * the paper; Algorithm 9 per matrix).  n_host: host array of sizes.  A_dev,
+ * W_dev, Q_dev: device arrays of `batch` device pointers (A read only,
+ * lda_i = n_i; Q_i is n_i x n_i, ld n_i).  sweeps_host (may be NULL): receives
+ * the FP64 sweep count per matrix.  tol <= 0 selects n_i 2^-53 ||A_i||_F per
+ * matrix.
+ * All matrices go through the rounds of a stage together, one launch per step
+ * of a round; those that have converged drop out.  The first call for a list
+ * of sizes plans: it orders the matrices by decreasing size and allocates a
+ * workspace with cudaMalloc (at most about 6 GB: larger batches run in
+ * several parts).  Later calls with the same sizes reuse it, whatever the
+ * pointers.  Up to 4 plans are kept (mpj_release_plans frees them); calls
+ * from several threads run one after the other.  Synchronizes `stream` (once
+ * per sweep, to read how many matrices still need one, and at the end), so it
+ * cannot be stream-captured.
+ * With MPJ_BATCHED_GROUP set, one thread group solves each matrix in one
+ * persistent launch instead; its plan also keeps the pointer arrays, the
+ * group size (fixed, or picked by timing 256, 512 and 1024 threads on this
+ * batch unless the size histogram was tuned before, see MPJ_AUTOTUNE_CACHE)
+ * and a CUDA graph of the launch.
+ * Returns MPJ_NOT_CONVERGED if any matrix hit the sweep cap, MPJ_ENONFINITE
+ * if any input holds a NaN or an infinity (the other matrices are solved). */
 int mpj_syev_batched(int batch, const int* n_host, const double* const* A_dev, double* const* W_dev,
                      double* const* Q_dev, double tol, int* sweeps_host, void* stream);
 
@@ -190,7 +196,8 @@ int mpj_syev_batched(int batch, const int* n_host, const double* const* A_dev, d
 void mpj_release_plans(void);
 
 /* The autotuned thread-group size recorded for this batch's size histogram
- * (256, 512 or 1024), or 0 if none has been tuned yet. */
+ * (256, 512 or 1024), or 0 if none has been tuned (none is unless
+ * MPJ_BATCHED_GROUP asks for it). */
 int mpj_batched_group_size(int batch, const int* n_host);
 
 /* Eigen-adjoint (not in the paper): with W, Q from a solve (Q n x n, ld ldq),

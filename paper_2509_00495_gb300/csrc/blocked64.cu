@@ -43,6 +43,7 @@
 #include <stdint.h>
 #include <stdio.h>
 
+#include "batch.cuh"
 #include "common.cuh"
 #include "jacobi64.cuh"
 
@@ -411,19 +412,52 @@ MPJ_DEV int pos_at(int i, int j) {
   return (2 * ea + eb) * SSTR + (a * (31 - a)) / 2 + (b - a - 1);
 }
 
+// One subproblem: pair P of round R of a matrix, and where its digits,
+// exponents and flag go.
+struct Sub64 {
+  const double* A;
+  int lda, n, nb, P;
+  double skip_abs;
+  __nv_bfloat16* sl;
+  int *ex, *rot;
+  unsigned* nrot;
+};
+struct OneSub64 {  // the block pairs of one matrix
+  const double* A;
+  int lda, n, nb;
+  double skip_abs;
+  __nv_bfloat16* sl;
+  int *ex, *rot;
+  unsigned* nrot;
+  MPJ_DEV bool get(int bid, Sub64& v) const {
+    v = Sub64{A, lda, n, nb, bid, skip_abs, sl + (size_t)bid * NSL * (USL_BYTES / 2), ex + bid * W2, rot + bid, nrot};
+    return true;
+  }
+};
+struct BatchSub64 {  // the block pairs of a batch
+  BatchShape b;
+  int lo;
+  const double* A;
+  const double* skip_abs;
+  __nv_bfloat16* sl;
+  int *ex, *rot;
+  MPJ_DEV bool get(int bid, Sub64& v) const {
+    BatchTask t;
+    if (!batch_find(b, lo, bid, [](int np) { return np; }, t)) return false;
+    const int o = t.pair0 + t.local;
+    v = Sub64{A + t.el, t.N, t.n, t.N / BS, t.local, skip_abs[t.place], sl + (size_t)o * NSL * (USL_BYTES / 2),
+              ex + o * W2, rot + o, nullptr};
+    return true;
+  }
+};
 // CTAS: resident CTAs per SM the registers are limited for.  One (78 registers)
 // has the shorter latency and is taken when every subproblem of a round finds
 // its own SM; beyond that two (48 registers) have the higher rate: 16 against 21
 // us per subproblem and SM.
-template <int CTAS>
-__global__ void __launch_bounds__(SOLVE_THREADS, CTAS) blk_solve(const double* __restrict__ A, int lda, int n, int nb, int R,
-                                                 double skip, double skip_abs, __nv_bfloat16* __restrict__ Usl,
-                                                 int* __restrict__ Uexp, int* __restrict__ rotated,
-                                                 unsigned* __restrict__ nrot) {
+template <int CTAS, class Src>
+__global__ void __launch_bounds__(SOLVE_THREADS, CTAS) blk_solve(Src src, int R, double skip) {
   __shared__ __align__(16) SolveSmem sm;
-  const int P = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  int I, J;
-  block_pair(nb, R, P, I, J);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
     sm.emax_off = 0u;
     sm.emin_off = 0xFFFFu;
@@ -432,6 +466,13 @@ __global__ void __launch_bounds__(SOLVE_THREADS, CTAS) blk_solve(const double* _
   }
   __syncthreads();
   pdl_wait();
+  Sub64 sub;
+  if (!src.get(blockIdx.x, sub)) return;
+  const double* __restrict__ A = sub.A;
+  const int lda = sub.lda, n = sub.n;
+  const double skip_abs = sub.skip_abs;
+  int I, J;
+  block_pair(sub.nb, R, sub.P, I, J);
   constexpr int NE = (W2 * W2 + SOLVE_THREADS - 1) / SOLVE_THREADS;
   double v0[NE];
   {
@@ -469,7 +510,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS, CTAS) blk_solve(const double* _
   }
   __syncthreads();
   if (!sm.any) {  // every coupling is zero or at most skip_abs: nothing rotates
-    if (tid == 0) rotated[P] = 0;
+    if (tid == 0) *sub.rot = 0;
     return;
   }
   const int emax_off = (int)sm.emax_off, emin_off = (int)sm.emin_off;
@@ -697,7 +738,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS, CTAS) blk_solve(const double* _
   }
   __syncthreads();
   if (!sm.any) {
-    if (tid == 0) rotated[P] = 0;
+    if (tid == 0) *sub.rot = 0;
     return;
   }
   // U_P in fixed point, U = (u1 + u0 2^-30) 2^-30 with u0 in [-2^29, 2^29]
@@ -798,7 +839,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS, CTAS) blk_solve(const double* _
   }
   // digits of U_P's columns: column c is "row" c of the right operand, over
   // k = row of U_P; eight threads per column, four values each
-  __nv_bfloat16* dst = Usl + (size_t)P * NSL * (USL_BYTES / 2);
+  __nv_bfloat16* dst = sub.sl;
   if (tid < 8 * W2) {
     const long long* Fs = reinterpret_cast<const long long*>(&sm.f);
     const int c = tid >> 3, k0 = (tid & 7) * 4;
@@ -812,7 +853,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS, CTAS) blk_solve(const double* _
 #pragma unroll
     for (int o = 1; o < 8; o <<= 1) top |= __shfl_xor_sync(0xffffffffu, top, o);
     const int bits = 64 - __clzll((long long)top);  // max|F| < 2^bits
-    if ((tid & 7) == 0) Uexp[P * W2 + c] = bits - 60;
+    if ((tid & 7) == 0) sub.ex[c] = bits - 60;
     const int sh = bits - 56;  // Y = |F| 2^-sh rounded
     uint32_t d[4][NSL];
 #pragma unroll
@@ -830,8 +871,8 @@ __global__ void __launch_bounds__(SOLVE_THREADS, CTAS) blk_solve(const double* _
     }
   }
   if (tid == 0) {
-    rotated[P] = 1;
-    if (nrot) atomicAdd(nrot, 1u);
+    *sub.rot = 1;
+    if (sub.nrot) atomicAdd(sub.nrot, 1u);
   }
 }
 
@@ -947,16 +988,13 @@ MPJ_DEV bool tile_needed(int tri, int a, int Q) {
   return tri == TRI_ALL || (tri == TRI_FIRST ? a <= Q : a >= Q);
 }
 
-__global__ void __launch_bounds__(RM_THREADS, 2)
-    blk_rmul(const double* X, int ldx, int xmode, double* Y, int ldy, int n, int nb, int R,
-             const __nv_bfloat16* __restrict__ Usl, const int* __restrict__ Uexp, const int* __restrict__ rotated,
-             unsigned* __restrict__ flags, int tri) {
+MPJ_DEV void blk_rmul_tile(const double* X, int ldx, int xmode, double* Y, int ldy, int n, int nb, int R,
+                           const __nv_bfloat16* __restrict__ Usl, const int* __restrict__ Uexp,
+                           const int* __restrict__ rotated, unsigned* __restrict__ flags, int tri, int gx, int Q) {
   extern __shared__ __align__(1024) unsigned char dsm_raw[];
   RmulSmem& sm = *reinterpret_cast<RmulSmem*>(dsm_raw + ((1024 - (smem_u32(dsm_raw) & 1023)) & 1023));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int Q = blockIdx.y, gx = blockIdx.x;
   const int a0 = 4 * gx, a1 = min(4 * gx + 3, nb / 2 - 1);
-  pdl_wait();
   if (tri == TRI_FIRST && a0 > Q) return;
   if (tri == TRI_SECOND && a1 < Q) return;
   int I, J;
@@ -1128,6 +1166,34 @@ __global__ void __launch_bounds__(RM_THREADS, 2)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
 }
 
+__global__ void __launch_bounds__(RM_THREADS, 2)
+    blk_rmul(const double* X, int ldx, int xmode, double* Y, int ldy, int n, int nb, int R,
+             const __nv_bfloat16* __restrict__ Usl, const int* __restrict__ Uexp, const int* __restrict__ rotated,
+             unsigned* __restrict__ flags, int tri) {
+  pdl_wait();
+  blk_rmul_tile(X, ldx, xmode, Y, ldy, n, nb, R, Usl, Uexp, rotated, flags, tri, blockIdx.x, blockIdx.y);
+}
+
+// A batch: step 0, the tiles of B = A U~ and then of V <- V U~ per matrix;
+// step 1, those of A = B^T U~.
+__global__ void __launch_bounds__(RM_THREADS, 2)
+    blk_rmul_batch(BatchShape b, int lo, int R, int step, double* A, double* V, double* B,
+                   const __nv_bfloat16* __restrict__ sl, const int* __restrict__ ex, const int* __restrict__ rot,
+                   unsigned* __restrict__ flags) {
+  pdl_wait();
+  BatchTask t;
+  const int kinds = step == 0 ? 2 : 1;
+  if (!batch_find(b, lo, blockIdx.x, [kinds](int np) { return kinds * ((np + 3) / 4) * np; }, t)) return;
+  const int np = t.N / W2, per = ((np + 3) / 4) * np;
+  const bool v = t.local >= per;
+  const int l = v ? t.local - per : t.local;
+  const double* X = step == 1 ? B : v ? V : A;
+  double* Y = step == 1 ? A : v ? V : B;
+  blk_rmul_tile(X + t.el, t.N, step == 1 ? XMODE_ROWS : XMODE_COLS, Y + t.el, t.N, t.n, t.N / BS, R,
+                sl + (size_t)t.pair0 * NSL * (USL_BYTES / 2), ex + t.pair0 * W2, rot + t.pair0, flags,
+                step == 1 ? TRI_SECOND : v ? TRI_ALL : TRI_FIRST, l / np, l % np);
+}
+
 inline size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 }  // namespace
@@ -1170,6 +1236,8 @@ cudaError_t rmul_attr() {
   static bool done = false;
   if (done) return cudaSuccess;
   cudaError_t e = cudaFuncSetAttribute(blk_rmul, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rmul_smem());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(blk_rmul_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rmul_smem());
   if (e == cudaSuccess) done = true;
   return e;
 }
@@ -1189,8 +1257,8 @@ cudaError_t mpj_blocked_solve(const double* A, int lda, int n, int R, double ski
   const int N = (n + 2 * BS - 1) / (2 * BS) * (2 * BS);
   const int nb = N / BS;
   const USet u = uset(scratch, n, R & 1);
-  return mpj_launch_pdl(nb / 2 <= sm_count() ? blk_solve<1> : blk_solve<2>, dim3(nb / 2), dim3(SOLVE_THREADS), 0, s, A,
-                        lda, n, nb, R, skip, skip_abs, u.sl, u.ex, u.rot, nrot);
+  return mpj_launch_pdl(nb / 2 <= sm_count() ? blk_solve<1, OneSub64> : blk_solve<2, OneSub64>, dim3(nb / 2),
+                        dim3(SOLVE_THREADS), 0, s, OneSub64{A, lda, n, nb, skip_abs, u.sl, u.ex, u.rot, nrot}, R, skip);
 }
 
 // Round R, step 2: A <- U~^T A U~ through B (two right multiplications).
@@ -1221,6 +1289,28 @@ cudaError_t mpj_blocked_update_V(double* V, int ldv, int n, int R, void* scratch
   return mpj_launch_pdl(blk_rmul, grid, dim3(RM_THREADS), rmul_smem(), s, (const double*)V, ldv, (int)XMODE_COLS, V,
                         ldv, n, nb, R, (const __nv_bfloat16*)u.sl, (const int*)u.ex, (const int*)u.rot, flags,
                         (int)TRI_ALL);
+}
+
+size_t mpj_batch_digit_bytes(int pairs) { return uset_bytes(pairs); }
+
+cudaError_t mpj_batch_sweep64_round(const BatchShape& b, int R, double* A, double* V, double* B, const double* skip_abs,
+                                    void* digits, int pairs, unsigned* flags, cudaStream_t s) {
+  const int lo = batch_lowest_class(R);
+  const long long subs = batch_blocks(b, lo, [](int np) { return np; });
+  if (subs == 0) return cudaSuccess;
+  cudaError_t e = rmul_attr();
+  if (e != cudaSuccess) return e;
+  __nv_bfloat16* sl = (__nv_bfloat16*)digits;
+  int* ex = (int*)((char*)digits + al256((size_t)pairs * NSL * USL_BYTES));
+  int* rot = (int*)((char*)ex + al256((size_t)pairs * W2 * sizeof(int)));
+  const BatchSub64 src{b, lo, A, skip_abs, sl, ex, rot};
+  e = mpj_launch_pdl(subs <= sm_count() ? blk_solve<1, BatchSub64> : blk_solve<2, BatchSub64>, dim3((unsigned)subs),
+                     dim3(SOLVE_THREADS), 0, s, src, R, 0x1p-53);
+  const long long tiles = batch_blocks(b, lo, [](int np) { return ((np + 3) / 4) * np; });
+  for (int step = 0; step < 2 && e == cudaSuccess; ++step)
+    e = mpj_launch_pdl(blk_rmul_batch, dim3((unsigned)(step == 0 ? 2 * tiles : tiles)), dim3(RM_THREADS), rmul_smem(),
+                       s, b, lo, R, step, A, V, B, (const __nv_bfloat16*)sl, (const int*)ex, (const int*)rot, flags);
+  return e;
 }
 
 int mpj_blocked_rounds_per_sweep(int n) {

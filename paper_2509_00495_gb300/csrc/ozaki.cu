@@ -50,6 +50,7 @@
 #include <stdint.h>
 #include <stdio.h>
 
+#include "batch.cuh"
 #include "common.cuh"
 #include <stdlib.h>
 
@@ -301,25 +302,17 @@ struct __align__(1024) OzSmem {
   int abort_flag;
 };
 
-__global__ void __maxnreg__(168)
-    oz_gemm_kernel(const __nv_bfloat16* __restrict__ SA, const int* __restrict__ ea, int Rpa,
-                   const __nv_bfloat16* __restrict__ SB, const int* __restrict__ eb, int Rpb, int Kp, int sub0,
-                   int nsub, int m, int n, double alpha, double beta, const double* Cin, int ldcin, double* C,
-                   int ldc, unsigned* gflags, int lower) {
+// Output tile (mt, nt): C = alpha op(A) op(B) + beta Cin + dg I over k steps
+// sub0 .. sub0 + nsub - 1.  BATCH: with dg, and sym: entries on and below the
+// diagonal, each also written to its mirror.
+template <bool BATCH>
+MPJ_DEV void oz_tile(const __nv_bfloat16* __restrict__ SA, const int* __restrict__ ea, int Rpa,
+                     const __nv_bfloat16* __restrict__ SB, const int* __restrict__ eb, int Rpb, int Kp, int sub0,
+                     int nsub, int m, int n, int mt, int nt, double alpha, double beta, const double* Cin, int ldcin,
+                     double dg, double* C, int ldc, bool sym, unsigned* gflags) {
   extern __shared__ __align__(1024) unsigned char dsm_raw[];
   OzSmem& sm = *reinterpret_cast<OzSmem*>(dsm_raw + ((1024 - (smem_u32(dsm_raw) & 1023)) & 1023));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // tile order: groups of OZ_GROUP_M row tiles share the B tiles in L2
-  const int ntm = (m + OZ_TM - 1) / OZ_TM, ntn = (n + OZ_TN - 1) / OZ_TN;
-  const int id = blockIdx.x;
-  const int group = id / (OZ_GROUP_M * ntn);
-  const int first_m = group * OZ_GROUP_M;
-  const int gsz = min(ntm - first_m, OZ_GROUP_M);
-  const int local = id % (OZ_GROUP_M * ntn);
-  const int mt = first_m + local % gsz, nt = local / gsz;
-  // lower: only tiles that meet the lower triangle (row >= column) are formed
-  if (lower && mt * OZ_TM + OZ_TM - 1 < nt * OZ_TN) return;
-
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sm.tmem)),
                  "r"(OZ_TMEM_COLS)
@@ -410,7 +403,7 @@ __global__ void __maxnreg__(168)
     // ---------------- epilogue: warps 0-7
     const int quad = warp & 3, half = warp >> 2;
     const int row = mt * OZ_TM + quad * 32 + lane;
-    const int nchunks = nsub / (OZ_KC / OZ_KS);
+    const int nchunks = (nsub + OZ_KC / OZ_KS - 1) / (OZ_KC / OZ_KS);
     long long hi[32], lo[32];
 #pragma unroll
     for (int c = 0; c < 32; ++c) {
@@ -451,11 +444,13 @@ __global__ void __maxnreg__(168)
       for (int c = 0; c < 32; ++c) {
         const int cl = half * 32 + c;
         const int col = nt * OZ_TN + cl;
-        if (col < n) {
+        if (col < n && (!BATCH || !sym || row >= col)) {
           const double v = fma((double)hi[c], 0x1p-35, (double)lo[c] * 0x1p-63);
           double out = alpha * ldexp(v, er + sm.colexp[cl]);
           if (beta != 0.0) out = fma(beta, Cin[(long long)col * ldcin + row], out);
+          if (BATCH && dg != 0.0 && row == col) out += dg;
           C[(long long)col * ldc + row] = out;
+          if (BATCH && sym && row > col) C[(long long)row * ldc + col] = out;
         }
       }
     }
@@ -465,6 +460,89 @@ __global__ void __maxnreg__(168)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(OZ_TMEM_COLS) : "memory");
+}
+
+__global__ void __maxnreg__(168)
+    oz_gemm_kernel(const __nv_bfloat16* __restrict__ SA, const int* __restrict__ ea, int Rpa,
+                   const __nv_bfloat16* __restrict__ SB, const int* __restrict__ eb, int Rpb, int Kp, int sub0,
+                   int nsub, int m, int n, double alpha, double beta, const double* Cin, int ldcin, double* C,
+                   int ldc, unsigned* gflags, int lower) {
+  // tile order: groups of OZ_GROUP_M row tiles share the B tiles in L2
+  const int ntm = (m + OZ_TM - 1) / OZ_TM, ntn = (n + OZ_TN - 1) / OZ_TN;
+  const int id = blockIdx.x;
+  const int group = id / (OZ_GROUP_M * ntn);
+  const int first_m = group * OZ_GROUP_M;
+  const int gsz = min(ntm - first_m, OZ_GROUP_M);
+  const int local = id % (OZ_GROUP_M * ntn);
+  const int mt = first_m + local % gsz, nt = local / gsz;
+  // lower: only tiles that meet the lower triangle (row >= column) are formed
+  if (lower && mt * OZ_TM + OZ_TM - 1 < nt * OZ_TN) return;
+  oz_tile<false>(SA, ea, Rpa, SB, eb, Rpb, Kp, sub0, nsub, m, n, mt, nt, alpha, beta, Cin, ldcin, 0.0, C, ldc, false, gflags);
+}
+
+// ---- a batch of matrices with n <= 256 --------------------------------------
+MPJ_DEV int batch_oz_tiles(int np) { return ((32 * np + OZ_TM - 1) / OZ_TM) * ((32 * np + OZ_TN - 1) / OZ_TN); }
+__global__ void __maxnreg__(168)
+    oz_gemm_batch(BatchShape b, BatchOperand oa, BatchOperand ob, double alpha, double beta, const double* Cin,
+                  double dg, double* C, int sym, unsigned* gflags) {
+  BatchTask t;
+  if (!batch_find(b, 0, blockIdx.x, batch_oz_tiles, t)) return;
+  const int N = t.N, ntm = (N + OZ_TM - 1) / OZ_TM, mt = t.local % ntm, nt = t.local / ntm, Rp = batch_rp(N);
+  if (sym && mt * OZ_TM + OZ_TM - 1 < nt * OZ_TN) return;
+  oz_tile<true>(oa.sl + t.oz, oa.ex + t.place * BATCH_NMAX, Rp, ob.sl + t.oz, ob.ex + t.place * BATCH_NMAX, Rp, N, 0,
+          N / OZ_KS, N, N, mt, nt, alpha, beta, beta != 0.0 ? Cin + t.el : nullptr, N, dg, C + t.el, N, sym != 0,
+          gflags);
+}
+
+// The slices of 32 operand rows of one matrix: row maximum and digits in one
+// pass, a warp per row, lane l the values k = 8 l .. 8 l + 7.  Rows that are
+// strided in memory go through shared memory (32 consecutive rows per read).
+constexpr int OZ_PREP_THREADS = 256;
+constexpr size_t OZ_PREP_SMEM = (size_t)BATCH_NMAX * 33 * sizeof(double);
+__global__ void __launch_bounds__(OZ_PREP_THREADS) oz_prepare_batch(BatchShape b, const double* __restrict__ X,
+                                                                    const double* const* __restrict__ ptr,
+                                                                    const int* __restrict__ order, int byrow,
+                                                                    BatchOperand op) {
+  extern __shared__ __align__(16) double tile[];  // [k][row], row stride 33
+  BatchTask t;
+  if (!batch_find(b, 0, blockIdx.x, [](int np) { return np; }, t)) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, N = t.N, r0 = 32 * t.local;
+  const double* src = ptr ? ptr[order[t.place]] : X + t.el;
+  const int ld = ptr ? t.n : N, lim = ptr ? t.n : N;
+  if (byrow) {
+    for (int k = warp; k < N; k += OZ_PREP_THREADS / 32)
+      tile[k * 33 + lane] = (k < lim && r0 + lane < lim) ? src[(size_t)k * ld + r0 + lane] : 0.0;
+    __syncthreads();
+  }
+  const int Rp = batch_rp(N), k0 = 8 * lane;
+  for (int rl = warp; rl < 32; rl += OZ_PREP_THREADS / 32) {
+    const int r = r0 + rl;
+    double x[8];
+    unsigned long long m = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      x[j] = 0.0;
+      if (k0 < N) x[j] = byrow ? tile[(k0 + j) * 33 + rl] : (k0 + j < lim && r < lim) ? src[(size_t)r * ld + k0 + j] : 0.0;
+      m = max(m, oz_absbits(x[j]));
+    }
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    const int e = oz_exp_of(m);
+    if (lane == 0) op.ex[t.place * BATCH_NMAX + r] = e;
+    if (k0 >= N) continue;
+    uint32_t d[8][OZ_S];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) oz_digits(x[j], e, d[j]);
+    const long long off = t.oz + (long long)((k0 / OZ_KS) * (Rp / 64) + r / 64) * OZ_TILE64 + (kmaj16(r & 63, k0 & 31) >> 1);
+#pragma unroll
+    for (int s = 0; s < OZ_S; ++s) {
+      uint4 q;
+      q.x = oz_pack2(d[0][s], d[1][s]);
+      q.y = oz_pack2(d[2][s], d[3][s]);
+      q.z = oz_pack2(d[4][s], d[5][s]);
+      q.w = oz_pack2(d[6][s], d[7][s]);
+      *reinterpret_cast<uint4*>(op.sl + off + (long long)s * Rp * N) = q;
+    }
+  }
 }
 
 inline size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -557,6 +635,31 @@ cudaError_t mpj_oz_gemm(const OzOperand& a, const OzOperand& b, int m, int n, do
     }
   }
   return cudaSuccess;
+}
+
+cudaError_t mpj_batch_oz_prepare(const BatchShape& b, const double* X, const double* const* ptr, const int* order,
+                                 bool byrow, const BatchOperand& op, cudaStream_t s) {
+  const long long blocks = batch_blocks(b, 0, [](int np) { return np; });
+  if (blocks == 0) return cudaSuccess;
+  cudaError_t e = cudaFuncSetAttribute(oz_prepare_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_PREP_SMEM);
+  if (e != cudaSuccess) return e;
+  oz_prepare_batch<<<(unsigned)blocks, OZ_PREP_THREADS, byrow ? OZ_PREP_SMEM : 0, s>>>(b, X, ptr, order, byrow ? 1 : 0, op);
+  mpj_count_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t mpj_batch_oz_gemm(const BatchShape& b, const BatchOperand& oa, const BatchOperand& ob, double alpha,
+                              double beta, const double* Cin, double dg, double* C, bool sym, unsigned* flags,
+                              cudaStream_t s) {
+  const long long blocks =
+      batch_blocks(b, 0, [](int np) { return ((32 * np + OZ_TM - 1) / OZ_TM) * ((32 * np + OZ_TN - 1) / OZ_TN); });
+  if (blocks == 0) return cudaSuccess;
+  const size_t smem = sizeof(OzSmem) + 1024;
+  cudaError_t e = cudaFuncSetAttribute(oz_gemm_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  oz_gemm_batch<<<(unsigned)blocks, OZ_THREADS, smem, s>>>(b, oa, ob, alpha, beta, Cin, dg, C, sym ? 1 : 0, flags);
+  mpj_count_launch();
+  return cudaGetLastError();
 }
 
 extern "C" int mpj_dgemm_tc(char transa, char transb, int m, int n, int k, double alpha, const double* A, int lda,

@@ -25,6 +25,7 @@
 #include <cuda_fp16.h>
 #include <stdlib.h>
 
+#include "batch.cuh"
 #include "common.cuh"
 #include "stage1.cuh"
 #include "tc32.cuh"
@@ -139,27 +140,58 @@ MPJ_DEV int del0(int v, int h) { return ((v >> (h + 1)) << h) | (v & ((1 << h) -
 // divisions 23.8 us per launch; two index sets per thread and four-task warps
 // 18.4 us; this form 12.3 us.  The sweeps to reach
 // the stopping test are the same or one fewer (n = 96 .. 512, three spectra).
+// One subproblem: pair `slot` of round R of a matrix with nb blocks, and where
+// its S, U and T go.
+struct Sub32 {
+  const float* A;
+  int N, nb, slot;
+  float *S, *U;
+  unsigned* M;
+};
+struct OneSub32 {  // the block pairs of one matrix
+  const float* A;
+  int N, nb;
+  float *S, *U;
+  unsigned* M;
+  MPJ_DEV bool get(int bid, Sub32& v) const {
+    v = Sub32{A, N, nb, bid, S + (size_t)bid * W2 * W2, U + (size_t)bid * W2 * W2, M ? M + bid : nullptr};
+    return true;
+  }
+};
+struct BatchSub32 {  // the block pairs of a batch
+  BatchShape b;
+  int lo;
+  const float* A;
+  float *S, *U;
+  MPJ_DEV bool get(int bid, Sub32& v) const {
+    BatchTask t;
+    if (!batch_find(b, lo, bid, [](int np) { return np; }, t)) return false;
+    const size_t o = (size_t)(t.pair0 + t.local) * W2 * W2;
+    v = Sub32{A + t.el, t.N, t.N / BS, t.local, S + o, U + o, nullptr};
+    return true;
+  }
+};
 constexpr int S32_THREADS = 544;
 constexpr int SLD = 40;  // row stride of the packed S (8 more than 32: rows of d, d + 1, .. start 8 banks apart)
 // The CTA's barrier from the three roles' own code paths.
 MPJ_DEV void s32_barrier() { asm volatile("bar.sync 0, %0;\n" ::"n"(S32_THREADS) : "memory"); }
 
-template <bool HQ>
-__global__ void __launch_bounds__(S32_THREADS, 1) solve32(const float* __restrict__ A32, int N, int nb, int R,
-                                               float* __restrict__ Sbuf, float* __restrict__ Ubuf, bool urow,
-                                               unsigned* __restrict__ Mbuf) {
+template <bool HQ, class Src>
+__global__ void __launch_bounds__(S32_THREADS, 1) solve32(Src src, int R, bool urow) {
   __shared__ float S[2][W2 * SLD];
   __shared__ float U[W2][LD];  // U[column][row]
   __shared__ float dg[W2];     // the diagonal (warp 0 only)
   __shared__ Rot32 rec[2][W2 / 2];
-  const int slot = blockIdx.x;
-  int I, J;
-  block_pair(nb, R, slot, I, J);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   pdl_wait();
+  Sub32 sub;
+  if (!src.get(blockIdx.x, sub)) return;
+  int I, J;
+  block_pair(sub.nb, R, sub.slot, I, J);
+  unsigned* const Mbuf = sub.M;
   for (int e = tid; e < W2 * W2; e += S32_THREADS) {
     const int li = e % W2, lj = e / W2;
-    const float v = A32[(size_t)gidx(I, J, lj) * N + gidx(I, J, li)];
+    const float v = sub.A[(size_t)gidx(I, J, lj) * sub.N + gidx(I, J, li)];
     if (li == lj)
       dg[li] = v;
     else if (li < lj)
@@ -222,7 +254,7 @@ __global__ void __launch_bounds__(S32_THREADS, 1) solve32(const float* __restric
         p_cur = p;
       }
     }
-    if (lane == 0 && Mbuf) Mbuf[slot] = tmask;
+    if (lane == 0 && Mbuf) *Mbuf = tmask;
   } else if (warp < 9) {
     // half a block: pairs with 4-bit labels xl and yl = xl ^ dl, xl's bit at
     // dl's highest bit zero (15 x 8 unordered label pairs), and the row of
@@ -274,8 +306,7 @@ __global__ void __launch_bounds__(S32_THREADS, 1) solve32(const float* __restric
     }
   }
   s32_barrier();
-  float* So = Sbuf + (size_t)slot * W2 * W2;
-  float* Uo = Ubuf + (size_t)slot * W2 * W2;
+  float *So = sub.S, *Uo = sub.U;
   for (int e = tid; e < W2 * W2; e += S32_THREADS) {
     const int li = e % W2, lj = e / W2;
     So[e] = li == lj ? dg[li] : S[1][(li ^ lj) * SLD + min(li, lj)];
@@ -399,17 +430,22 @@ MPJ_DEV void load_u(const float* __restrict__ Ubuf, int P, float (*Us)[ULD], int
 // 32 w + 4 g .. +3 and columns 8 h .. +7: per k one float4 of X (8 distinct
 // in a warp: one shared-memory wavefront) and two float4 of U_Q (4 distinct:
 // one wavefront each) feed 32 FMAs.
-template <int TRI, bool MASKED>
-__global__ void __launch_bounds__(RT) rmul32(const float* X, float* Y, int N, int nb, int R,
-                                             const float* __restrict__ Sbuf, const float* __restrict__ Ubuf, bool hq,
-                                             bool ucol, const unsigned* __restrict__ Mbuf) {
-  __shared__ __align__(16) float Xs[W2][XLD];  // Xs[k][r] = X_Q(r, k); R32_BOTH: then T = X_Q U_Q per warp
-  __shared__ __align__(16) float Us[W2][ULD];  // Us[k][c] = U_Q(k, c)
-  __shared__ __align__(16) float Ua[TRI == R32_BOTH ? 4 : 1][W2][ULD];  // U_a of each warp's pair
+template <int NUA>
+struct __align__(16) Rmul32Smem {
+  float Xs[W2][XLD];       // Xs[k][r] = X_Q(r, k); R32_BOTH: then T = X_Q U_Q per warp
+  float Us[W2][ULD];       // Us[k][c] = U_Q(k, c)
+  float Ua[NUA][W2][ULD];  // R32_BOTH: U_a of each warp's pair
+};
+template <int TRI, bool MASKED, int NUA>
+MPJ_DEV void rmul32_tile(Rmul32Smem<NUA>& sm, const float* X, float* Y, int N, int nb, int R,
+                         const float* __restrict__ Sbuf, const float* __restrict__ Ubuf, bool hq, bool ucol,
+                         const unsigned* __restrict__ Mbuf, int gx, int Q) {
+  auto& Xs = sm.Xs;
+  auto& Us = sm.Us;
+  auto& Ua = sm.Ua;
   const int tid = threadIdx.x;
-  const int Q = blockIdx.y, gx = blockIdx.x, npairs = nb / 2;
+  const int npairs = nb / 2;
   const int a0 = 4 * gx, a1 = min(4 * gx + 3, npairs - 1);
-  pdl_wait();
   if (TRI == R32_BOTH && a1 < Q) return;
   const int warp = tid >> 5, lane = tid & 31;
   const int a = a0 + warp;  // this warp's block pair
@@ -520,7 +556,47 @@ __global__ void __launch_bounds__(RT) rmul32(const float* X, float* Y, int N, in
   }
 }
 
+template <int TRI, bool MASKED>
+__global__ void __launch_bounds__(RT) rmul32(const float* X, float* Y, int N, int nb, int R,
+                                             const float* __restrict__ Sbuf, const float* __restrict__ Ubuf, bool hq,
+                                             bool ucol, const unsigned* __restrict__ Mbuf) {
+  __shared__ Rmul32Smem<TRI == R32_BOTH ? 4 : 1> sm;
+  pdl_wait();
+  rmul32_tile<TRI, MASKED>(sm, X, Y, N, nb, R, Sbuf, Ubuf, hq, ucol, Mbuf, blockIdx.x, blockIdx.y);
+}
+
+// A batch: the tiles of A <- U~^T A U~, then those of V <- V U~, per matrix.
+MPJ_DEV int batch_tiles32(int np) { return 2 * ((np + 3) / 4) * np; }
+__global__ void __launch_bounds__(RT) rmul32_batch(BatchShape b, int lo, int R, float* A32, float* V32,
+                                                   const float* __restrict__ S, const float* __restrict__ U) {
+  __shared__ Rmul32Smem<4> sm;
+  pdl_wait();
+  BatchTask t;
+  if (!batch_find(b, lo, blockIdx.x, batch_tiles32, t)) return;
+  const int np = t.N / W2, per = ((np + 3) / 4) * np, nb = t.N / BS;
+  const float *Sm = S + (size_t)t.pair0 * W2 * W2, *Um = U + (size_t)t.pair0 * W2 * W2;
+  if (t.local < per)
+    rmul32_tile<R32_BOTH, false>(sm, A32 + t.el, A32 + t.el, t.N, nb, R, Sm, Um, false, false, nullptr, t.local / np,
+                                 t.local % np);
+  else
+    rmul32_tile<R32_ALL, false>(sm, V32 + t.el, V32 + t.el, t.N, nb, R, Sm, Um, false, false, nullptr,
+                                (t.local - per) / np, (t.local - per) % np);
+}
+
 }  // namespace
+
+cudaError_t mpj_batch_stage1_round(const BatchShape& b, int R, float* A32, float* V32, float* S, float* U,
+                                   cudaStream_t s) {
+  const int lo = batch_lowest_class(R);
+  const long long subs = batch_blocks(b, lo, [](int np) { return np; });
+  if (subs == 0) return cudaSuccess;
+  cudaError_t e = mpj_launch_pdl(solve32<false, BatchSub32>, dim3((unsigned)subs), dim3(S32_THREADS), 0, s,
+                                 BatchSub32{b, lo, A32, S, U}, R, true);
+  if (e != cudaSuccess) return e;
+  const long long tiles = batch_blocks(b, lo, [](int np) { return 2 * ((np + 3) / 4) * np; });
+  return mpj_launch_pdl(rmul32_batch, dim3((unsigned)tiles), dim3(RT), 0, s, b, lo, R, A32, V32, (const float*)S,
+                        (const float*)U);
+}
 
 int mpj_stage1_padded(int n) { return ((n + W2 - 1) / W2) * W2; }
 
@@ -586,8 +662,8 @@ cudaError_t stage1_sweep(const Stage1Bufs& b, cudaStream_t s, SideStream* side) 
     float* Ubuf = b.Ub[par];
     if (side && vpending[par]) S1_TRY(cudaStreamWaitEvent(s, side->done[par], 0));
     unsigned* Mbuf = b.sparse ? b.Mb[par] : nullptr;
-    S1_TRY(mpj_launch_pdl(b.half ? solve32<true> : solve32<false>, dim3(npairs), dim3(S32_THREADS), 0, s,
-                          (const float*)b.A32, N, nb, R, Sbuf, Ubuf, b.tc != 1, Mbuf));
+    S1_TRY(mpj_launch_pdl(b.half ? solve32<true, OneSub32> : solve32<false, OneSub32>, dim3(npairs), dim3(S32_THREADS),
+                          0, s, OneSub32{b.A32, N, nb, Sbuf, Ubuf, Mbuf}, R, b.tc != 1));
     auto vmul = b.sparse ? rmul32<R32_ALL, true> : rmul32<R32_ALL, false>;
     // V <- V U~
     if (side) {

@@ -299,9 +299,9 @@ def stage1_panel(R: int, U: torch.Tensor, In: torch.Tensor, transpose_out: bool 
 
 # ------------------------------------------------------------------ batched
 class BatchedSolver:
-    """Repeated mpj_syev_batched calls on fixed device buffers (the planned,
-    graph-replayed path): inputs are copied into the solver's own matrices,
-    so every call after the first replays the same CUDA graph."""
+    """Repeated mpj_syev_batched calls on fixed device buffers: inputs are
+    copied into the solver's own matrices, and every call after the first
+    reuses the plan (ordering, workspace) of the same sizes."""
 
     def __init__(self, sizes, device="cuda"):
         self.sizes = [int(n) for n in sizes]
@@ -315,8 +315,10 @@ class BatchedSolver:
 
     def solve(self, mats=None, tol: float = 0.0):
         if mats is not None:
-            for dst, src in zip(self.A, mats):
-                dst.copy_(src)
+            # one fused copy: 2048 separate ones cost 8 ms of launches before the solve
+            pairs = list(zip(self.A, mats))
+            if pairs:
+                torch._foreach_copy_([d for d, _ in pairs], [m for _, m in pairs])
         sweeps = (ctypes.c_int * len(self.sizes))()
         st = lib().mpj_syev_batched(len(self.sizes), self.ns, _ptr(self.pa), _ptr(self.pw), _ptr(self.pq), tol,
                                     sweeps, _stream())
