@@ -22,24 +22,22 @@
 //                     written to its mirror, so A stays exactly symmetric),
 //   V[:, P]          (V <- V U~, in place).
 //
-// The right multiplication is FP64-accurate on the bf16 tensor cores: each
+// The right multiplication is FP64-accurate on the 16-bit tensor cores: each
 // CTA takes 128 rows of X_P (K = 32 values each), finds each row's largest
 // exponent e_r (max |x_rk| < 2^e_r), and cuts x_rk * 2^(56 - e_r), rounded to
 // an integer (magnitude below 2^56; the rounding is below 2^(e_r - 57)), into
 // seven signed digits of 8 bits (|d_0| <= 256, |d_i| <= 128, each exactly a
-// bf16).  U_P's columns are cut the same way when the subproblem is solved.
+// binary16).  U_P's columns are cut the same way when the subproblem is solved.
 // The digit products of levels L = i + j <= 6 (28 pairs) go to seven FP32
 // accumulators in tensor memory; over K = 32 a level sum is an integer of
 // magnitude at most (2 * 256 * 128 + 5 * 128^2) * 32 = 2^22.2.  Measured on
 // this GPU: the tensor cores' FP32 accumulation of such integer sums is exact
 // below 2^23 but not in [2^23, 2^24) (unsigned byte digits, whose level sums
-// reach 2^23.8, lost accuracy), so every bound here is kept below 2^23.  The epilogue reads the level sums, forms
-// Z = sum_L s_L 2^(8 (6 - L)) exactly in two 64-bit integers, rounds Z to FP64
-// once and scales by 2^(e_r + f_c - 64).  Dropped levels (L >= 7) are below
-// 2^-55 of max|x_r.| max|u_.c| per term.  The epilogue uses integer
-// instructions only (no FP64: on this GPU an FP64 instruction costs 64 times
-// an FP32 one), so the products cost tensor time plus integer work.
-#include <cuda_bf16.h>
+// reach 2^23.8, lost accuracy), so every bound here is kept below 2^23.  The
+// epilogue reads the level sums, forms Z = sum_L s_L 2^(8 (6 - L)) exactly in
+// two 64-bit integers, rounds Z to FP64 once and scales by 2^(e_r + f_c - 64).
+// Dropped levels (L >= 7) are below 2^-55 of max|x_r.| max|u_.c| per term.
+#include <cuda_fp16.h>
 #include <stdint.h>
 #include <stdio.h>
 
@@ -75,69 +73,44 @@ MPJ_DEV void block_pair(int nb, int R, int slot, int& I, int& J) {
 // core matrices (k-adjacent cores 128 bytes apart, 8-row groups 512 apart)
 MPJ_DEV int kmaj16(int row, int k) { return (((row >> 3) * 4 + (k >> 3)) << 7) + ((row & 7) << 4) + ((k & 7) << 1); }
 
-// Seven digits of an integer value: Y = |x| 2^(56 - e) < 2^56 rounded, sign sg
-// = +-1 (the weights are in digits_f32).
-MPJ_DEV void digits_of(unsigned long long Y, float sg, uint32_t d[NSL]) {
-  const unsigned long long T = Y + 0x0000808080808080ULL;
-  const uint32_t lo = (uint32_t)T, hi = (uint32_t)(T >> 32);
-  const float c128 = -8388736.0f * sg;  // -(2^23 + 128) sign(x)
-  // bytes of lo: d6+128, d5+128, d4+128, d3+128; of hi: d2+128, d1+128; hi >> 16: d0
-  d[6] = __float_as_uint(fmaf(__uint_as_float(__byte_perm(lo, 0x4B00u, 0x5440)), sg, c128));
-  d[5] = __float_as_uint(fmaf(__uint_as_float(__byte_perm(lo, 0x4B00u, 0x5441)), sg, c128));
-  d[4] = __float_as_uint(fmaf(__uint_as_float(__byte_perm(lo, 0x4B00u, 0x5442)), sg, c128));
-  d[3] = __float_as_uint(fmaf(__uint_as_float(__byte_perm(lo, 0x4B00u, 0x5443)), sg, c128));
-  d[2] = __float_as_uint(fmaf(__uint_as_float(__byte_perm(hi, 0x4B00u, 0x5440)), sg, c128));
-  d[1] = __float_as_uint(fmaf(__uint_as_float(__byte_perm(hi, 0x4B00u, 0x5441)), sg, c128));
-  d[0] = __float_as_uint(fmaf(__uint_as_float(0x4B000000u | (hi >> 16)), sg, -8388608.0f * sg));
+// Seven signed digits of 8 bits of x on the grid 2^e (|x| < 2^e): x = sum_i d_i
+// 2^(e - 8 (i + 1)) + r, |r| <= 2^(e - 57), |d_0| <= 256, |d_i| <= 128 (i >= 1).
+// Y = |x| 2^(56 - e) rounded to an integer (half up; Y < 2^56); adding 128 to
+// each of its six low bytes (one 64-bit add, carries included) makes byte j of
+// the sum T d_(6-j) + 128 for centred digits d in [-128, 127], and the part
+// above bit 48 d_0 in [0, 256].  Centred digits keep every level sum of the
+// products below 2^23 (see the file comment).
+constexpr unsigned long long DIGIT_BIAS = 0x0000808080808080ULL;
+MPJ_DEV unsigned long long biased_digits(double x, int e) {
+  const uint32_t xh = (uint32_t)__double2hiint(x), xl = (uint32_t)__double2loint(x);
+  const int ex = (int)((xh >> 20) & 0x7FF);
+  const uint32_t mh = (xh & 0xFFFFFu) | (ex ? 0x100000u : 0u);
+  const int r = min(e + 1022 - max(ex, 1), 63);  // 2 Y = (mantissa 2^4) 2^-r, r >= 0
+  const unsigned long long w = (((unsigned long long)mh << 32) | xl) << 4;
+  return ((w >> r) + (1ULL + 2 * DIGIT_BIAS)) >> 1;  // rounding and bias in one add
 }
 
-// The seven signed digits of x on the grid 2^e (|x| < 2^e): x = sum_i d_i
-// 2^(e - 8 (i + 1)) + r, |r| <= 2^(e - 57), |d_0| <= 256, |d_i| <= 128 (i >= 1),
-// returned as FP32 bit patterns (exact small integers; their top 16 bits are
-// the bf16).  Y = round(|x| 2^(56 - e)) < 2^56; adding 128 to each of its six
-// low bytes (one 64-bit add, carries included) makes byte j of the sum
-// d_(6-j) + 128 for centred digits d in [-128, 127], and the part above bit 48
-// d_0 in [0, 256].  A byte b becomes a float through the bit pattern of
-// 2^23 + b (one byte permute), then one FMA gives sign(x) (b - 128).
-// Centred digits keep every level sum of the products below 2^23 (see the
-// file comment).
-MPJ_DEV void digits_f32(double x, int e, uint32_t d[NSL]) {
-  const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
-  const int ex = (int)((bits >> 52) & 0x7FF);
-  const unsigned long long mant = bits & 0xFFFFFFFFFFFFFULL;
-  const unsigned long long M = ex ? (mant | (1ULL << 52)) : mant;
-  const int sh = (ex ? ex : 1) - 1019 - e;  // |x| 2^(56 - e) = M 2^sh, sh <= 3
-  unsigned long long Y;
-  if (sh >= 0)
-    Y = M << sh;
-  else if (sh > -62)
-    Y = (M + (1ULL << (-sh - 1))) >> (-sh);
-  else
-    Y = 0;
-  digits_of(Y, (bits >> 63) ? -1.0f : 1.0f, d);
-}
-
-// Two FP32 digit patterns packed as two bf16 (a in the low half).
-MPJ_DEV uint32_t pack_bf16x2(uint32_t a, uint32_t b) { return __byte_perm(a, b, 0x7632); }
-
-// The same from the bit pattern of max|x| (a non-negative double), with
-// integer instructions only: the smallest e with max|x| < 2^e (0 for zero).
-MPJ_DEV int exp_of_maxbits(unsigned long long b) {
-  if (b == 0) return 0;
-  const int ex = (int)(b >> 52);
-  if (ex > 0) return ex - 1022;                     // 1.m 2^(ex-1023) < 2^(ex-1022)
-  return (64 - __clzll((long long)b)) - 1074;       // subnormal: mant 2^-1074
-}
-
-// v 2^E as a double, exact for |v| < 2^53 when the result is a normal
-// number (integer instructions only); 0 for v = 0.
-MPJ_DEV double exact_scaled(long long v, int E) {
-  if (v == 0) return 0.0;
-  const unsigned long long sign = v < 0 ? (1ULL << 63) : 0ULL;
-  const unsigned long long a = v < 0 ? (unsigned long long)(-v) : (unsigned long long)v;
-  const int p = 63 - __clzll((long long)a);  // leading bit, < 53
-  const unsigned long long m = (a << (52 - p)) & ((1ULL << 52) - 1ULL);
-  return __longlong_as_double((long long)(sign | ((unsigned long long)(p + E + 1023) << 52) | m));
+// The digits of two values (T from biased_digits, the signs in bit 31 of s0,
+// s1) as pairs of binary16 integers, first value in the low half.  A byte b
+// becomes 1024 + b by its bit pattern, and one packed FMA gives sign (b - 128):
+// three instructions for two digits, where FP32 patterns packed to bf16 took
+// five.
+MPJ_DEV void digit_pairs(unsigned long long T0, uint32_t s0, unsigned long long T1, uint32_t s1, uint32_t d[NSL]) {
+  const uint32_t lo0 = (uint32_t)T0, hi0 = (uint32_t)(T0 >> 32), lo1 = (uint32_t)T1, hi1 = (uint32_t)(T1 >> 32);
+  const uint32_t sg = ((s0 >> 16) & 0x8000u) | (s1 & 0x80000000u);
+  const uint32_t one = 0x3C003C00u | sg, c128 = 0xE480E480u ^ sg, c0 = 0xE400E400u ^ sg;  // sign, -1152 sign, -1024 sign
+  auto digit = [&](uint32_t v, uint32_t c) {
+    uint32_t r;
+    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(v | 0x64006400u), "r"(one), "r"(c));
+    return r;
+  };
+  d[6] = digit(__byte_perm(lo0, lo1, 0x0400) & 0x00FF00FFu, c128);
+  d[5] = digit(__byte_perm(lo0, lo1, 0x0501) & 0x00FF00FFu, c128);
+  d[4] = digit(__byte_perm(lo0, lo1, 0x0602) & 0x00FF00FFu, c128);
+  d[3] = digit(__byte_perm(lo0, lo1, 0x0703) & 0x00FF00FFu, c128);
+  d[2] = digit(__byte_perm(hi0, hi1, 0x0400) & 0x00FF00FFu, c128);
+  d[1] = digit(__byte_perm(hi0, hi1, 0x0501) & 0x00FF00FFu, c128);
+  d[0] = digit(__byte_perm(hi0, hi1, 0x7632), c0);
 }
 
 // Z 2^E rounded to the nearest double (ties to even), Z = hi 2^32 + lo with
@@ -418,7 +391,7 @@ struct Sub64 {
   const double* A;
   int lda, n, nb, P;
   double skip_abs;
-  __nv_bfloat16* sl;
+  __half* sl;
   int *ex, *rot;
   unsigned* nrot;
 };
@@ -426,7 +399,7 @@ struct OneSub64 {  // the block pairs of one matrix
   const double* A;
   int lda, n, nb;
   double skip_abs;
-  __nv_bfloat16* sl;
+  __half* sl;
   int *ex, *rot;
   unsigned* nrot;
   MPJ_DEV bool get(int bid, Sub64& v) const {
@@ -439,7 +412,7 @@ struct BatchSub64 {  // the block pairs of a batch
   int lo;
   const double* A;
   const double* skip_abs;
-  __nv_bfloat16* sl;
+  __half* sl;
   int *ex, *rot;
   MPJ_DEV bool get(int bid, Sub64& v) const {
     BatchTask t;
@@ -839,7 +812,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS, CTAS) blk_solve(Src src, int R,
   }
   // digits of U_P's columns: column c is "row" c of the right operand, over
   // k = row of U_P; eight threads per column, four values each
-  __nv_bfloat16* dst = sub.sl;
+  __half* dst = sub.sl;
   if (tid < 8 * W2) {
     const long long* Fs = reinterpret_cast<const long long*>(&sm.f);
     const int c = tid >> 3, k0 = (tid & 7) * 4;
@@ -855,20 +828,20 @@ __global__ void __launch_bounds__(SOLVE_THREADS, CTAS) blk_solve(Src src, int R,
     const int bits = 64 - __clzll((long long)top);  // max|F| < 2^bits
     if ((tid & 7) == 0) sub.ex[c] = bits - 60;
     const int sh = bits - 56;  // Y = |F| 2^-sh rounded
-    uint32_t d[4][NSL];
+    unsigned long long T[4];
+    uint32_t neg[4], d[2][NSL];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const unsigned long long m = (unsigned long long)(v[j] < 0 ? -v[j] : v[j]);
-      const unsigned long long Y = sh > 0 ? (m + (1ULL << (sh - 1))) >> sh : m << -sh;
-      digits_of(Y, v[j] < 0 ? -1.0f : 1.0f, d[j]);
+      T[j] = (sh > 0 ? (m + (1ULL << (sh - 1))) >> sh : m << -sh) + DIGIT_BIAS;
+      neg[j] = (uint32_t)((unsigned long long)v[j] >> 32);
     }
+    digit_pairs(T[0], neg[0], T[1], neg[1], d[0]);
+    digit_pairs(T[2], neg[2], T[3], neg[3], d[1]);
 #pragma unroll
-    for (int sl = 0; sl < NSL; ++sl) {
-      uint2 q;
-      q.x = pack_bf16x2(d[0][sl], d[1][sl]);
-      q.y = pack_bf16x2(d[2][sl], d[3][sl]);
-      *reinterpret_cast<uint2*>(reinterpret_cast<char*>(dst + (size_t)sl * (USL_BYTES / 2)) + kmaj16(c, k0)) = q;
-    }
+    for (int sl = 0; sl < NSL; ++sl)
+      *reinterpret_cast<uint2*>(reinterpret_cast<char*>(dst + (size_t)sl * (USL_BYTES / 2)) + kmaj16(c, k0)) =
+          make_uint2(d[0][sl], d[1][sl]);
   }
   if (tid == 0) {
     *sub.rot = 1;
@@ -883,9 +856,9 @@ MPJ_DEV uint64_t sdesc(uint32_t saddr) {
          ((uint64_t)1 << 46);
 }
 
-// kind::f16 instruction descriptor: D F32, A and B bf16, both K-major
+// kind::f16 instruction descriptor: D F32, A and B binary16, both K-major
 __host__ __device__ constexpr uint32_t idesc_f16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+  return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 MPJ_DEV void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
@@ -909,20 +882,10 @@ MPJ_DEV bool mbar_test(uint32_t mbar, uint32_t parity) {
   return ok != 0;
 }
 
-#define BLK_LD32(taddr, v)                                                                                         \
-  asm volatile(                                                                                                    \
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18," \
-      "%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"                                               \
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),           \
-        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),     \
-        "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),   \
-        "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])    \
-      : "r"(taddr))
-
 struct __align__(1024) RmulSmem {
   unsigned char xs[NSL][XSL_BYTES];  // digits of the 128 x 32 tile of X_P
   unsigned char us[NSL][USL_BYTES];  // digits of U_P
-  int uexp[W2];
+  int uexp[W2];  // column exponent of U_P, shifted to a double's exponent field
   int rexp[TM];
   uint64_t mbar;
   uint32_t tmem;
@@ -944,33 +907,46 @@ enum { XMODE_COLS = 0, XMODE_ROWS = 1 };
 //             the diagonal, mirrored.  So Y = U~^T A U~ stays exactly
 //             symmetric, and the second step reads B only in tiles (Q, a),
 //             Q <= a, the ones TRI_FIRST formed.
-// 256 threads: thread t digitizes tile row t/2 over block half t%2 (the 16
-// indices of block I or J of Q); warp w reads the TMEM lanes of rows
-// 32 (w mod 4) .. +31 and the 16 output columns 16 (w / 4) .. +15 of each level.
-constexpr int RM_THREADS = 256;
+// 512 threads: thread t digitizes eight values, tile row t / 4 and quarter t mod
+// 4 of the contraction index (two quarters per block I, J of Q); warp w reads
+// the TMEM lanes of rows 32 (w mod 4) .. +31 and the 8 output columns
+// 8 (w / 4) .. +7 of each level.
+//
+// What bounds it: instructions and their latency (DRAM 10 - 14 %, tensor pipe 5
+// - 7 %), so both ends are counted.  Per value the digits take one shift, one
+// add and 1.5 instructions per digit (digit_pairs); per output the level sums
+// become integers by one FP32 add each (the conversion instruction issues at
+// an eighth of that rate), two shift-adds and two 64-bit multiply-adds place
+// them in the mantissas of two doubles with a fixed leading bit, and two FP64
+// adds remove it and round (the integer normalisation they replace took some
+// 30 instructions).  32 warps per SM hide what latency remains.
+// Measured at n = 4096, all block pairs rotating: V U~ 187 -> 142 us, A U~
+// 111 -> 84 us, B^T U~ 147 -> 94 us (its mirror also written in 64-byte runs).
+constexpr int RM_THREADS = 512;
+constexpr int QK = 8;  // values per thread
 enum { TRI_ALL = 0, TRI_FIRST = 1, TRI_SECOND = 2 };
 
-// The 16 values X_Q(row, k), k = g0 .. g0 + 15 (block I or J of Q); zeros for
-// row < 0 (no such block pair or a tile that is not formed), row >= n, or
+// The 8 values X_Q(row, k), k = g0 .. g0 + 7 (half of block I or J of Q); zeros
+// for row < 0 (no such block pair or a tile that is not formed), row >= n, or
 // indices >= n.
-MPJ_DEV void load_xrow(const double* X, int ldx, int xmode, int n, int row, int g0, double x[BS]) {
+MPJ_DEV void load_xrow(const double* X, int ldx, int xmode, int n, int row, int g0, double x[QK]) {
   if (row < 0) {
 #pragma unroll
-    for (int k = 0; k < BS; ++k) x[k] = 0.0;
+    for (int k = 0; k < QK; ++k) x[k] = 0.0;
   } else if (xmode == XMODE_COLS) {
 #pragma unroll
-    for (int k = 0; k < BS; ++k) x[k] = (row < n && g0 + k < n) ? X[(size_t)(g0 + k) * ldx + row] : 0.0;
-  } else if (row < n && g0 + BS <= n && ((((size_t)row * ldx + g0) & 1) == 0)) {
+    for (int k = 0; k < QK; ++k) x[k] = (row < n && g0 + k < n) ? X[(size_t)(g0 + k) * ldx + row] : 0.0;
+  } else if (row < n && g0 + QK <= n && ((((size_t)row * ldx + g0) & 1) == 0)) {
     const double2* src = reinterpret_cast<const double2*>(X + (size_t)row * ldx + g0);
 #pragma unroll
-    for (int k = 0; k < BS / 2; ++k) {
+    for (int k = 0; k < QK / 2; ++k) {
       const double2 v = src[k];
       x[2 * k] = v.x;
       x[2 * k + 1] = v.y;
     }
   } else {
 #pragma unroll
-    for (int k = 0; k < BS; ++k) x[k] = (row < n && g0 + k < n) ? X[(size_t)row * ldx + g0 + k] : 0.0;
+    for (int k = 0; k < QK; ++k) x[k] = (row < n && g0 + k < n) ? X[(size_t)row * ldx + g0 + k] : 0.0;
   }
 }
 
@@ -989,7 +965,7 @@ MPJ_DEV bool tile_needed(int tri, int a, int Q) {
 }
 
 MPJ_DEV void blk_rmul_tile(const double* X, int ldx, int xmode, double* Y, int ldy, int n, int nb, int R,
-                           const __nv_bfloat16* __restrict__ Usl, const int* __restrict__ Uexp,
+                           const __half* __restrict__ Usl, const int* __restrict__ Uexp,
                            const int* __restrict__ rotated, unsigned* __restrict__ flags, int tri, int gx, int Q) {
   extern __shared__ __align__(1024) unsigned char dsm_raw[];
   RmulSmem& sm = *reinterpret_cast<RmulSmem*>(dsm_raw + ((1024 - (smem_u32(dsm_raw) & 1023)) & 1023));
@@ -1005,15 +981,15 @@ MPJ_DEV void blk_rmul_tile(const double* X, int ldx, int xmode, double* Y, int l
     // keeps its values: the second step leaves it alone, so the first need not
     // copy it to B.
     if (X == Y && xmode == XMODE_COLS) return;
-    const int rl = tid >> 1, half = tid & 1;
+    const int rl = tid >> 2, qk = tid & 3;
     const int a = a0 + (rl >> 5);
     const int row = tile_row(nb, R, gx, rl);
-    const int g0 = (half ? J : I) * BS;
+    const int g0 = (qk & 2 ? J : I) * BS + QK * (qk & 1);
     if (row >= 0 && row < n && tile_needed(tri, a, Q) && (tri == TRI_ALL || rotated[a])) {
-      double x[BS];
+      double x[QK];
       load_xrow(X, ldx, xmode, n, row, g0, x);
 #pragma unroll
-      for (int c = 0; c < BS; ++c) {
+      for (int c = 0; c < QK; ++c) {
         const int g = g0 + c;
         if (g < n && (tri != TRI_SECOND || a > Q || row >= g)) {
           Y[(size_t)g * ldy + row] = x[c];
@@ -1035,41 +1011,37 @@ MPJ_DEV void blk_rmul_tile(const double* X, int ldx, int xmode, double* Y, int l
     const uint4* src = reinterpret_cast<const uint4*>(Usl + (size_t)Q * NSL * (USL_BYTES / 2));
     uint4* dst = reinterpret_cast<uint4*>(sm.us[0]);
     for (int i = tid; i < NSL * USL_BYTES / 16; i += RM_THREADS) dst[i] = src[i];
-    if (tid < W2) sm.uexp[tid] = Uexp[Q * W2 + tid];
+    if (tid < W2) sm.uexp[tid] = Uexp[Q * W2 + tid] << 20;
   }
-  // digits of X_Q: this thread's tile row, 16 values of one block (zeros for
+  // digits of X_Q: this thread's tile row, 8 values of one block (zeros for
   // rows of tiles that are not formed)
   {
-    const int rl = tid >> 1, half = tid & 1;
+    const int rl = tid >> 2, qk = tid & 3;
     const int row = tile_row(nb, R, gx, rl);
-    const int g0 = (half ? J : I) * BS;
-    double x[BS];
+    const int g0 = (qk & 2 ? J : I) * BS + QK * (qk & 1);
+    double x[QK];
     load_xrow(X, ldx, xmode, n, tile_needed(tri, a0 + (rl >> 5), Q) ? row : -1, g0, x);
-    unsigned long long maxbits = 0;
+    uint32_t mh = 0, ml = 0;  // largest high word of the magnitudes, all low words
 #pragma unroll
-    for (int k = 0; k < BS; ++k) {
-      const unsigned long long b = (unsigned long long)__double_as_longlong(x[k]) & 0x7FFFFFFFFFFFFFFFULL;
-      maxbits = b > maxbits ? b : maxbits;
+    for (int k = 0; k < QK; ++k) {
+      mh = max(mh, (uint32_t)__double2hiint(x[k]) & 0x7FFFFFFFu);
+      ml |= (uint32_t)__double2loint(x[k]);
     }
-    const unsigned long long other = __shfl_xor_sync(0xffffffffu, maxbits, 1);
-    maxbits = other > maxbits ? other : maxbits;
-    const int er = exp_of_maxbits(maxbits);
-    if (half == 0) sm.rexp[rl] = er;
+    mh = max(mh, __shfl_xor_sync(0xffffffffu, mh, 1));
+    mh = max(mh, __shfl_xor_sync(0xffffffffu, mh, 2));
+    ml |= __shfl_xor_sync(0xffffffffu, ml, 1);
+    ml |= __shfl_xor_sync(0xffffffffu, ml, 2);
+    // max|x| < 2^er; subnormal rows take the bound 2^-1021 (their grid is finer than any double's)
+    const int er = (mh | ml) == 0 ? 0 : max((int)(mh >> 20), 1) - 1022;
+    if (qk == 0) sm.rexp[rl] = er;
+    uint32_t d[QK / 2][NSL];
 #pragma unroll
-    for (int k0 = 0; k0 < BS; k0 += 8) {
-      uint32_t d[8][NSL];
+    for (int j = 0; j < QK / 2; ++j)
+      digit_pairs(biased_digits(x[2 * j], er), (uint32_t)__double2hiint(x[2 * j]), biased_digits(x[2 * j + 1], er),
+                  (uint32_t)__double2hiint(x[2 * j + 1]), d[j]);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) digits_f32(x[k0 + j], er, d[j]);
-#pragma unroll
-      for (int s = 0; s < NSL; ++s) {
-        uint4 q;
-        q.x = pack_bf16x2(d[0][s], d[1][s]);
-        q.y = pack_bf16x2(d[2][s], d[3][s]);
-        q.z = pack_bf16x2(d[4][s], d[5][s]);
-        q.w = pack_bf16x2(d[6][s], d[7][s]);
-        *reinterpret_cast<uint4*>(sm.xs[s] + kmaj16(rl, half * BS + k0)) = q;
-      }
-    }
+    for (int s = 0; s < NSL; ++s)
+      *reinterpret_cast<uint4*>(sm.xs[s] + kmaj16(rl, QK * qk)) = make_uint4(d[0][s], d[1][s], d[2][s], d[3][s]);
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1115,48 +1087,68 @@ MPJ_DEV void blk_rmul_tile(const double* X, int ldx, int xmode, double* Y, int l
   if (ok && a < nb / 2 && tile_needed(tri, a, Q)) {
     const int rl = quad * 32 + lane;
     const int row = tile_row(nb, R, gx, rl);
-    // Z = sum_L s_L 2^(8 (6 - L)) = hi 2^32 + lo, hi = s0 2^16 + (s1 2^8 + s2),
-    // lo = (s3 2^8 + s4) 2^16 + (s5 2^8 + s6); the bracketed pairs fit 32 bits
-    // (|s_L| < 2^22.2), so levels are read in pairs and combined in int32
-    int t[4][BS];
+    const int er = sm.rexp[rl];
+    const int g0 = (ch & 2 ? J : I) * BS + QK * (ch & 1);
+    const bool diag = tri == TRI_SECOND && a == Q;
+    double out[QK];
 #pragma unroll
-    for (int c = 0; c < BS; ++c) t[0][c] = t[1][c] = t[2][c] = t[3][c] = 0;
+    for (int c0 = 0; c0 < QK; c0 += 4) {
+      uint32_t v[NLEV][4];
 #pragma unroll
-    for (int l = 0; l < NLEV; ++l) {
-      uint32_t v[16];
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-          : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-            "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-          : "r"(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(l * W2 + ch * BS)));
+      for (int l = 0; l < NLEV; ++l)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(v[l][0]), "=r"(v[l][1]), "=r"(v[l][2]), "=r"(v[l][3])
+                     : "r"(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(l * W2 + ch * QK + c0)));
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      // level l goes to partial (l + 1) / 2 with weight 2^8 if l is odd (l = 1, 3, 5), 1 otherwise
-      const int slot = (l + 1) >> 1;
+      const int4 ue = *reinterpret_cast<const int4*>(&sm.uexp[ch * QK + c0]);
+      const int uec[4] = {ue.x, ue.y, ue.z, ue.w};
 #pragma unroll
-      for (int c = 0; c < BS; ++c) {
-        const int q = __float2int_rz(__uint_as_float(v[c]));  // exact integer below 2^23
-        t[slot][c] = (l & 1) ? (q << 8) : t[slot][c] + q;
+      for (int c = 0; c < 4; ++c) {
+        // Z = sum_L s_L 2^(8 (6 - L)) = hi 2^32 + lo, hi = s0 2^16 + (s1 2^8 + s2),
+        // lo = (s3 2^8 + s4) 2^16 + (s5 2^8 + s6); the bracketed pairs fit 32 bits
+        // (|s_L| < 2^22.2).  s + 1.5 2^23 has the bit pattern 0x4B400000 + s.
+        uint32_t q[NLEV];
+#pragma unroll
+        for (int l = 0; l < NLEV; ++l) q[l] = __float_as_uint(__fadd_rn(__uint_as_float(v[l][c]), 12582912.0f));
+        constexpr uint32_t B0 = 0x4B400000u, B1 = (B0 << 8) + B0;
+        const int t0 = (int)(q[0] - B0), t1 = (int)((q[1] << 8) + q[2] - B1);
+        const int t2 = (int)((q[3] << 8) + q[4] - B1), t3 = (int)((q[5] << 8) + q[6] - B1);
+        if ((unsigned)(er + 900) < 1800u) {
+          // |hi| < 2^39, |lo| < 2^47: with 1.5 2^52 added they are mantissas of the doubles
+          // (1.5 2^52 + hi) 2^(32 + E) and (1.5 2^52 + lo) 2^E, E = er + ue - 64.  Taking
+          // 1.5 2^(52 + E) (2^32 + 1) from the first is exact and leaves hi 2^(32 + E) minus the
+          // second's bias, so the last add is the one rounding of Z 2^E.
+          const int kh = ((er + 32 - 64 + 1075) << 20) + uec[c] + 0x80000, kl = kh - (32 << 20);
+          const long long hi = (long long)t0 * 65536 + (((long long)kh << 32) + (long long)t1);
+          const long long lo = (long long)t2 * 65536 + (((long long)kl << 32) + (long long)t3);
+          const double x = __dsub_rn(__longlong_as_double(hi), __hiloint2double(kh, 0x00180000));
+          out[c0 + c] = __dadd_rn(x, __longlong_as_double(lo));
+        } else {
+          out[c0 + c] = z_to_double(((long long)t0 << 16) + t1, ((long long)t2 << 16) + t3, er + (uec[c] >> 20) - 64);
+        }
       }
     }
     if (row >= 0 && row < n) {
-      const int er = sm.rexp[rl];
-      const int g0 = (ch ? J : I) * BS;
-      const bool diag = tri == TRI_SECOND && a == Q;
 #pragma unroll
-      for (int c = 0; c < BS; ++c) {
+      for (int c = 0; c < QK; ++c) {
         const int g = g0 + c;
-        if (g < n && (!diag || row >= g)) {
-          // hi 2^32 + lo from the partials, both exact as doubles (|hi| < 2^39, |lo| < 2^47);
-          // one FP64 add rounds the sum once (the same as rounding Z)
-          const int E = er + sm.uexp[ch * BS + c] - 64;
-          const long long hi = ((long long)t[0][c] << 16) + t[1][c];
-          const long long lo = ((long long)t[2][c] << 16) + t[3][c];
-          const int bexp = 32 + E + 1023;
-          const double v = (bexp > 60 && bexp < 2000) ? exact_scaled(hi, 32 + E) + exact_scaled(lo, E)
-                                                      : z_to_double(hi, lo, E);
-          Y[(size_t)g * ldy + row] = v;
-          if (tri == TRI_SECOND && (!diag || row > g)) Y[(size_t)row * ldy + g] = v;  // the mirror entry
-        }
+        if (g < n && (!diag || row >= g)) Y[(size_t)g * ldy + row] = out[c];
+      }
+    }
+    if (tri == TRI_SECOND) {
+      // the mirror entries, through shared memory so that eight lanes write
+      // 64 contiguous bytes (the digit tiles are free: the products are done)
+      double* buf = reinterpret_cast<double*>(sm.xs[0]) + warp * 32 * (QK + 1);
+#pragma unroll
+      for (int c = 0; c < QK; ++c) buf[lane * (QK + 1) + c] = out[c];
+      __syncwarp();
+      int Ia, Ja;
+      block_pair(nb, R, a, Ia, Ja);
+      const int g = g0 + (lane & 7);
+#pragma unroll
+      for (int i = 0; i < QK; ++i) {
+        const int l = 4 * i + (lane >> 3), r = gidx(Ia, Ja, l);
+        if (r < n && g < n && (!diag || r > g)) Y[(size_t)r * ldy + g] = buf[l * (QK + 1) + (lane & 7)];
       }
     }
   }
@@ -1168,7 +1160,7 @@ MPJ_DEV void blk_rmul_tile(const double* X, int ldx, int xmode, double* Y, int l
 
 __global__ void __launch_bounds__(RM_THREADS, 2)
     blk_rmul(const double* X, int ldx, int xmode, double* Y, int ldy, int n, int nb, int R,
-             const __nv_bfloat16* __restrict__ Usl, const int* __restrict__ Uexp, const int* __restrict__ rotated,
+             const __half* __restrict__ Usl, const int* __restrict__ Uexp, const int* __restrict__ rotated,
              unsigned* __restrict__ flags, int tri) {
   pdl_wait();
   blk_rmul_tile(X, ldx, xmode, Y, ldy, n, nb, R, Usl, Uexp, rotated, flags, tri, blockIdx.x, blockIdx.y);
@@ -1178,7 +1170,7 @@ __global__ void __launch_bounds__(RM_THREADS, 2)
 // step 1, those of A = B^T U~.
 __global__ void __launch_bounds__(RM_THREADS, 2)
     blk_rmul_batch(BatchShape b, int lo, int R, int step, double* A, double* V, double* B,
-                   const __nv_bfloat16* __restrict__ sl, const int* __restrict__ ex, const int* __restrict__ rot,
+                   const __half* __restrict__ sl, const int* __restrict__ ex, const int* __restrict__ rot,
                    unsigned* __restrict__ flags) {
   pdl_wait();
   BatchTask t;
@@ -1213,7 +1205,7 @@ size_t mpj_blocked_scratch_bytes(int n) {
 
 namespace {
 struct USet {
-  __nv_bfloat16* sl;
+  __half* sl;
   int* ex;
   int* rot;
 };
@@ -1222,7 +1214,7 @@ USet uset(void* scratch, int n, int parity) {
   const int npairs = N / (2 * BS);
   char* base = (char*)scratch + (size_t)parity * uset_bytes(npairs);
   USet u;
-  u.sl = (__nv_bfloat16*)base;
+  u.sl = (__half*)base;
   u.ex = (int*)(base + al256((size_t)npairs * NSL * USL_BYTES));
   u.rot = (int*)((char*)u.ex + al256((size_t)npairs * W2 * sizeof(int)));
   return u;
@@ -1271,10 +1263,10 @@ cudaError_t mpj_blocked_update_A(double* A, int lda, double* B, int n, int R, vo
   if (e != cudaSuccess) return e;
   const dim3 grid((nb / 2 + 3) / 4, nb / 2);
   e = mpj_launch_pdl(blk_rmul, grid, dim3(RM_THREADS), rmul_smem(), s, (const double*)A, lda, (int)XMODE_COLS, B, n,
-                     n, nb, R, (const __nv_bfloat16*)u.sl, (const int*)u.ex, (const int*)u.rot, flags, (int)TRI_FIRST);
+                     n, nb, R, (const __half*)u.sl, (const int*)u.ex, (const int*)u.rot, flags, (int)TRI_FIRST);
   if (e != cudaSuccess) return e;
   return mpj_launch_pdl(blk_rmul, grid, dim3(RM_THREADS), rmul_smem(), s, (const double*)B, n, (int)XMODE_ROWS, A,
-                        lda, n, nb, R, (const __nv_bfloat16*)u.sl, (const int*)u.ex, (const int*)u.rot, flags,
+                        lda, n, nb, R, (const __half*)u.sl, (const int*)u.ex, (const int*)u.rot, flags,
                         (int)TRI_SECOND);
 }
 
@@ -1287,7 +1279,7 @@ cudaError_t mpj_blocked_update_V(double* V, int ldv, int n, int R, void* scratch
   if (e != cudaSuccess) return e;
   const dim3 grid((nb / 2 + 3) / 4, nb / 2);
   return mpj_launch_pdl(blk_rmul, grid, dim3(RM_THREADS), rmul_smem(), s, (const double*)V, ldv, (int)XMODE_COLS, V,
-                        ldv, n, nb, R, (const __nv_bfloat16*)u.sl, (const int*)u.ex, (const int*)u.rot, flags,
+                        ldv, n, nb, R, (const __half*)u.sl, (const int*)u.ex, (const int*)u.rot, flags,
                         (int)TRI_ALL);
 }
 
@@ -1300,7 +1292,7 @@ cudaError_t mpj_batch_sweep64_round(const BatchShape& b, int R, double* A, doubl
   if (subs == 0) return cudaSuccess;
   cudaError_t e = rmul_attr();
   if (e != cudaSuccess) return e;
-  __nv_bfloat16* sl = (__nv_bfloat16*)digits;
+  __half* sl = (__half*)digits;
   int* ex = (int*)((char*)digits + al256((size_t)pairs * NSL * USL_BYTES));
   int* rot = (int*)((char*)ex + al256((size_t)pairs * W2 * sizeof(int)));
   const BatchSub64 src{b, lo, A, skip_abs, sl, ex, rot};
@@ -1309,7 +1301,7 @@ cudaError_t mpj_batch_sweep64_round(const BatchShape& b, int R, double* A, doubl
   const long long tiles = batch_blocks(b, lo, [](int np) { return ((np + 3) / 4) * np; });
   for (int step = 0; step < 2 && e == cudaSuccess; ++step)
     e = mpj_launch_pdl(blk_rmul_batch, dim3((unsigned)(step == 0 ? 2 * tiles : tiles)), dim3(RM_THREADS), rmul_smem(),
-                       s, b, lo, R, step, A, V, B, (const __nv_bfloat16*)sl, (const int*)ex, (const int*)rot, flags);
+                       s, b, lo, R, step, A, V, B, (const __half*)sl, (const int*)ex, (const int*)rot, flags);
   return e;
 }
 
