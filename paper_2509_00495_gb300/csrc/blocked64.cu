@@ -861,23 +861,39 @@ __host__ __device__ constexpr uint32_t idesc_f16(int M, int N) {
   return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// One MMA.  A's use of the collector buffer: successive products with the same
+// A tile read it from shared memory once (fill, use .., last) -- with N = 32 the
+// 4 KB of A per product are what the tensor core waits for.
+enum { A_ONCE = 0, A_FILL = 1, A_USE = 2, A_LAST = 3 };
+template <int COLLECT>
 MPJ_DEV void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
-      : "memory");
+#define BLK_MMA(usage)                                                          \
+  asm volatile(                                                                 \
+      "{\n\t.reg .pred p;\n\t"                                                 \
+      "setp.ne.b32 p, %4, 0;\n\t"                                              \
+      "tcgen05.mma.cta_group::1.kind::f16" usage " [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d), \
+      "l"(a), "l"(b), "r"(idesc), "r"(acc)                                      \
+      : "memory")
+  if (COLLECT == A_FILL)
+    BLK_MMA(".collector::a::fill");
+  else if (COLLECT == A_USE)
+    BLK_MMA(".collector::a::use");
+  else if (COLLECT == A_LAST)
+    BLK_MMA(".collector::a::lastuse");
+  else
+    BLK_MMA("");
+#undef BLK_MMA
 }
 
-MPJ_DEV bool mbar_test(uint32_t mbar, uint32_t parity) {
+// Waits up to about a microsecond in hardware for the phase of that parity.
+MPJ_DEV bool mbar_try(uint32_t mbar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}\n"
       : "=r"(ok)
-      : "r"(mbar), "r"(parity)
+      : "r"(mbar), "r"(parity), "r"(1000u)
       : "memory");
   return ok != 0;
 }
@@ -920,8 +936,10 @@ enum { XMODE_COLS = 0, XMODE_ROWS = 1 };
 // them in the mantissas of two doubles with a fixed leading bit, and two FP64
 // adds remove it and round (the integer normalisation they replace took some
 // 30 instructions).  32 warps per SM hide what latency remains.
-// Measured at n = 4096, all block pairs rotating: V U~ 187 -> 142 us, A U~
-// 111 -> 84 us, B^T U~ 147 -> 94 us (its mirror also written in 64-byte runs).
+// Measured at n = 4096, all block pairs rotating: V U~ 187 -> 139 us, A U~
+// 111 -> 81 us, B^T U~ 147 -> 96 us (its mirror also written in 64-byte runs);
+// of that 3 % from reading each A tile into the tensor core once and from
+// waiting for the products in hardware instead of polling.
 constexpr int RM_THREADS = 512;
 constexpr int QK = 8;  // values per thread
 enum { TRI_ALL = 0, TRI_FIRST = 1, TRI_SECOND = 2 };
@@ -1051,34 +1069,45 @@ MPJ_DEV void blk_rmul_tile(const double* X, int ldx, int xmode, double* Y, int l
   const uint32_t mb = smem_u32(&sm.mbar);
   if (tid == 0) {
     constexpr uint32_t idesc = idesc_f16(TM, W2);
-    uint32_t started = 0;
-    for (int i = 0; i < NSL; ++i)
-      for (int j = 0; i + j < NLEV; ++j) {
-        const int l = i + j;
+    const uint64_t xd = sdesc(smem_u32(sm.xs[0])), ud = sdesc(smem_u32(sm.us[0]));
+    // digit pair (i, j), i + j <= 6: level i + j; the products of one A tile in a row
 #pragma unroll
-        for (int kk = 0; kk < W2 / 16; ++kk) {
-          mma_f16(tmem + (uint32_t)(l * W2), sdesc(smem_u32(sm.xs[i]) + kk * 256), sdesc(smem_u32(sm.us[j]) + kk * 256),
-                  idesc, (started >> l) & 1u);
-          started |= 1u << l;
+    for (int i = 0; i < NSL; ++i) {
+#pragma unroll
+      for (int kk = 0; kk < W2 / 16; ++kk) {
+        const uint64_t ad = xd + (uint64_t)((i * XSL_BYTES + kk * 256) >> 4);
+#pragma unroll
+        for (int j = 0; i + j < NLEV; ++j) {
+          const uint64_t bd = ud + (uint64_t)((j * USL_BYTES + kk * 256) >> 4);
+          const uint32_t d = tmem + (uint32_t)((i + j) * W2), acc = i > 0 || kk > 0;
+          if (i == NSL - 1)
+            mma_f16<A_ONCE>(d, ad, bd, idesc, acc);
+          else if (j == 0)
+            mma_f16<A_FILL>(d, ad, bd, idesc, acc);
+          else if (i + j == NLEV - 1)
+            mma_f16<A_LAST>(d, ad, bd, idesc, acc);
+          else
+            mma_f16<A_USE>(d, ad, bd, idesc, acc);
         }
       }
+    }
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mb) : "memory");
   }
   // bounded wait for the products
   bool ok = true;
   {
     const long long t0 = clock64();
-    while (!mbar_test(mb, 0)) {
+    while (!mbar_try(mb, 0)) {
       if (clock64() - t0 > WAIT_CYCLES) {
         ok = false;
         break;
       }
-      __nanosleep(20);
     }
     if (!ok) {
       if (lane == 0 && flags) atomicOr(flags, MPJ_FLAG_TIMEOUT);
       const long long t1 = clock64();  // the products may still be in flight
-      while (!mbar_test(mb, 0) && clock64() - t1 <= WAIT_CYCLES) __nanosleep(64);
+      while (!mbar_try(mb, 0) && clock64() - t1 <= WAIT_CYCLES) {
+      }
     }
   }
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
