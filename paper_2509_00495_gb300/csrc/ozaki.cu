@@ -94,13 +94,30 @@ __host__ __device__ constexpr uint32_t oz_idesc(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// One MMA.  A's use of the collector buffer: successive products with the same
+// A tile read it from shared memory once (fill, use .., last).  The 4 KB of A
+// were two thirds of what an N = 64 product reads, and the reads, not the
+// multipliers, bound it: a 4096^3 product took 9.3 ms, with one read per A tile
+// 6.3 ms.
+enum { A_ONCE = 0, A_FILL = 1, A_USE = 2, A_LAST = 3 };
+template <int COLLECT>
 MPJ_DEV void oz_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
-      : "memory");
+#define OZ_MMA(usage)                                                           \
+  asm volatile(                                                                 \
+      "{\n\t.reg .pred p;\n\t"                                                 \
+      "setp.ne.b32 p, %4, 0;\n\t"                                              \
+      "tcgen05.mma.cta_group::1.kind::f16" usage " [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d), \
+      "l"(a), "l"(b), "r"(idesc), "r"(acc)                                      \
+      : "memory")
+  if (COLLECT == A_FILL)
+    OZ_MMA(".collector::a::fill");
+  else if (COLLECT == A_USE)
+    OZ_MMA(".collector::a::use");
+  else if (COLLECT == A_LAST)
+    OZ_MMA(".collector::a::lastuse");
+  else
+    OZ_MMA("");
+#undef OZ_MMA
 }
 
 MPJ_DEV void oz_commit(uint32_t mbar) {
@@ -379,19 +396,30 @@ MPJ_DEV void oz_tile(const __nv_bfloat16* __restrict__ SA, const int* __restrict
         if (chunk_start && chunk > 0 && !oz_wait(smem_u32(&sm.tmem_empty), (chunk - 1) & 1, abort_flag, gflags))
           break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t aB = stage0 + st * OZ_STAGE_BYTES, bB = aB + OZ_S * OZ_A_BYTES;
-        uint32_t started = chunk_start ? 0u : 0xFFu;
-        for (int i = 1; i <= OZ_S; ++i)
-          for (int j = 1; i + j <= OZ_S + 1; ++j) {
-            const int l = i + j - 2;
-            const uint32_t d = tmem + (uint32_t)(l * OZ_TN);
+        const uint64_t ad0 = oz_desc(stage0 + st * OZ_STAGE_BYTES);
+        const uint64_t bd0 = oz_desc(stage0 + st * OZ_STAGE_BYTES + OZ_S * OZ_A_BYTES);
+        // slice pair (i, j), i + j <= 9 (here from 0: i + j <= 7): level i + j;
+        // the products of one A tile in a row
 #pragma unroll
-            for (int kk = 0; kk < OZ_KS / 16; ++kk) {
-              oz_mma(d, oz_desc(aB + (i - 1) * OZ_A_BYTES + kk * 256), oz_desc(bB + (j - 1) * OZ_B_BYTES + kk * 256),
-                     idesc, (started >> l) & 1u);
-              started |= 1u << l;
+        for (int i = 0; i < OZ_S; ++i) {
+#pragma unroll
+          for (int kk = 0; kk < OZ_KS / 16; ++kk) {
+            const uint64_t ad = ad0 + (uint64_t)((i * OZ_A_BYTES + kk * 256) >> 4);
+#pragma unroll
+            for (int j = 0; i + j < OZ_LEVELS; ++j) {
+              const uint64_t bd = bd0 + (uint64_t)((j * OZ_B_BYTES + kk * 256) >> 4);
+              const uint32_t d = tmem + (uint32_t)((i + j) * OZ_TN), acc = i > 0 || kk > 0 ? 1u : (chunk_start ? 0u : 1u);
+              if (i == OZ_S - 1)
+                oz_mma<A_ONCE>(d, ad, bd, idesc, acc);
+              else if (j == 0)
+                oz_mma<A_FILL>(d, ad, bd, idesc, acc);
+              else if (i + j == OZ_LEVELS - 1)
+                oz_mma<A_LAST>(d, ad, bd, idesc, acc);
+              else
+                oz_mma<A_USE>(d, ad, bd, idesc, acc);
             }
           }
+        }
         oz_commit(smem_u32(&sm.empty[st]));
         last_commit_sub = sub;
         if ((sub + 1) % (OZ_KC / OZ_KS) == 0 || sub + 1 == nsub) oz_commit(smem_u32(&sm.tmem_full));
