@@ -247,8 +247,10 @@ MPJ_DEV uint32_t oz_pack2(uint32_t a, uint32_t b) { return __byte_perm(a, b, 0x7
 // Largest |x(r, k)| per row as the bit pattern of a non-negative double
 // (ordered like the value), combined with atomicMax.  Rows of a column-major
 // matrix (rs == 1): one thread per row over a strip of k, coalesced across rows.
-__global__ void oz_rowmax_cols(const double* __restrict__ X, long long ks, int R, int K, int kstrip,
-                               unsigned long long* __restrict__ mx) {
+__global__ void oz_rowmax_cols(const double* __restrict__ X, long long ks, long long sx, int R, int K, int kstrip,
+                               unsigned long long* __restrict__ mx, long long smx) {
+  X += blockIdx.z * sx;
+  mx += blockIdx.z * smx;
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= R) return;
   const int k0 = blockIdx.y * kstrip, k1 = min(K, k0 + kstrip);
@@ -258,8 +260,10 @@ __global__ void oz_rowmax_cols(const double* __restrict__ X, long long ks, int R
 }
 
 // Rows stored contiguously (or any other stride): one warp per row.
-__global__ void oz_rowmax_warp(const double* __restrict__ X, long long rs, long long ks, int R, int K,
-                               unsigned long long* __restrict__ mx) {
+__global__ void oz_rowmax_warp(const double* __restrict__ X, long long rs, long long ks, long long sx, int R, int K,
+                               unsigned long long* __restrict__ mx, long long smx) {
+  X += blockIdx.z * sx;
+  mx += blockIdx.z * smx;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (warp >= R) return;
   unsigned long long m = 0;
@@ -271,9 +275,13 @@ __global__ void oz_rowmax_warp(const double* __restrict__ X, long long rs, long 
 // The 8 slices of 8 consecutive k values of one row per thread, written as
 // one 16-byte core-matrix row per slice.  rows_fast: consecutive threads take
 // consecutive rows (coalesced reads of column-major rows).
-__global__ void oz_slice(const double* __restrict__ X, long long rs, long long ks, int R, int K, int Rp, int Kp,
-                         int rows_fast, const unsigned long long* __restrict__ mx, int* __restrict__ exps,
-                         __nv_bfloat16* __restrict__ S) {
+__global__ void oz_slice(const double* __restrict__ X, long long rs, long long ks, long long sx, int R, int K, int Rp,
+                         int Kp, int rows_fast, const unsigned long long* __restrict__ mx, int* __restrict__ exps,
+                         __nv_bfloat16* __restrict__ S, long long sop) {
+  X += blockIdx.z * sx;
+  mx = (const unsigned long long*)((const char*)mx + blockIdx.z * sop);
+  exps = (int*)((char*)exps + blockIdx.z * sop);
+  S = (__nv_bfloat16*)((char*)S + blockIdx.z * sop);
   const long long total = (long long)Rp * (Kp / 8);
   const long long slice_elems = (long long)Rp * Kp;
   for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -494,7 +502,14 @@ __global__ void __maxnreg__(168)
     oz_gemm_kernel(const __nv_bfloat16* __restrict__ SA, const int* __restrict__ ea, int Rpa,
                    const __nv_bfloat16* __restrict__ SB, const int* __restrict__ eb, int Rpb, int Kp, int sub0,
                    int nsub, int m, int n, double alpha, double beta, const double* Cin, int ldcin, double* C,
-                   int ldc, unsigned* gflags, int lower) {
+                   int ldc, unsigned* gflags, int lower, long long sa, long long sb, long long sc) {
+  // matrix blockIdx.y: operands sa, sb bytes apart, results sc elements
+  SA = (const __nv_bfloat16*)((const char*)SA + blockIdx.y * sa);
+  ea = (const int*)((const char*)ea + blockIdx.y * sa);
+  SB = (const __nv_bfloat16*)((const char*)SB + blockIdx.y * sb);
+  eb = (const int*)((const char*)eb + blockIdx.y * sb);
+  if (Cin) Cin += blockIdx.y * sc;  // with a batch, Cin is C
+  C += blockIdx.y * sc;
   // tile order: groups of OZ_GROUP_M row tiles share the B tiles in L2
   const int ntm = (m + OZ_TM - 1) / OZ_TM, ntn = (n + OZ_TN - 1) / OZ_TN;
   const int id = blockIdx.x;
@@ -594,20 +609,22 @@ size_t mpj_oz_operand_bytes(int R, int K) {
 }
 
 cudaError_t mpj_oz_prepare(const double* X, long long rs, long long ks, int R, int K, void* buf, OzOperand* op,
-                           cudaStream_t s) {
+                           cudaStream_t s, int batch, long long sx) {
   const int Rp = pad_rows(R), Kp = pad_k(K);
+  const size_t ob = mpj_oz_operand_bytes(R, K);
   char* b = (char*)buf;
   __nv_bfloat16* S = (__nv_bfloat16*)b;
   int* exps = (int*)(b + al256((size_t)OZ_S * Rp * Kp * 2));
   unsigned long long* mx = (unsigned long long*)((char*)exps + al256((size_t)Rp * sizeof(int)));
-  cudaError_t e = cudaMemsetAsync(mx, 0, (size_t)Rp * sizeof(unsigned long long), s);
+  const long long smx = (long long)(ob / sizeof(unsigned long long));
+  cudaError_t e = cudaMemset2DAsync(mx, ob, 0, (size_t)Rp * sizeof(unsigned long long), batch, s);
   if (e != cudaSuccess) return e;
   if (rs == 1) {
     const int kstrip = 64;
-    dim3 grid((R + 127) / 128, (K + kstrip - 1) / kstrip);
-    oz_rowmax_cols<<<grid, 128, 0, s>>>(X, ks, R, K, kstrip, mx);
+    dim3 grid((R + 127) / 128, (K + kstrip - 1) / kstrip, batch);
+    oz_rowmax_cols<<<grid, 128, 0, s>>>(X, ks, sx, R, K, kstrip, mx, smx);
   } else {
-    oz_rowmax_warp<<<(R + 7) / 8, 256, 0, s>>>(X, rs, ks, R, K, mx);
+    oz_rowmax_warp<<<dim3((R + 7) / 8, 1, batch), 256, 0, s>>>(X, rs, ks, sx, R, K, mx, smx);
   }
   mpj_count_launch();
   e = cudaGetLastError();
@@ -617,7 +634,8 @@ cudaError_t mpj_oz_prepare(const double* X, long long rs, long long ks, int R, i
   }
   const long long total = (long long)Rp * (Kp / 8);
   const int blocks = (int)((total + 255) / 256 > 8192 ? 8192 : (total + 255) / 256);
-  oz_slice<<<blocks, 256, 0, s>>>(X, rs, ks, R, K, Rp, Kp, rs == 1 ? 1 : 0, mx, exps, S);
+  oz_slice<<<dim3(blocks, 1, batch), 256, 0, s>>>(X, rs, ks, sx, R, K, Rp, Kp, rs == 1 ? 1 : 0, mx, exps, S,
+                                                  (long long)ob);
   mpj_count_launch();
   e = cudaGetLastError();
   if (e != cudaSuccess) {
@@ -635,8 +653,10 @@ cudaError_t mpj_oz_prepare(const double* X, long long rs, long long ks, int R, i
 
 cudaError_t mpj_oz_gemm(const OzOperand& a, const OzOperand& b, int m, int n, double alpha, double beta,
                         const double* Cin, int ldcin, double* C, int ldc, unsigned* flags, cudaStream_t s,
-                        bool lower) {
-  if (a.Kp != b.Kp || m > a.R || n > b.R || m < 1 || n < 1) return cudaErrorInvalidValue;
+                        bool lower, int batch, long long sc) {
+  if (a.Kp != b.Kp || m > a.R || n > b.R || m < 1 || n < 1 || batch < 1) return cudaErrorInvalidValue;
+  if (batch > 1 && beta != 0.0 && Cin != C) return cudaErrorInvalidValue;
+  const long long sa = (long long)mpj_oz_operand_bytes(a.R, a.K), sb = (long long)mpj_oz_operand_bytes(b.R, b.K);
   const size_t smem = sizeof(OzSmem) + 1024;
   cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -645,9 +665,9 @@ cudaError_t mpj_oz_gemm(const OzOperand& a, const OzOperand& b, int m, int n, do
   for (int sub0 = 0; sub0 < total; sub0 += OZ_PASS_SUBS) {
     const int ns = total - sub0 < OZ_PASS_SUBS ? total - sub0 : OZ_PASS_SUBS;
     const bool first = sub0 == 0;
-    oz_gemm_kernel<<<ntm * ntn, OZ_THREADS, smem, s>>>(a.slices, a.exps, a.Rp, b.slices, b.exps, b.Rp, a.Kp, sub0, ns,
-                                                        m, n, alpha, first ? beta : 1.0, first ? Cin : C,
-                                                        first ? ldcin : ldc, C, ldc, flags, lower ? 1 : 0);
+    oz_gemm_kernel<<<dim3(ntm * ntn, batch), OZ_THREADS, smem, s>>>(
+        a.slices, a.exps, a.Rp, b.slices, b.exps, b.Rp, a.Kp, sub0, ns, m, n, alpha, first ? beta : 1.0,
+        first ? Cin : C, first ? ldcin : ldc, C, ldc, flags, lower ? 1 : 0, sa, sb, sc);
     mpj_count_launch();
     e = cudaGetLastError();
     if (e != cudaSuccess) {
