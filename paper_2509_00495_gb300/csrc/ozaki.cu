@@ -661,7 +661,7 @@ cudaError_t mpj_oz_gemm(const OzOperand& a, const OzOperand& b, int m, int n, do
   cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int ntm = (m + OZ_TM - 1) / OZ_TM, ntn = (n + OZ_TN - 1) / OZ_TN;
-  const int total = a.Kp / OZ_KS;
+  const int total = (a.K + OZ_KS - 1) / OZ_KS;  // the padding to a whole chunk is zeros: left out
   for (int sub0 = 0; sub0 < total; sub0 += OZ_PASS_SUBS) {
     const int ns = total - sub0 < OZ_PASS_SUBS ? total - sub0 : OZ_PASS_SUBS;
     const bool first = sub0 == 0;
