@@ -14,6 +14,7 @@
 // operands of the tensor-core products (16 n^2 bytes each) and a small
 // scratch area.  About 56 n^2 + 8 N^2 bytes: 1 GiB at n = 4096.  The solve
 // allocates nothing when the caller passes a workspace.
+#include <cooperative_groups.h>
 #include <stdio.h>
 #include <string.h>
 
@@ -247,22 +248,16 @@ int fill_opts(int n, const mpj_opts* in, mpj_opts* o) {
   return MPJ_OK;
 }
 
-// y = E x / ||x|| for the symmetric n x n E (column i of E dotted with x, one
-// warp per column); partial[0..n) is y, the norm of x comes from *nrm.
-__global__ void pow_step(const double* __restrict__ E, int n, const double* __restrict__ x,
-                         const double* __restrict__ nrm, double* __restrict__ y) {
-  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (i >= n) return;
+// One row of y = E x / ||x|| by a warp (column i of the symmetric E dotted with x).
+MPJ_DEV double pow_row(const double* __restrict__ E, int n, const double* x, int i, int lane, double nx) {
   double t = 0.0;
   for (int j = lane; j < n; j += 32) t = fma(E[(size_t)i * n + j], x[j], t);
   for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  const double nx = *nrm;
-  if (lane == 0) y[i] = nx > 0.0 ? t / nx : 0.0;  // E x = 0 exactly: the estimate stays 0
+  return nx > 0.0 ? t / nx : 0.0;  // E x = 0 exactly: the estimate stays 0
 }
 
-// *nrm = ||y|| (one CTA, fixed order)
-__global__ void pow_norm(const double* __restrict__ y, int n, double* __restrict__ nrm) {
-  __shared__ double sh[256];
+// ||y|| by 256 threads in a fixed order
+MPJ_DEV double pow_norm(const volatile double* y, int n, double* sh) {
   double s = 0.0;
   for (int i = threadIdx.x; i < n; i += 256) s = fma(y[i], y[i], s);
   sh[threadIdx.x] = s;
@@ -271,33 +266,90 @@ __global__ void pow_norm(const double* __restrict__ y, int n, double* __restrict
     if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
     __syncthreads();
   }
-  if (threadIdx.x == 0) *nrm = sqrt(sh[0]);
+  const double r = sqrt(sh[0]);
+  __syncthreads();
+  return r;
 }
 
-__global__ void pow_init(double* __restrict__ x, int n) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) x[i] = 1.0 + 0.5 * sin((double)i);
+constexpr int POW_STEPS = 30;
+
+// One step: y = E x / *nrm, and the last CTA to finish leaves ||y|| in *nrm
+// (*ticket counts them and is zero again afterwards).  it < 0: the start vector
+// y and its norm.
+__global__ void __launch_bounds__(256) pow_step(const double* __restrict__ E, int n, const double* __restrict__ x,
+                                                double* __restrict__ nrm, double* __restrict__ y,
+                                                unsigned* __restrict__ ticket, int it) {
+  __shared__ double sh[256];
+  __shared__ bool last;
+  pdl_wait();
+  const int i = (blockIdx.x * 256 + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (it < 0) {
+    if (i < n && lane == 0) y[i] = 1.0 + 0.5 * sin((double)i);
+  } else if (i < n) {
+    const double t = pow_row(E, n, x, i, lane, *(const volatile double*)nrm);
+    if (lane == 0) y[i] = t;
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const double r = pow_norm(y, n, sh);
+  if (threadIdx.x == 0) {
+    *nrm = r;
+    *ticket = 0u;
+  }
+}
+
+// All steps by one cluster of POW_CTAS CTAs, the vector in each one's shared
+// memory: every CTA forms its rows and writes them to all.  61 launches of 3.9
+// us become one kernel; beyond POW_SMALL rows the FP64 pipes of eight SMs would
+// be slower than the launches.
+constexpr int POW_CTAS = 8, POW_SMALL = 384;
+__global__ void __cluster_dims__(POW_CTAS, 1, 1) __launch_bounds__(256)
+    pow_cluster(const double* __restrict__ E, int n, double* __restrict__ out) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  __shared__ double v[2][POW_SMALL], sh[256];
+  const int rank = (int)cluster.block_rank(), warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int i = threadIdx.x; i < n; i += 256) v[0][i] = 1.0 + 0.5 * sin((double)i);
+  __syncthreads();
+  double nx = pow_norm(v[0], n, sh);
+  cluster.sync();  // every CTA has started before its shared memory is written
+  for (int it = 0; it < POW_STEPS; ++it) {
+    const double* x = v[it & 1];
+    double* y = v[(it & 1) ^ 1];
+    for (int i = rank * 8 + warp; i < n; i += 8 * POW_CTAS) {
+      const double t = pow_row(E, n, x, i, lane, nx);
+      if (lane < POW_CTAS) cluster.map_shared_rank(y, lane)[i] = t;
+    }
+    cluster.sync();
+    nx = pow_norm(y, n, sh);
+  }
+  if (rank == 0 && threadIdx.x == 0) *out = nx;
 }
 
 // Estimate of ||E||_2 for symmetric E by 30 steps of the power iteration on
-// two n-vectors in `vec` (2n doubles) and one scalar.
+// two n-vectors in `vec` (2n doubles) and two words at `scal`.
 int premise_norm(int n, const double* E, double* vec, double* scal, double* out, cudaStream_t s) {
-  double* x = vec;
-  double* y = vec + n;
-  pow_init<<<(n + 255) / 256, 256, 0, s>>>(x, n);
-  mpj_count_launch();
-  pow_norm<<<1, 256, 0, s>>>(x, n, scal);
-  mpj_count_launch();
-  for (int it = 0; it < 30; ++it) {
-    pow_step<<<(n + 7) / 8, 256, 0, s>>>(E, n, x, scal, y);
+  if (n <= POW_SMALL) {
+    pow_cluster<<<POW_CTAS, 256, 0, s>>>(E, n, scal);
     mpj_count_launch();
-    pow_norm<<<1, 256, 0, s>>>(y, n, scal);
-    mpj_count_launch();
-    double* t = x;
-    x = y;
-    y = t;
+    MPJ_CUDA_TRY(cudaGetLastError());
+  } else {
+    double* x = vec;
+    double* y = vec + n;
+    unsigned* ticket = (unsigned*)(scal + 1);
+    MPJ_CUDA_TRY(cudaMemsetAsync(ticket, 0, sizeof(unsigned), s));
+    for (int it = -1; it < POW_STEPS; ++it) {
+      MPJ_CUDA_TRY(mpj_launch_pdl(pow_step, dim3((n + 7) / 8), dim3(256), 0, s, E, n, (const double*)x, scal, y, ticket,
+                                  it));
+      double* t = x;
+      x = y;
+      y = t;
+    }
   }
-  MPJ_CUDA_TRY(cudaGetLastError());
   MPJ_CUDA_TRY(cudaMemcpyAsync(out, scal, sizeof(double), cudaMemcpyDeviceToHost, s));
   MPJ_CUDA_TRY(cudaStreamSynchronize(s));
   return MPJ_OK;
