@@ -150,14 +150,15 @@ size_t mpj_syev_workspace(int n, const mpj_opts* o);
 /* Mixed precision symmetric eigensolver (Alg. 9), default options.
  * A_dev: n x n input, read only.  W_dev: n eigenvalues (ascending).
  * Q_dev: n x n eigenvectors, ldq = n.  tol <= 0 selects n 2^-53 ||A||_F.
- * Allocates its workspace with cudaMallocAsync on `stream` and frees it before
- * returning; synchronizes `stream`.  Returns MPJ_OK, MPJ_NOT_CONVERGED, or an
+ * Allocates its workspace on `stream` from the library's memory pool (which
+ * keeps up to 2 GB of freed memory per device between calls, see
+ * mpj_release_plans) and frees it before returning; synchronizes `stream`.  Returns MPJ_OK, MPJ_NOT_CONVERGED, or an
  * error code. */
 int mpj_syev(int n, const double* A_dev, int lda, double* W_dev, double* Q_dev, double tol, void* stream);
 
 /* Same with explicit options, output leading dimension, optional host `info`
  * (may be NULL) and optional caller workspace (work_dev may be NULL: then the
- * library allocates it with cudaMallocAsync and frees it before returning;
+ * library allocates it from its memory pool and frees it before returning;
  * else work_bytes >= mpj_syev_workspace(n, o) and the call allocates nothing:
  * every buffer, including the sliced operands of the tensor-core products,
  * is carved from work_dev).  Synchronizes `stream` once per sweep (to read
@@ -192,7 +193,8 @@ int mpj_syev_ex(int n, const double* A_dev, int lda, double* W_dev, double* Q_de
 int mpj_syev_batched(int batch, const int* n_host, const double* const* A_dev, double* const* W_dev,
                      double* const* Q_dev, double tol, int* sweeps_host, void* stream);
 
-/* Frees the workspaces and graphs of all cached batched plans. */
+/* Frees the workspaces and graphs of all cached batched plans and returns the
+ * memory that the library's pools keep between calls. */
 void mpj_release_plans(void);
 
 /* The autotuned thread-group size recorded for this batch's size histogram
@@ -225,7 +227,7 @@ int mpj_newton_schulz(int n, double* X_dev, int ldx, int steps, void* stream);
 /* Preconditioning: Ac = Qd^T A Qd (Alg. 9 step 3); Ac is written exactly
  * symmetric (lower triangle mirrored).  Products as in the solve: the
  * tensor-core exact-slice engine unless MPJ_GEMM_TC=0 selects the FP64 DMMA
- * kernel.  Allocates its scratch with cudaMallocAsync; synchronizes. */
+ * kernel.  Allocates its scratch from the memory pool; synchronizes. */
 int mpj_precondition(int n, const double* A_dev, int lda, const double* Qd_dev, int ldq, double* Ac_dev, int ldc,
                      void* stream);
 
@@ -293,7 +295,7 @@ int mpj_dgemm(char transa, char transb, int m, int n, int k, double alpha, const
  * in one step (no intermediate underflow).  The error is within a small
  * multiple of 2^-53 (|op(A)| |op(B)|)_rc plus k 2^-54 max|op(A)(r,:)|
  * max|op(B)(:,c)| per entry.  Allocates about 16 (m + n) k bytes of scratch
- * with cudaMallocAsync; synchronizes the stream.  Returns MPJ_EINVAL,
+ * from the memory pool; synchronizes the stream.  Returns MPJ_EINVAL,
  * MPJ_ENOMEM, MPJ_ETIMEOUT (the tensor cores did not signal completion within
  * about 2 s) or MPJ_ECUDA on failure. */
 int mpj_dgemm_tc(char transa, char transb, int m, int n, int k, double alpha, const double* A_dev, int lda,

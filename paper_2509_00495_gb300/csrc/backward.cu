@@ -100,7 +100,7 @@ extern "C" int mpj_syev_backward(int batch, int n, const double* W, const double
   }
   void* w = nullptr;
   size_t bytes = ((2 * (size_t)batch * sq * sizeof(double) + 255) & ~(size_t)255) + 512 + 2 * ob * (size_t)(tc ? group : 0);
-  if (cudaMallocAsync(&w, bytes, s) != cudaSuccess) return MPJ_ENOMEM;
+  if (mpj_alloc_async(&w, bytes, s) != cudaSuccess) return MPJ_ENOMEM;
   mpj_count_alloc();
   double* M = (double*)w;
   double* T = M + (size_t)batch * sq;

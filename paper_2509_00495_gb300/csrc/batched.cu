@@ -633,6 +633,7 @@ cudaError_t enqueue(const Plan* p, const Layout& L, const double* const* A, doub
 }  // namespace
 
 extern "C" void mpj_release_plans(void) {
+  mpj_release_pools();
   mpj_batched_rounds_release();
   std::lock_guard<std::mutex> lock(g_mu);
   for (Plan* p : g_plans) free_plan(p);

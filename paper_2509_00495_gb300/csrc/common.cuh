@@ -242,3 +242,8 @@ bool mpj_v_overlap_enabled();
 // Counts every device (or pinned host) allocation the library makes
 // (diagnostic, mpj_device_allocations).
 void mpj_count_alloc();
+
+// Stream-ordered allocation from the library's own memory pool of the current
+// device (freed with cudaFreeAsync), and giving back what the pools hold.
+cudaError_t mpj_alloc_async(void** p, size_t bytes, cudaStream_t s);
+void mpj_release_pools();

@@ -721,7 +721,7 @@ extern "C" int mpj_dgemm_tc(char transa, char transb, int m, int n, int k, doubl
   const size_t ba = mpj_oz_operand_bytes(m, k), bb = mpj_oz_operand_bytes(n, k);
   const size_t bytes = ba + bb + 256;
   char* w = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&w, bytes, s);
+  cudaError_t e = mpj_alloc_async((void**)&w, bytes, s);
   mpj_count_alloc();
   if (e != cudaSuccess) {
     mpj_set_cuda_error(e, "mpj_dgemm_tc workspace", __LINE__);
