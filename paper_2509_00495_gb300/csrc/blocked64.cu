@@ -252,22 +252,6 @@ MPJ_DEV Df2 df2_rot(const RotC& r, const Df2& x, const Df2& y) {
   return o;
 }
 
-MPJ_DEV float rcp_ftz(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-MPJ_DEV float rsqrt_ftz(float x) {
-  float r;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-MPJ_DEV float sqrt_ftz(float x) {
-  float r;
-  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-
 // Algorithm 2 on FP32 pairs for the slot's indices (x, y): coupling a, d =
 // a_yy - a_xx, giving t (the root of a t^2 + d t - a with |t| <= 1, the sign of
 // `tie` for d = 0), c = 1 / sqrt(1 + t^2) and s = t c.  From an FP32 seed t0,

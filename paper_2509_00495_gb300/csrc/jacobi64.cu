@@ -542,36 +542,6 @@ __global__ void check_symmetric(const double* __restrict__ A, int lda, int n, un
 // pair's own 2 x 2 block (J^T B J) is stored with its two off-diagonal values
 // averaged, which is what the paper's end-of-sweep symmetrization does.
 
-struct WaveRec {
-  double c, s;
-  int rot;
-  int pad;
-};
-
-// Rotation parameters of the wavefront's pairs (skip rule of Algorithm 4).
-__global__ void cyc_wave_params(const double* __restrict__ A, int lda, int n, int t, int plo, int k, double skip,
-                                double skip_abs, WaveRec* __restrict__ rec, int* __restrict__ rotated) {
-  const int kp = blockIdx.x * blockDim.x + threadIdx.x;
-  if (kp >= k) return;
-  const int p = plo + kp, q = t - p;
-  const double app = A[(size_t)p * lda + p], aqq = A[(size_t)q * lda + q], apq = A[(size_t)p * lda + q];
-  WaveRec r;
-  r.c = 1.0;
-  r.s = 0.0;
-  r.rot = 0;
-  r.pad = 0;
-  if (fabs(apq) > skip * sqrt(fabs(app * aqq)) && fabs(apq) > skip_abs) {
-    // Algorithm 2, stable form (Appendix A approach 2)
-    const double tau = (aqq - app) / (2.0 * apq);
-    const double tt = tau >= 0.0 ? 1.0 / (tau + sqrt(1.0 + tau * tau)) : 1.0 / (tau - sqrt(1.0 + tau * tau));
-    r.c = 1.0 / sqrt(1.0 + tt * tt);
-    r.s = tt * r.c;
-    r.rot = 1;
-    *rotated = 1;
-  }
-  rec[kp] = r;
-}
-
 // new (x_p, x_q) = (c x_p - s x_q, s x_p + c x_q): the row update J^T x and
 // the column / vector update x J of Sec. 3.2.2 have the same form.
 MPJ_DEV void jrot(double c, double s, double& xp, double& xq) {
@@ -580,23 +550,145 @@ MPJ_DEV void jrot(double c, double s, double& xp, double& xq) {
   xq = nq;
 }
 
-// One wavefront: CTA (chunk, kp) owns columns p, q of pair kp (rows
-// j in its chunk) and of V.  Rows j outside the wavefront get the column
-// update and its mirror (rows p, q of column j).  Rows of another pair kj of
-// the wavefront: the thread of that pair's first index computes the whole
-// 2 x 2 block of rows (p_j, q_j) in columns (p, q) in the canonical order
-// (lower pair index first); the other pair's CTA computes the mirror block
-// from the same operands in the same order.  Nothing a CTA reads is written
-// by another CTA of the same launch.
-__global__ void __launch_bounds__(256) cyc_wave_update(double* __restrict__ A, int lda, double* __restrict__ V,
-                                                       int ldv, int n, int t, int plo, int phi,
-                                                       const WaveRec* __restrict__ rec) {
-  const int kp = blockIdx.y;
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+// A pair of a wavefront: its rotation, its entries before it, and whether it rotates.
+struct WaveRec {
+  double c, s, app, aqq, apq;
+  int rot, pad;
+};
+
+// Rotation of a pair from its entries (skip rule of Algorithm 4, compared in squares).
+MPJ_DEV WaveRec wave_rec(double app, double aqq, double apq, double skip, double skip_abs, int* __restrict__ rotated) {
+  WaveRec r;
+  r.c = 1.0;
+  r.s = 0.0;
+  r.app = app;
+  r.aqq = aqq;
+  r.apq = apq;
+  r.rot = 0;
+  r.pad = 0;
+  if (apq * apq > (skip * skip) * fabs(app * aqq) && fabs(apq) > skip_abs) {
+    double t;
+    jacobi_angle(aqq - app, apq, t, r.c);
+    r.s = t * r.c;
+    r.rot = 1;
+    *rotated = 1;
+  }
+  return r;
+}
+
+// A pair's own block after its rotation: rows (J^T B), then columns (.. J), the
+// two off-diagonal values averaged.
+MPJ_DEV void wave_block(const WaveRec& r, double& npp, double& nqq, double& off) {
+  npp = r.app;
+  nqq = r.aqq;
+  off = r.apq;
+  if (!r.rot) return;
+  double bqp = r.apq, bpq = r.apq;
+  jrot(r.c, r.s, npp, bqp);  // column p of B: rows p, q
+  jrot(r.c, r.s, bpq, nqq);  // column q of B
+  jrot(r.c, r.s, npp, bpq);  // row p: columns p, q
+  jrot(r.c, r.s, bqp, nqq);  // row q
+  off = 0.5 * (bpq + bqp);
+}
+
+// Row j and pair kp of wavefront t.  The pair's thread group owns columns p, q
+// of A and of V.  Rows j outside the wavefront get the column update and
+// its mirror (rows p, q of column j).  Rows of another pair kj of the wavefront:
+// the thread of that pair's first index computes the whole 2 x 2 block of rows
+// (p_j, q_j) in columns (p, q) in the canonical order (lower pair index first);
+// the thread group of the other pair computes the mirror block from the same
+// operands in the same order.  Nothing that is read is written by another
+// thread group in the same wavefront.
+//
+// The next wavefront's records are formed here as well.  Its pair (p, t + 1 - p)
+// has p in this wavefront's pair (p, t - p) and t + 1 - p in the pair (p - 1,
+// t + 1 - p), so the new coupling is one entry of the block between the two,
+// held by one thread, and the new diagonal follows from the two records.  Two
+// pairs have an index outside this wavefront: (0, t + 1) while t + 1 < n, and
+// (t/2, t/2 + 1) for even t.
+MPJ_DEV void wave_row(double* A, int lda, double* V, int ldv, int n, int t, int plo, int phi, int kp, int j, double skip,
+                      double skip_abs, const WaveRec* rec, WaveRec* next, int* rotated) {
   const WaveRec ra = rec[kp];
   const int p = plo + kp, q = t - p;
-  if (j >= n) return;
   const size_t cp = (size_t)p * lda, cq = (size_t)q * lda;
+  const int plo2 = t + 1 - (n - 1) > 0 ? t + 1 - (n - 1) : 0;
+  const bool more = t < 2 * n - 3;
+  const int qlo = t - phi;
+  const bool in_p = j >= plo && j <= phi;
+  const bool in_q = j >= qlo && j <= t - plo;
+  if (!in_p && !in_q) {
+    const bool first = more && p == 0 && j == t + 1;         // next pair (0, t + 1)
+    const bool middle = more && 2 * j == t && kp == phi - plo;  // next pair (t/2, t/2 + 1)
+    if (ra.rot || first || middle) {
+      double xp = A[cp + j], xq = A[cq + j];
+      if (ra.rot) {
+        jrot(ra.c, ra.s, xp, xq);
+        A[cp + j] = xp;
+        A[cq + j] = xq;
+        A[(size_t)j * lda + p] = xp;
+        A[(size_t)j * lda + q] = xq;
+      }
+      if (first || middle) {
+        const double ajj = A[(size_t)j * lda + j];  // not touched by this wavefront
+        double npp, nqq, off;
+        wave_block(ra, npp, nqq, off);
+        if (first) next[0 - plo2] = wave_rec(npp, ajj, xp, skip, skip_abs, rotated);
+        if (middle) next[j - plo2] = wave_rec(ajj, nqq, xq, skip, skip_abs, rotated);
+      }
+    }
+  } else if (in_p) {  // rows of a pair are handled by the thread of its first index
+    const int kj = j - plo;
+    const int pj = j, qj = t - j;
+    const WaveRec rb = rec[kj];
+    if (kj == kp) {
+      if (ra.rot) {
+        double npp, nqq, off;
+        wave_block(ra, npp, nqq, off);
+        A[cp + p] = npp;
+        A[cq + q] = nqq;
+        A[cp + q] = off;
+        A[cq + p] = off;
+      }
+    } else {
+      const bool ahead = more && kj == kp - 1 && p >= plo2;  // next pair (p, q_j), q_j = t + 1 - p
+      if (ra.rot || rb.rot || ahead) {
+        // rows (pj, qj) x columns (p, q): B(r, c) = A[row + col * lda]
+        double b00 = A[cp + pj], b10 = A[cp + qj];
+        double b01 = A[cq + pj], b11 = A[cq + qj];
+        if (ra.rot || rb.rot) {
+          if (kj < kp) {
+            // T = (J_kj^T B) J_kp, stored as is
+            jrot(rb.c, rb.s, b00, b10);  // rows pj, qj of column p
+            jrot(rb.c, rb.s, b01, b11);  // of column q
+            jrot(ra.c, ra.s, b00, b01);  // columns p, q of row pj
+            jrot(ra.c, ra.s, b10, b11);  // of row qj
+          } else {
+            // canonical order with kp first: T' = (J_kp^T B^T) J_kj, stored transposed;
+            // B^T(r', c') has rows (p, q), columns (pj, qj): B^T = [b00 b10; b01 b11]
+            double t00 = b00, t01 = b10, t10 = b01, t11 = b11;
+            jrot(ra.c, ra.s, t00, t10);  // rows p, q of column pj
+            jrot(ra.c, ra.s, t01, t11);  // of column qj
+            jrot(rb.c, rb.s, t00, t01);  // columns pj, qj of row p
+            jrot(rb.c, rb.s, t10, t11);  // of row q
+            b00 = t00;
+            b10 = t01;
+            b01 = t10;
+            b11 = t11;
+          }
+          A[cp + pj] = b00;
+          A[cp + qj] = b10;
+          A[cq + pj] = b01;
+          A[cq + qj] = b11;
+        }
+        if (ahead) {
+          double npp, nqq, off, mpp, mqq;
+          wave_block(ra, npp, nqq, off);
+          wave_block(rb, mpp, mqq, off);
+          next[p - plo2] = wave_rec(npp, mqq, b10, skip, skip_abs, rotated);
+        }
+      }
+    }
+  }
   // vectors: V(:, [p q]) = V(:, [p q]) J
   if (ra.rot) {
     double vp = V[(size_t)p * ldv + j], vq = V[(size_t)q * ldv + j];
@@ -604,64 +696,25 @@ __global__ void __launch_bounds__(256) cyc_wave_update(double* __restrict__ A, i
     V[(size_t)p * ldv + j] = vp;
     V[(size_t)q * ldv + j] = vq;
   }
-  const int qlo = t - phi;
-  const bool in_p = j >= plo && j <= phi;
-  const bool in_q = j >= qlo && j <= t - plo;
-  if (!in_p && !in_q) {
-    if (!ra.rot) return;
-    double xp = A[cp + j], xq = A[cq + j];
-    jrot(ra.c, ra.s, xp, xq);
-    A[cp + j] = xp;
-    A[cq + j] = xq;
-    A[(size_t)j * lda + p] = xp;
-    A[(size_t)j * lda + q] = xq;
-    return;
-  }
-  if (in_q) return;  // rows of a pair are handled by the thread of its first index
-  const int kj = j - plo;
-  const int pj = j, qj = t - j;
-  const WaveRec rb = rec[kj];
-  if (kj == kp) {
-    if (!ra.rot) return;
-    // own block: rows (J^T B), then columns (.. J)
-    double bpp = A[cp + p], bqp = A[cp + q], bpq = A[cq + p], bqq = A[cq + q];
-    jrot(ra.c, ra.s, bpp, bqp);  // column p of B: rows p, q
-    jrot(ra.c, ra.s, bpq, bqq);  // column q of B
-    jrot(ra.c, ra.s, bpp, bpq);  // row p: columns p, q
-    jrot(ra.c, ra.s, bqp, bqq);  // row q
-    const double off = 0.5 * (bpq + bqp);
-    A[cp + p] = bpp;
-    A[cq + q] = bqq;
-    A[cp + q] = off;
-    A[cq + p] = off;
-    return;
-  }
-  if (!ra.rot && !rb.rot) return;
-  // rows (pj, qj) x columns (p, q): B(r, c) = A[row + col * lda]
-  double b00 = A[cp + pj], b10 = A[cp + qj], b01 = A[cq + pj], b11 = A[cq + qj];
-  if (kj < kp) {
-    // T = (J_kj^T B) J_kp, stored as is
-    jrot(rb.c, rb.s, b00, b10);  // rows pj, qj of column p
-    jrot(rb.c, rb.s, b01, b11);  // of column q
-    jrot(ra.c, ra.s, b00, b01);  // columns p, q of row pj
-    jrot(ra.c, ra.s, b10, b11);  // of row qj
-  } else {
-    // canonical order with kp first: T' = (J_kp^T B^T) J_kj, stored transposed;
-    // B^T(r', c') has rows (p, q), columns (pj, qj): B^T = [b00 b10; b01 b11]
-    double t00 = b00, t01 = b10, t10 = b01, t11 = b11;
-    jrot(ra.c, ra.s, t00, t10);  // rows p, q of column pj
-    jrot(ra.c, ra.s, t01, t11);  // of column qj
-    jrot(rb.c, rb.s, t00, t01);  // columns pj, qj of row p
-    jrot(rb.c, rb.s, t10, t11);  // of row q
-    b00 = t00;
-    b10 = t01;
-    b01 = t10;
-    b11 = t11;
-  }
-  A[cp + pj] = b00;
-  A[cp + qj] = b10;
-  A[cq + pj] = b01;
-  A[cq + qj] = b11;
+}
+
+// One launch per wavefront (thread group = CTA), after cyc_first.  What bounds a
+// wavefront is its chain of loads, update and next angle on a contended FP64
+// pipe.  n = 300, per wavefront: 13.4 us with the records in a launch of their
+// own, divisions and square roots in their chain; 7.3 us in this form.  (One
+// cooperative launch per sweep with a grid barrier between the wavefronts took
+// the same time, and 1.4 times as long at n = 2000.)
+constexpr int CYC_ROWS = 128;  // rows per thread group
+__global__ void cyc_first(const double* __restrict__ A, int lda, double skip, double skip_abs, WaveRec* __restrict__ rec,
+                          int* __restrict__ rotated) {
+  rec[0] = wave_rec(A[0], A[(size_t)lda + 1], A[1], skip, skip_abs, rotated);
+}
+__global__ void __launch_bounds__(CYC_ROWS) cyc_wave(double* A, int lda, double* V, int ldv, int n, int t, int plo,
+                                                     int phi, double skip, double skip_abs, const WaveRec* rec,
+                                                     WaveRec* next, int* rotated) {
+  pdl_wait();
+  const int j = blockIdx.x * CYC_ROWS + threadIdx.x;
+  if (j < n) wave_row(A, lda, V, ldv, n, t, plo, phi, blockIdx.y, j, skip, skip_abs, rec, next, rotated);
 }
 
 }  // namespace
@@ -929,17 +982,17 @@ int mpj_jacobi64_run(int n, double* A, int lda, double* V, int ldv, double tol, 
         status = MPJ_NOT_CONVERGED;
         break;
       }
-      // one sweep = 2n - 3 wavefronts; the rotation records use the record area
-      WaveRec* wrec = reinterpret_cast<WaveRec*>(rec[0]);
+      // one sweep = 2n - 3 wavefronts; their records alternate between the two record areas
+      WaveRec *wrec0 = reinterpret_cast<WaveRec*>(rec[0]), *wrec1 = reinterpret_cast<WaveRec*>(rec[1]);
       MPJ_CUDA_TRY(cudaMemsetAsync(iscal, 0, sizeof(int), s));
+      cyc_first<<<1, 1, 0, s>>>(A, lda, skip, skip_abs, wrec1, iscal);
+      mpj_count_launch();
+      MPJ_CUDA_TRY(cudaGetLastError());
       for (int t = 1; t <= 2 * n - 3; ++t) {
-        const int plo = t - (n - 1) > 0 ? t - (n - 1) : 0;
-        const int phi = (t - 1) / 2;
-        const int k = phi - plo + 1;
-        cyc_wave_params<<<(k + 127) / 128, 128, 0, s>>>(A, lda, n, t, plo, k, skip, skip_abs, wrec, iscal);
-        mpj_count_launch();
-        cyc_wave_update<<<dim3((n + 255) / 256, k), 256, 0, s>>>(A, lda, V, ldv, n, t, plo, phi, wrec);
-        mpj_count_launch();
+        const int plo = t - (n - 1) > 0 ? t - (n - 1) : 0, phi = (t - 1) / 2;
+        MPJ_CUDA_TRY(mpj_launch_pdl(cyc_wave, dim3((n + CYC_ROWS - 1) / CYC_ROWS, phi - plo + 1), dim3(CYC_ROWS), 0, s, A,
+                                    lda, V, ldv, n, t, plo, phi, skip, skip_abs, (const WaveRec*)(t & 1 ? wrec1 : wrec0),
+                                    t & 1 ? wrec0 : wrec1, iscal));
       }
       MPJ_CUDA_TRY(cudaGetLastError());
       int rotated = 0;

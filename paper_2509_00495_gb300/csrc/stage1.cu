@@ -83,16 +83,6 @@ __global__ void widen(const float* __restrict__ V32, int N, int n, double* __res
 struct Rot32 {
   float cm1, sig;
 };
-MPJ_DEV float rcp_ftz(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-MPJ_DEV float rsqrt_ftz(float x) {
-  float r;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
 MPJ_DEV bool rot32(float& app, float& aqq, float apq, float skip, Rot32& rr) {
   const bool rot = apq * apq > (skip * skip) * fabsf(app * aqq);
   const float tau = (aqq - app) * rcp_ftz(2.0f * apq), at = fminf(fabsf(tau), 1e18f);
