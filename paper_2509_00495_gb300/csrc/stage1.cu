@@ -46,6 +46,19 @@ MPJ_DEV void block_pair(int nb, int R, int slot, int& I, int& J) {
   J = x < y ? y : x;
 }
 
+// Where the two blocks of pair `slot` of round R >= 1 were in round R - 1: slots
+// a (of the lower block) and q, and the blocks' offsets in those pairs.
+MPJ_DEV void prev_slots(int nb, int R, int slot, int& a, int& oa, int& q, int& oq) {
+  int I, J, y, lo, hi;
+  block_pair(nb, R, slot, I, J);
+  rr_slot_of(nb, R - 1, I, a, y);
+  block_pair(nb, R - 1, a, lo, hi);
+  oa = I == hi ? BS : 0;
+  rr_slot_of(nb, R - 1, J, q, y);
+  block_pair(nb, R - 1, q, lo, hi);
+  oq = J == hi ? BS : 0;
+}
+
 // hq: the half-precision stage (binary16 values; Ch. 6 further work item 3):
 // every stored value and rotation parameter is rounded to binary16.
 MPJ_DEV float qh(float v, bool hq) { return hq ? __half2float(__float2half_rn(v)) : v; }
@@ -137,14 +150,17 @@ struct Sub32 {
   int N, nb, slot;
   float *S, *U;
   unsigned* M;
+  const float *Sp, *Up, *T;  // looking ahead: S and U of the previous round's pairs, this pair's saved tile
 };
 struct OneSub32 {  // the block pairs of one matrix
   const float* A;
   int N, nb;
   float *S, *U;
   unsigned* M;
+  const float *Sp, *Up, *T;
   MPJ_DEV bool get(int bid, Sub32& v) const {
-    v = Sub32{A, N, nb, bid, S + (size_t)bid * W2 * W2, U + (size_t)bid * W2 * W2, M ? M + bid : nullptr};
+    v = Sub32{A, N, nb, bid, S + (size_t)bid * W2 * W2, U + (size_t)bid * W2 * W2, M ? M + bid : nullptr,
+              Sp, Up, T + (size_t)bid * W2 * W2};
     return true;
   }
 };
@@ -157,7 +173,7 @@ struct BatchSub32 {  // the block pairs of a batch
     BatchTask t;
     if (!batch_find(b, lo, bid, [](int np) { return np; }, t)) return false;
     const size_t o = (size_t)(t.pair0 + t.local) * W2 * W2;
-    v = Sub32{A + t.el, t.N, t.N / BS, t.local, S + o, U + o, nullptr};
+    v = Sub32{A + t.el, t.N, t.N / BS, t.local, S + o, U + o, nullptr, nullptr, nullptr, nullptr};
     return true;
   }
 };
@@ -171,6 +187,7 @@ __global__ void __launch_bounds__(S32_THREADS, 1) solve32(Src src, int R, bool u
   __shared__ float S[2][W2 * SLD];
   __shared__ float U[W2][LD];  // U[column][row]
   __shared__ float dg[W2];     // the diagonal (warp 0 only)
+  __shared__ float Uh[2][W2][BS];  // looking ahead: the halves of U_a and U_q
   __shared__ Rot32 rec[2][W2 / 2];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   pdl_wait();
@@ -179,14 +196,58 @@ __global__ void __launch_bounds__(S32_THREADS, 1) solve32(Src src, int R, bool u
   int I, J;
   block_pair(sub.nb, R, sub.slot, I, J);
   unsigned* const Mbuf = sub.M;
-  for (int e = tid; e < W2 * W2; e += S32_THREADS) {
-    const int li = e % W2, lj = e / W2;
-    const float v = sub.A[(size_t)gidx(I, J, lj) * sub.N + gidx(I, J, li)];
-    if (li == lj)
-      dg[li] = v;
-    else if (li < lj)
-      S[0][(li ^ lj) * SLD + li] = v;
-    U[lj][li] = (li == lj) ? 1.0f : 0.0f;
+  if (sub.Sp) {
+    // the subproblem before A has received the previous round's update: its two
+    // diagonal blocks are blocks of that round's solved subproblems, its
+    // coupling block is U_a^T T U_q on the tile T between their pairs
+    int a, oa, q, oq;
+    prev_slots(sub.nb, R, sub.slot, a, oa, q, oq);
+    const float *Sa = sub.Sp + (size_t)a * W2 * W2, *Sq = sub.Sp + (size_t)q * W2 * W2;
+    const float *Ua = sub.Up + (size_t)a * W2 * W2, *Uq = sub.Up + (size_t)q * W2 * W2;
+    float(*Ts)[LD] = reinterpret_cast<float(*)[LD]>(S[1]);  // T(r, k) at [k][r]
+    for (int e = tid; e < W2 * W2; e += S32_THREADS) {
+      const int li = e % W2, lj = e / W2;
+      Ts[lj][li] = sub.T[e];
+      if (li <= lj && (lj < BS || li >= BS)) {
+        const float v = lj < BS ? Sa[(oa + lj) * W2 + oa + li] : Sq[(oq + lj - BS) * W2 + oq + li - BS];
+        if (li == lj)
+          dg[li] = v;
+        else
+          S[0][(li ^ lj) * SLD + li] = v;
+      }
+      if (e < W2 * BS) {
+        const int k = e / BS, c = e % BS;
+        Uh[0][k][c] = Ua[k * W2 + oa + c];
+        Uh[1][k][c] = Uq[k * W2 + oq + c];
+      }
+    }
+    __syncthreads();
+    if (tid < W2 * BS) {  // T U_q, into U's place as [column][row]
+      float acc = 0.0f;
+#pragma unroll 8
+      for (int k = 0; k < W2; ++k) acc = fmaf(Ts[k][lane], Uh[1][k][warp], acc);
+      U[warp][lane] = acc;
+    }
+    __syncthreads();
+    if (tid < BS * BS) {
+      const int i = tid % BS, j = tid / BS;
+      float acc = 0.0f;
+#pragma unroll 8
+      for (int r = 0; r < W2; ++r) acc = fmaf(Uh[0][r][i], U[j][r], acc);
+      S[0][(i ^ (BS + j)) * SLD + i] = qh(acc, HQ);
+    }
+    __syncthreads();
+    for (int e = tid; e < W2 * W2; e += S32_THREADS) U[e / W2][e % W2] = (e % W2 == e / W2) ? 1.0f : 0.0f;
+  } else {
+    for (int e = tid; e < W2 * W2; e += S32_THREADS) {
+      const int li = e % W2, lj = e / W2;
+      const float v = sub.A[(size_t)gidx(I, J, lj) * sub.N + gidx(I, J, li)];
+      if (li == lj)
+        dg[li] = v;
+      else if (li < lj)
+        S[0][(li ^ lj) * SLD + li] = v;
+      U[lj][li] = (li == lj) ? 1.0f : 0.0f;
+    }
   }
   __syncthreads();
   const float skip = HQ ? 0x1p-11f : 0x1p-24f;
@@ -304,6 +365,19 @@ __global__ void __launch_bounds__(S32_THREADS, 1) solve32(Src src, int R, bool u
   }
 }
 
+
+// Saves, for every pair of round R >= 1, the 32 x 32 tile of A between the pairs
+// of round R - 1 that held its two blocks (rows of the lower block's pair).
+__global__ void __launch_bounds__(256) snap32(const float* __restrict__ A32, int N, int nb, int R, float* __restrict__ T) {
+  pdl_wait();
+  int a, oa, q, oq, Ia, Ja, Iq, Jq;
+  prev_slots(nb, R, blockIdx.x, a, oa, q, oq);
+  block_pair(nb, R - 1, a, Ia, Ja);
+  block_pair(nb, R - 1, q, Iq, Jq);
+  float* t = T + (size_t)blockIdx.x * W2 * W2;
+  for (int e = threadIdx.x; e < W2 * W2; e += 256)
+    t[e] = A32[(size_t)gidx(Iq, Jq, e / W2) * N + gidx(Ia, Ja, e % W2)];
+}
 
 // Packed pairs of FP32 values (low word first) and the paired FMA
 // d = a * b + d, each half rounded to nearest like fmaf.
@@ -591,14 +665,14 @@ cudaError_t mpj_batch_stage1_round(const BatchShape& b, int R, float* A32, float
 int mpj_stage1_padded(int n) { return ((n + W2 - 1) / W2) * W2; }
 
 // A32, V32, two sets of the per-pair S and U (alternate rounds), the
-// tensor-core update's transposed intermediate B^T, a flag word and two sets
-// of the per-pair rotated-index masks.
+// tensor-core update's transposed intermediate B^T, a flag word, two sets of
+// the per-pair rotated-index masks, two of the saved tiles.
 static int stage1_tensor_cores();
 
 size_t mpj_stage1_bytes(int n) {
   size_t N = (size_t)mpj_stage1_padded(n);
   size_t nb = N / BS;
-  return 3 * N * N * sizeof(float) + 4 * (nb / 2) * W2 * W2 * sizeof(float) + 4096 + 2 * (nb / 2) * sizeof(unsigned);
+  return 3 * N * N * sizeof(float) + 6 * (nb / 2) * W2 * W2 * sizeof(float) + 4096 + 2 * (nb / 2) * sizeof(unsigned);
 }
 
 // MPJ_STAGE1_TC=1 runs the A update of each block round on the tcgen05
@@ -621,14 +695,22 @@ cudaError_t mpj_sumsq32(const float* A, int lda, int n, double* partial, double*
 
 
 namespace {
-// One stage-1 sweep (nb - 1 block rounds) enqueued on stream s.  V <- V U~ of
-// round R runs on the side stream (when given), overlapping round R + 1's
-// subproblems; the S/U sets alternate between rounds, round R + 2's
-// subproblems wait for round R's V update before overwriting its set, and
-// the side stream is joined into s at the end of the sweep.
+// One stage-1 sweep (nb - 1 block rounds) enqueued on stream s.
+//
+// The subproblems of round R + 1 do not wait for round R's update of A: their
+// diagonal blocks come from round R's solved subproblems and their coupling
+// blocks from tiles of A saved before that update (snap32).  So the chain of a
+// sweep is the subproblems alone; A's updates (with the saving of tiles) and
+// V's run on two side streams (when given), two rounds behind at most: round
+// R's subproblems wait for the tiles saved after round R - 2's update, which
+// also frees the S, U and T sets that alternate between rounds, and for V's
+// update of round R - 2.  Both streams are joined into s at the end.  Before, a
+// round was the subproblems, then A's update: n = 96 25 us a round, now 20;
+// n = 300 20.6, now 18; n = 1024 20.0, now 19.3 (there the updates, sharing SMs
+// with the subproblems, take turns with them: the subproblems alone run at 12.5).
 struct Stage1Bufs {
   int N, nb;
-  float *A32, *V32, *Sb[2], *Ub[2], *Bt;
+  float *A32, *V32, *Sb[2], *Ub[2], *Tb[2], *Bt;
   unsigned* tflag;
   unsigned* Mb[2];  // per-pair rotated-index masks, by round parity
   bool half;
@@ -636,36 +718,70 @@ struct Stage1Bufs {
   int tc;
 };
 
-cudaError_t stage1_sweep(const Stage1Bufs& b, cudaStream_t s, SideStream* side) {
-  const int N = b.N, nb = b.nb, npairs = nb / 2;
+// The side streams and events of a sweep; joined into the owner stream on every
+// exit (owner = null: the caller has joined them, e.g. inside a captured graph).
+struct SweepStreams {
+  cudaStream_t owner = nullptr, sa = nullptr, sv = nullptr;
+  cudaEvent_t solved[2] = {nullptr, nullptr}, a[2] = {nullptr, nullptr}, v[2] = {nullptr, nullptr};
+  bool ok = true;
+  explicit SweepStreams(cudaStream_t s) : owner(s) {
+    ok = cudaStreamCreateWithFlags(&sa, cudaStreamNonBlocking) == cudaSuccess &&
+         cudaStreamCreateWithFlags(&sv, cudaStreamNonBlocking) == cudaSuccess;
+    for (cudaEvent_t* e : {&solved[0], &solved[1], &a[0], &a[1], &v[0], &v[1]})
+      ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) (void)cudaGetLastError();
+  }
+  ~SweepStreams() {
+    if (ok && owner) {
+      if (cudaEventRecord(a[0], sa) == cudaSuccess) (void)cudaStreamWaitEvent(owner, a[0], 0);
+      if (cudaEventRecord(v[0], sv) == cudaSuccess) (void)cudaStreamWaitEvent(owner, v[0], 0);
+    }
+    for (cudaEvent_t e : {solved[0], solved[1], a[0], a[1], v[0], v[1]})
+      if (e) cudaEventDestroy(e);
+    if (sv) cudaStreamDestroy(sv);
+    if (sa) cudaStreamDestroy(sa);
+  }
+};
+
+// Kernels of one sweep.
+long long stage1_sweep_launches(const Stage1Bufs& b) {
+  const long long rounds = b.nb - 1;
+  return b.tc == 1 ? 4 * rounds : 3 * rounds + (rounds - 1);
+}
+
+cudaError_t stage1_sweep(const Stage1Bufs& b, cudaStream_t s, SweepStreams* side) {
+  const int N = b.N, nb = b.nb, npairs = nb / 2, rounds = nb - 1;
   const dim3 g32((npairs + 3) / 4, npairs);
-  bool vpending[2] = {false, false};
+  const bool look = b.tc != 1;  // the tensor-core update transposes through Bt, in order
+  cudaStream_t sa = side ? side->sa : s, sv = side ? side->sv : s;
   cudaError_t e = cudaSuccess;
 #define S1_TRY(x)                    \
   do {                               \
     e = (x);                         \
     if (e != cudaSuccess) return e;  \
   } while (0)
-  for (int R = 0; R < nb - 1; ++R) {
+  auto snap = [&](int R, cudaStream_t st) {
+    return mpj_launch_pdl(snap32, dim3(npairs), dim3(256), 0, st, (const float*)b.A32, N, nb, R, b.Tb[R & 1]);
+  };
+  if (look && rounds > 1) S1_TRY(snap(1, s));
+  for (int R = 0; R < rounds; ++R) {
     const int par = R & 1;
-    float* Sbuf = b.Sb[par];
-    float* Ubuf = b.Ub[par];
-    if (side && vpending[par]) S1_TRY(cudaStreamWaitEvent(s, side->done[par], 0));
+    float *Sbuf = b.Sb[par], *Ubuf = b.Ub[par];
+    if (side && R >= 2) {
+      S1_TRY(cudaStreamWaitEvent(s, side->a[par], 0));
+      S1_TRY(cudaStreamWaitEvent(s, side->v[par], 0));
+    }
     unsigned* Mbuf = b.sparse ? b.Mb[par] : nullptr;
+    const bool ahead = look && R > 0;
     S1_TRY(mpj_launch_pdl(b.half ? solve32<true, OneSub32> : solve32<false, OneSub32>, dim3(npairs), dim3(S32_THREADS),
-                          0, s, OneSub32{b.A32, N, nb, Sbuf, Ubuf, Mbuf}, R, b.tc != 1));
-    auto vmul = b.sparse ? rmul32<R32_ALL, true> : rmul32<R32_ALL, false>;
-    // V <- V U~
+                          0, s,
+                          OneSub32{b.A32, N, nb, Sbuf, Ubuf, Mbuf, ahead ? b.Sb[par ^ 1] : nullptr, b.Ub[par ^ 1],
+                                   b.Tb[par]},
+                          R, b.tc != 1));
     if (side) {
-      S1_TRY(cudaEventRecord(side->ready, s));
-      S1_TRY(cudaStreamWaitEvent(side->sv, side->ready, 0));
-      S1_TRY(mpj_launch_pdl(vmul, g32, dim3(RT), 0, side->sv, (const float*)b.V32, b.V32, N, nb, R, (const float*)Sbuf,
-                            (const float*)Ubuf, b.half, b.tc == 1, (const unsigned*)Mbuf));
-      S1_TRY(cudaEventRecord(side->done[par], side->sv));
-      vpending[par] = true;
-    } else {
-      S1_TRY(mpj_launch_pdl(vmul, g32, dim3(RT), 0, s, (const float*)b.V32, b.V32, N, nb, R, (const float*)Sbuf,
-                            (const float*)Ubuf, b.half, b.tc == 1, (const unsigned*)Mbuf));
+      S1_TRY(cudaEventRecord(side->solved[par], s));
+      S1_TRY(cudaStreamWaitEvent(sa, side->solved[par], 0));
+      S1_TRY(cudaStreamWaitEvent(sv, side->solved[par], 0));
     }
     if (b.tc == 1) {
       // A' = U^T A U = (A U)^T U (A symmetric): B^T = (A U)^T, then
@@ -675,13 +791,22 @@ cudaError_t stage1_sweep(const Stage1Bufs& b, cudaStream_t s, SideStream* side) 
     } else {
       // A <- U~^T A U~ in one pass (tiles a > Q, mirrored; S on the diagonal)
       auto amul = b.sparse ? rmul32<R32_BOTH, true> : rmul32<R32_BOTH, false>;
-      S1_TRY(mpj_launch_pdl(amul, g32, dim3(RT), 0, s, (const float*)b.A32, b.A32, N, nb, R, (const float*)Sbuf,
+      S1_TRY(mpj_launch_pdl(amul, g32, dim3(RT), 0, sa, (const float*)b.A32, b.A32, N, nb, R, (const float*)Sbuf,
                             (const float*)Ubuf, b.half, false, (const unsigned*)Mbuf));
+      if (R + 2 < rounds) S1_TRY(snap(R + 2, sa));
     }
+    if (side) S1_TRY(cudaEventRecord(side->a[par], sa));
+    // V <- V U~
+    auto vmul = b.sparse ? rmul32<R32_ALL, true> : rmul32<R32_ALL, false>;
+    S1_TRY(mpj_launch_pdl(vmul, g32, dim3(RT), 0, sv, (const float*)b.V32, b.V32, N, nb, R, (const float*)Sbuf,
+                          (const float*)Ubuf, b.half, b.tc == 1, (const unsigned*)Mbuf));
+    if (side) S1_TRY(cudaEventRecord(side->v[par], sv));
   }
   if (side)
-    for (int par = 0; par < 2; ++par)
-      if (vpending[par]) S1_TRY(cudaStreamWaitEvent(s, side->done[par], 0));
+    for (int par = 0; par < 2 && par < rounds; ++par) {
+      S1_TRY(cudaStreamWaitEvent(s, side->a[par], 0));
+      S1_TRY(cudaStreamWaitEvent(s, side->v[par], 0));
+    }
 #undef S1_TRY
   return cudaGetLastError();
 }
@@ -742,13 +867,11 @@ std::shared_ptr<SweepGraph> sweep_graph(const Stage1Bufs& b, void* work, bool us
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaError_t e = cudaSuccess;
-  // kernels of one sweep: per round the subproblems, V U~ and the A update
-  // (one launch, or two tensor-core panels)
-  const long long per = (long long)(b.nb - 1) * (b.tc == 1 ? 4 : 3);
+  const long long per = stage1_sweep_launches(b);
   {
-    std::unique_ptr<SideStream> side;
+    std::unique_ptr<SweepStreams> side;
     if (use_side) {
-      side.reset(new SideStream(cap));
+      side.reset(new SweepStreams(cap));
       if (!side->ok) e = cudaErrorUnknown;
       side->owner = nullptr;  // joined inside the captured sweep
     }
@@ -802,6 +925,8 @@ int mpj_stage1_run(int n, const double* A, int lda, double* Ql, int ldq, double 
   b.tflag = (unsigned*)(b.Bt + (size_t)N * N);
   b.Mb[0] = b.tflag + 64;
   b.Mb[1] = b.Mb[0] + nb / 2;
+  b.Tb[0] = (float*)(((size_t)(b.Mb[1] + nb / 2) + 255) & ~(size_t)255);
+  b.Tb[1] = b.Tb[0] + pset;
   b.half = half;
   b.sparse = sparse;
   b.tc = stage1_tensor_cores() && !half;
@@ -817,9 +942,9 @@ int mpj_stage1_run(int n, const double* A, int lda, double* Ql, int ldq, double 
   MPJ_CUDA_TRY(cudaStreamSynchronize(s));
   double off = sqrt(off2);
   int sweeps = 0, status = MPJ_OK;
-  const bool use_side = mpj_v_overlap_enabled() && nb / 2 >= 8;
+  const bool use_side = mpj_v_overlap_enabled() && nb / 2 >= 2;
   std::shared_ptr<SweepGraph> graph;
-  std::unique_ptr<SideStream> side;
+  std::unique_ptr<SweepStreams> side;
   while (off > tol32) {
     if (sweeps >= max_sweeps) {
       status = MPJ_NOT_CONVERGED;
@@ -831,7 +956,7 @@ int mpj_stage1_run(int n, const double* A, int lda, double* Ql, int ldq, double 
       mpj_count_launches(graph->launches);
     } else {
       if (use_side && !side) {
-        side.reset(new SideStream(s));
+        side.reset(new SweepStreams(s));
         if (!side->ok) side.reset();
       }
       MPJ_CUDA_TRY(stage1_sweep(b, s, side.get()));
