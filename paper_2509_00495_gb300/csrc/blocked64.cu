@@ -1246,13 +1246,6 @@ cudaError_t rmul_attr() {
   if (e == cudaSuccess) done = true;
   return e;
 }
-int sm_count() {
-  int dev = 0, sms = 152;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    (void)cudaGetLastError();
-  return sms;
-}
 }  // namespace
 
 // Round R, step 1: the subproblems of the block pairs, U_P into set R mod 2;

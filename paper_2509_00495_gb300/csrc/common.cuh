@@ -256,6 +256,15 @@ cudaError_t mpj_launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size
   return e;
 }
 
+// SMs of the current device.
+inline int sm_count() {
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    (void)cudaGetLastError();
+  return sms;
+}
+
 // Side stream and events for overlapping the V updates with the rotation
 // rounds; released when the solve returns.  On every exit (also an early
 // error return) the owner stream is first made to wait for the side stream,

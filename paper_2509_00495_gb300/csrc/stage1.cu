@@ -368,7 +368,8 @@ __global__ void __launch_bounds__(S32_THREADS, 1) solve32(Src src, int R, bool u
 
 // Saves, for every pair of round R >= 1, the 32 x 32 tile of A between the pairs
 // of round R - 1 that held its two blocks (rows of the lower block's pair).
-__global__ void __launch_bounds__(256) snap32(const float* __restrict__ A32, int N, int nb, int R, float* __restrict__ T) {
+__global__ void __launch_bounds__(256) snap32(const float* __restrict__ A32, int N, int nb, int R,
+                                              float* __restrict__ T) {
   pdl_wait();
   int a, oa, q, oq, Ia, Ja, Iq, Jq;
   prev_slots(nb, R, blockIdx.x, a, oa, q, oq);
@@ -629,6 +630,218 @@ __global__ void __launch_bounds__(RT) rmul32(const float* X, float* Y, int N, in
   rmul32_tile<TRI, MASKED>(sm, X, Y, N, nb, R, Sbuf, Ubuf, hq, ucol, Mbuf, blockIdx.x, blockIdx.y);
 }
 
+// ---------------------------------------------------------------- both updates in one launch
+// The tiles of A <- U~^T A U~ and V <- V U~ formed by persistent CTAs of two
+// warps, each from a queue: while a tile is multiplied, the next one's values
+// and rotations are on their way (cp.async, two stages).  Half-warp w forms the
+// 32 x 32 block of block pair 4 gx + w, each lane 8 x 8 of it: 16 shared-memory
+// floats per 64 FMAs, where rmul32's 4 x 8 take 12 per 32.  What rmul32 spends
+// its time on at n = 4096 (A 46 us, V 33 us, DRAM traffic 46 and 79 MB): its
+// loads keep the shared-memory pipe 70-75 % busy, and every tile waits for its
+// values with 17 to 25 warps resident.  More outputs per lane alone, without the
+// pipeline, lost (A's and V's rounds 88 us instead of 82: half the warps to hide
+// the wait with).  Measured per round, subproblems included (they overlap):
+// see update_form.
+constexpr int PT = 64;
+template <bool VONLY>
+struct __align__(16) PipeStage {
+  float X[W2][XLD];     // X[k][r] = X_Q(r, k); A: then T = X_Q U_Q per half-warp
+  float U[W2][W2];      // U[k][c] = U_Q(k, c)
+  float Ua[4][W2][W2];  // A: U_a of each half-warp's pair
+};
+template <>
+struct __align__(16) PipeStage<true> {
+  float X[W2][XLD];
+  float U[W2][W2];
+};
+
+MPJ_DEV void cp16(float* dst, const float* src, bool valid) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(valid ? 16 : 0)
+               : "memory");
+}
+
+// The 32 x 32 product of a half-warp: acc(i, j) = sum_k L(k, r_i) R(k, c_j) for
+// the lane's rows r = {0 .. 3, 16 .. 19} and columns c alike, relative to L and R
+// (k-major, row strides LDL, LDR); the sums are warp_mm32's.
+template <int LDL, int LDR>
+MPJ_DEV void half_mm32(const float* L, const float* R, float acc[8][8]) {
+  unsigned long long acc2[8][4];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int jp = 0; jp < 4; ++jp) acc2[i][jp] = 0ULL;
+#pragma unroll 4
+  for (int k = 0; k < W2; ++k) {
+    const float4 x0 = *reinterpret_cast<const float4*>(L + k * LDL);
+    const float4 x1 = *reinterpret_cast<const float4*>(L + k * LDL + 16);
+    const float4 u0 = *reinterpret_cast<const float4*>(R + k * LDR);
+    const float4 u1 = *reinterpret_cast<const float4*>(R + k * LDR + 16);
+    const float xa[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+    const unsigned long long up[4] = {pk2(u0.x, u0.y), pk2(u0.z, u0.w), pk2(u1.x, u1.y), pk2(u1.z, u1.w)};
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const unsigned long long xx = pk2(xa[i], xa[i]);
+#pragma unroll
+      for (int jp = 0; jp < 4; ++jp) fma2(acc2[i][jp], xx, up[jp]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int jp = 0; jp < 4; ++jp) unpk2(acc2[i][jp], acc[i][2 * jp], acc[i][2 * jp + 1]);
+}
+
+// Tile t of the queue: A's first (row groups gx >= Q / 4 of column Q; the
+// larger ones, so that the end is of small ones), then V's.
+struct PipeTile {
+  int gx, Q;
+  bool both;  // A <- U~^T A U~
+};
+__host__ __device__ inline int pipe_before(int gxn, int grp) { return 4 * grp * gxn - 2 * grp * (grp - 1); }
+__host__ __device__ inline int pipe_tiles_a(int npairs) {  // column groups of 4: gxn - group tiles per column
+  const int gxn = (npairs + 3) / 4;
+  return pipe_before(gxn, gxn) - (4 * gxn - npairs);
+}
+__host__ __device__ inline int pipe_tiles_v(int npairs) { return npairs * ((npairs + 3) / 4); }
+__host__ __device__ inline PipeTile pipe_tile(int npairs, int t) {
+  const int gxn = (npairs + 3) / 4, ta = pipe_tiles_a(npairs);
+  if (t >= ta) return {(t - ta) % gxn, (t - ta) / gxn, false};
+  // the group: largest grp with pipe_before(grp) <= t
+  const float b = 2.0f * gxn + 1.0f;
+  int grp = (int)(0.5f * (b - sqrtf(fmaxf(b * b - 2.0f * t, 0.0f))));
+  grp = grp < 0 ? 0 : grp >= gxn ? gxn - 1 : grp;
+  while (grp > 0 && pipe_before(gxn, grp) > t) --grp;
+  while (grp + 1 < gxn && pipe_before(gxn, grp + 1) <= t) ++grp;
+  const int rest = t - pipe_before(gxn, grp);
+  return {grp + rest % (gxn - grp), 4 * grp + rest / (gxn - grp), true};
+}
+
+// Tiles first .. end - 1 of the queue (VONLY: all of them V's; half the shared
+// memory).  queue[0]: tiles handed out beyond the first gridDim.x, queue[1]:
+// CTAs done; both 0 before and after.
+template <bool VONLY>
+__global__ void __launch_bounds__(PT, VONLY ? 5 : 3) rmul32_pipe(float* A32, float* V32, int N, int nb, int R,
+                                                     const float* __restrict__ Sbuf, const float* __restrict__ Ubuf,
+                                                     bool hq, int first, int end, unsigned* queue) {
+  extern __shared__ __align__(16) unsigned char pipe_raw[];
+  PipeStage<VONLY>* st = reinterpret_cast<PipeStage<VONLY>*>(pipe_raw);
+  __shared__ int slot[2];
+  const int tid = threadIdx.x, npairs = nb / 2;
+  const int w = tid >> 4, g = tid & 3, h = (tid >> 2) & 3;
+  pdl_wait();
+  auto fetch = [&](PipeStage<VONLY>& p, int t) {
+    if (t < end) {
+      PipeTile q = pipe_tile(npairs, t);
+      if (VONLY) q.both = false;
+      int I, J, IQ, JQ;
+      block_pair(nb, R, q.Q, IQ, JQ);
+      // X_Q(r, k) = X[g_Q(k) N + row(r)]: rows 4 (t mod 32) .. +3, k = t / 32 + 2 i
+      const int rq = tid & 31, ar = 4 * q.gx + (rq >> 3);
+      const bool valid = ar < npairs && (!q.both || ar > q.Q);
+      block_pair(nb, R, valid ? ar : q.Q, I, J);
+      const float* x = (q.both ? A32 : V32) + gidx(I, J, (4 * rq) & 31);
+#pragma unroll
+      for (int i = 0; i < W2 / 2; ++i) {
+        const int k = (tid >> 5) + 2 * i;
+        cp16(&p.X[k][4 * rq], x + (size_t)gidx(IQ, JQ, k) * N, valid);
+      }
+      const float* u = Ubuf + (size_t)q.Q * W2 * W2 + 4 * tid;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) cp16(&p.U[0][0] + 4 * tid + 256 * i, u + 256 * i, true);
+      if constexpr (!VONLY) {
+        if (q.both)
+          for (int j = 0; j < 4; ++j) {
+            const int a = 4 * q.gx + j;
+            if (a <= q.Q || a >= npairs) continue;
+            const float* ua = Ubuf + (size_t)a * W2 * W2 + 4 * tid;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) cp16(&p.Ua[j][0][0] + 4 * tid + 256 * i, ua + 256 * i, true);
+          }
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  int t = first + blockIdx.x;
+  fetch(st[0], t);
+  if (tid == 0) slot[1] = first + gridDim.x + atomicAdd(queue, 1u);
+  __syncthreads();
+  for (int it = 0; t < end; ++it) {
+    const int next = slot[(it + 1) & 1];
+    unsigned after = 0;
+    if (tid == 0 && next < end) after = atomicAdd(queue, 1u);
+    fetch(st[(it + 1) & 1], next);
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();
+    PipeStage<VONLY>& p = st[it & 1];
+    PipeTile q = pipe_tile(npairs, t);
+    if (VONLY) q.both = false;
+    const int a = 4 * q.gx + w, aw = 4 * q.gx + 2 * (tid >> 5);  // this half-warp's block pair, the warp's first
+    if (aw < npairs && (!q.both || aw + 1 >= q.Q)) {
+      float acc[8][8];
+      half_mm32<XLD, W2>(&p.X[0][32 * w + 4 * g], &p.U[0][4 * h], acc);
+      if constexpr (!VONLY) {
+        if (q.both) {
+          // T = X_Q U_Q in place of X_Q (T(i, c) at X[i][32 w + c]), then U_a^T T
+          __syncwarp();
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            float* d = &p.X[4 * g + (i & 3) + 4 * (i & 4)][32 * w + 4 * h];
+            *reinterpret_cast<float4*>(d) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+            *reinterpret_cast<float4*>(d + 16) = make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
+          }
+          __syncwarp();
+          half_mm32<W2, XLD>(&p.Ua[w][0][4 * g], &p.X[0][32 * w + 4 * h], acc);
+        }
+      }
+      if (a < npairs && (!q.both || a >= q.Q)) {
+        int I, J, IQ, JQ;
+        block_pair(nb, R, a, I, J);
+        block_pair(nb, R, q.Q, IQ, JQ);
+        const int r0 = I * BS + 4 * g, r1 = J * BS + 4 * g, c0 = IQ * BS + 4 * h, c1 = JQ * BS + 4 * h;
+        float* Y = q.both ? A32 : V32;
+        if (q.both && a == q.Q) {
+          // the diagonal tile: the solved subproblem
+          const float* Sq = Sbuf + (size_t)q.Q * W2 * W2 + 4 * g;
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const float* c = Sq + W2 * (4 * h + (j & 3) + 4 * (j & 4));
+            float* y = Y + (size_t)(j < 4 ? c0 + j : c1 + j - 4) * N;
+            *reinterpret_cast<float4*>(y + r0) = *reinterpret_cast<const float4*>(c);
+            *reinterpret_cast<float4*>(y + r1) = *reinterpret_cast<const float4*>(c + 16);
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[i][j] = qh(acc[i][j], hq);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            float* y = Y + (size_t)(j < 4 ? c0 + j : c1 + j - 4) * N;
+            *reinterpret_cast<float4*>(y + r0) = make_float4(acc[0][j], acc[1][j], acc[2][j], acc[3][j]);
+            *reinterpret_cast<float4*>(y + r1) = make_float4(acc[4][j], acc[5][j], acc[6][j], acc[7][j]);
+          }
+          if (q.both) {  // the mirror
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              float* y = Y + (size_t)(i < 4 ? r0 + i : r1 + i - 4) * N;
+              *reinterpret_cast<float4*>(y + c0) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+              *reinterpret_cast<float4*>(y + c1) = make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
+            }
+          }
+        }
+      }
+    }
+    if (tid == 0) slot[it & 1] = next < end ? (int)(first + gridDim.x + after) : end;
+    t = next;
+    __syncthreads();
+  }
+  if (tid == 0 && atomicAdd(queue + 1, 1u) == gridDim.x - 1) {  // the last CTA: no one asks any more
+    queue[0] = 0;
+    queue[1] = 0;
+  }
+}
+
 // A batch: the tiles of A <- U~^T A U~, then those of V <- V U~, per matrix.
 MPJ_DEV int batch_tiles32(int np) { return 2 * ((np + 3) / 4) * np; }
 __global__ void __launch_bounds__(RT) rmul32_batch(BatchShape b, int lo, int R, float* A32, float* V32,
@@ -665,7 +878,7 @@ cudaError_t mpj_batch_stage1_round(const BatchShape& b, int R, float* A32, float
 int mpj_stage1_padded(int n) { return ((n + W2 - 1) / W2) * W2; }
 
 // A32, V32, two sets of the per-pair S and U (alternate rounds), the
-// tensor-core update's transposed intermediate B^T, a flag word, two sets of
+// tensor-core update's transposed intermediate B^T, flag and queue words, two sets of
 // the per-pair rotated-index masks, two of the saved tiles.
 static int stage1_tensor_cores();
 
@@ -678,7 +891,7 @@ size_t mpj_stage1_bytes(int n) {
 // MPJ_STAGE1_TC=1 runs the A update of each block round on the tcgen05
 // tensor cores (3xTF32, two panel products, see tc32.cu) and the V update on
 // the FP32 pipe.  Off by default: on GB300 at n = 4096 it is slower (600 vs
-// 435 ms for the stage), and V must stay on the FP32 pipe because the tensor
+// 178 ms for the stage), and V must stay on the FP32 pipe because the tensor
 // cores' FP32 accumulation drifts the column norms over thousands of products
 // (||V^T V - I||_F 0.08 instead of 0.007).
 static int stage1_tensor_cores() {
@@ -701,17 +914,17 @@ namespace {
 // diagonal blocks come from round R's solved subproblems and their coupling
 // blocks from tiles of A saved before that update (snap32).  So the chain of a
 // sweep is the subproblems alone; A's updates (with the saving of tiles) and
-// V's run on two side streams (when given), two rounds behind at most: round
-// R's subproblems wait for the tiles saved after round R - 2's update, which
-// also frees the S, U and T sets that alternate between rounds, and for V's
-// update of round R - 2.  Both streams are joined into s at the end.  Before, a
-// round was the subproblems, then A's update: n = 96 25 us a round, now 20;
-// n = 300 20.6, now 18; n = 1024 20.0, now 19.3 (there the updates, sharing SMs
-// with the subproblems, take turns with them: the subproblems alone run at 12.5).
+// V's run on side streams (when given; in one launch, update_form), two rounds
+// behind at most: round R's subproblems wait for the tiles saved after round
+// R - 2's update, which also frees the S, U and T sets that alternate between
+// rounds, and for V's update of round R - 2.  The streams are joined into s at
+// the end.  Before, a round was the subproblems, then A's update: n = 96 25 us a
+// round, now 20; n = 300 20.6, now 16.5; n = 1024 20.0, now 15.7 (the
+// subproblems alone 12.5).
 struct Stage1Bufs {
   int N, nb;
   float *A32, *V32, *Sb[2], *Ub[2], *Tb[2], *Bt;
-  unsigned* tflag;
+  unsigned* tflag;  // word 0: flags of the tensor-core update; from 8, 16: rmul32_pipe's queues
   unsigned* Mb[2];  // per-pair rotated-index masks, by round parity
   bool half;
   bool sparse;  // products over the rotated indices only (masked kernels)
@@ -743,15 +956,49 @@ struct SweepStreams {
   }
 };
 
+// How a round's updates run.  Microseconds per round (subproblems included)
+// with rmul32 per matrix / both matrices in one rmul32_pipe / one rmul32_pipe
+// each:
+//   n    257   512   768   1024  1280  1536  2048  2560  2944  3072  4096  6144
+//        17.2  16.2  15.6  19.8  18.9  22.3  27.0  37.1  44.9  47.7  82.2  171
+//        16.5  15.4  15.6  15.7  19.4  22.4  31.5  44.1        58.2  97.0
+//                          15.7  21.4  25.5  32.7  39.2  45.7  46.6  69.8  147
+// One launch wins while all its tiles run at once, three CTAs per SM (a launch
+// and a stream's events fewer per round); one launch each, V's tiles five CTAs
+// per SM, once A's fill the SMs several times over (two per SM leave room for V's
+// and for the next subproblems: three took 80 us at n = 4096).  In between the
+// waves of rmul32's CTAs fit better around the subproblems.
+enum { UPD_RMUL, UPD_ONE, UPD_EACH };
+int update_form(const Stage1Bufs& b) {
+  if (b.tc == 1 || b.sparse) return UPD_RMUL;
+  const int np = b.nb / 2, ta = pipe_tiles_a(np), tv = pipe_tiles_v(np), sms = sm_count();
+  return ta + tv <= 3 * sms ? UPD_ONE : 2 * ta >= 15 * sms ? UPD_EACH : UPD_RMUL;
+}
+
+template <bool VONLY>
+cudaError_t pipe_attr() {
+  return cudaFuncSetAttribute(rmul32_pipe<VONLY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              2 * (int)sizeof(PipeStage<VONLY>));
+}
+template <bool VONLY>
+cudaError_t pipe_launch(const Stage1Bufs& b, int R, const float* S, const float* U, int first, int end, int per_sm,
+                        cudaStream_t s) {
+  const int most = per_sm * sm_count();
+  return mpj_launch_pdl(rmul32_pipe<VONLY>, dim3(end - first < most ? end - first : most), dim3(PT),
+                        2 * sizeof(PipeStage<VONLY>), s, b.A32, b.V32, b.N, b.nb, R, S, U, b.half, first, end,
+                        b.tflag + (VONLY ? 16 : 8));
+}
+
 // Kernels of one sweep.
 long long stage1_sweep_launches(const Stage1Bufs& b) {
   const long long rounds = b.nb - 1;
-  return b.tc == 1 ? 4 * rounds : 3 * rounds + (rounds - 1);
+  return b.tc == 1 ? 4 * rounds : (update_form(b) == UPD_ONE ? 2 : 3) * rounds + (rounds - 1);
 }
 
 cudaError_t stage1_sweep(const Stage1Bufs& b, cudaStream_t s, SweepStreams* side) {
   const int N = b.N, nb = b.nb, npairs = nb / 2, rounds = nb - 1;
   const dim3 g32((npairs + 3) / 4, npairs);
+  const int form = update_form(b), ta = pipe_tiles_a(npairs), tv = pipe_tiles_v(npairs);
   const bool look = b.tc != 1;  // the tensor-core update transposes through Bt, in order
   cudaStream_t sa = side ? side->sa : s, sv = side ? side->sv : s;
   cudaError_t e = cudaSuccess;
@@ -763,13 +1010,17 @@ cudaError_t stage1_sweep(const Stage1Bufs& b, cudaStream_t s, SweepStreams* side
   auto snap = [&](int R, cudaStream_t st) {
     return mpj_launch_pdl(snap32, dim3(npairs), dim3(256), 0, st, (const float*)b.A32, N, nb, R, b.Tb[R & 1]);
   };
+  if (form != UPD_RMUL) {
+    S1_TRY(pipe_attr<false>());
+    S1_TRY(pipe_attr<true>());
+  }
   if (look && rounds > 1) S1_TRY(snap(1, s));
   for (int R = 0; R < rounds; ++R) {
     const int par = R & 1;
     float *Sbuf = b.Sb[par], *Ubuf = b.Ub[par];
     if (side && R >= 2) {
       S1_TRY(cudaStreamWaitEvent(s, side->a[par], 0));
-      S1_TRY(cudaStreamWaitEvent(s, side->v[par], 0));
+      if (form != UPD_ONE) S1_TRY(cudaStreamWaitEvent(s, side->v[par], 0));
     }
     unsigned* Mbuf = b.sparse ? b.Mb[par] : nullptr;
     const bool ahead = look && R > 0;
@@ -781,7 +1032,7 @@ cudaError_t stage1_sweep(const Stage1Bufs& b, cudaStream_t s, SweepStreams* side
     if (side) {
       S1_TRY(cudaEventRecord(side->solved[par], s));
       S1_TRY(cudaStreamWaitEvent(sa, side->solved[par], 0));
-      S1_TRY(cudaStreamWaitEvent(sv, side->solved[par], 0));
+      if (form != UPD_ONE) S1_TRY(cudaStreamWaitEvent(sv, side->solved[par], 0));
     }
     if (b.tc == 1) {
       // A' = U^T A U = (A U)^T U (A symmetric): B^T = (A U)^T, then
@@ -790,22 +1041,31 @@ cudaError_t stage1_sweep(const Stage1Bufs& b, cudaStream_t s, SweepStreams* side
       S1_TRY(mpj_tc_panel(N, nb, R, Ubuf, b.Bt, b.A32, 0, nullptr, nullptr, b.tflag, s));
     } else {
       // A <- U~^T A U~ in one pass (tiles a > Q, mirrored; S on the diagonal)
-      auto amul = b.sparse ? rmul32<R32_BOTH, true> : rmul32<R32_BOTH, false>;
-      S1_TRY(mpj_launch_pdl(amul, g32, dim3(RT), 0, sa, (const float*)b.A32, b.A32, N, nb, R, (const float*)Sbuf,
-                            (const float*)Ubuf, b.half, false, (const unsigned*)Mbuf));
+      if (form == UPD_RMUL) {
+        auto amul = b.sparse ? rmul32<R32_BOTH, true> : rmul32<R32_BOTH, false>;
+        S1_TRY(mpj_launch_pdl(amul, g32, dim3(RT), 0, sa, (const float*)b.A32, b.A32, N, nb, R, (const float*)Sbuf,
+                              (const float*)Ubuf, b.half, false, (const unsigned*)Mbuf));
+      } else {
+        S1_TRY(pipe_launch<false>(b, R, Sbuf, Ubuf, 0, form == UPD_ONE ? ta + tv : ta, form == UPD_ONE ? 3 : 2, sa));
+      }
       if (R + 2 < rounds) S1_TRY(snap(R + 2, sa));
     }
     if (side) S1_TRY(cudaEventRecord(side->a[par], sa));
+    if (form == UPD_ONE) continue;
     // V <- V U~
-    auto vmul = b.sparse ? rmul32<R32_ALL, true> : rmul32<R32_ALL, false>;
-    S1_TRY(mpj_launch_pdl(vmul, g32, dim3(RT), 0, sv, (const float*)b.V32, b.V32, N, nb, R, (const float*)Sbuf,
-                          (const float*)Ubuf, b.half, b.tc == 1, (const unsigned*)Mbuf));
+    if (form == UPD_EACH) {
+      S1_TRY(pipe_launch<true>(b, R, Sbuf, Ubuf, ta, ta + tv, 5, sv));
+    } else {
+      auto vmul = b.sparse ? rmul32<R32_ALL, true> : rmul32<R32_ALL, false>;
+      S1_TRY(mpj_launch_pdl(vmul, g32, dim3(RT), 0, sv, (const float*)b.V32, b.V32, N, nb, R, (const float*)Sbuf,
+                            (const float*)Ubuf, b.half, b.tc == 1, (const unsigned*)Mbuf));
+    }
     if (side) S1_TRY(cudaEventRecord(side->v[par], sv));
   }
   if (side)
     for (int par = 0; par < 2 && par < rounds; ++par) {
       S1_TRY(cudaStreamWaitEvent(s, side->a[par], 0));
-      S1_TRY(cudaStreamWaitEvent(s, side->v[par], 0));
+      if (form != UPD_ONE) S1_TRY(cudaStreamWaitEvent(s, side->v[par], 0));
     }
 #undef S1_TRY
   return cudaGetLastError();
@@ -932,7 +1192,7 @@ int mpj_stage1_run(int n, const double* A, int lda, double* Ql, int ldq, double 
   b.tc = stage1_tensor_cores() && !half;
   float* A32 = b.A32;
   float* V32 = b.V32;
-  MPJ_CUDA_TRY(cudaMemsetAsync(b.tflag, 0, sizeof(unsigned), s));
+  MPJ_CUDA_TRY(cudaMemsetAsync(b.tflag, 0, 64 * sizeof(unsigned), s));
   init32<<<1024, 256, 0, s>>>(A, lda, n, N, A32, V32, half);
   mpj_count_launch();
   MPJ_CUDA_TRY(cudaGetLastError());
