@@ -1259,6 +1259,17 @@ cudaError_t mpj_blocked_solve(const double* A, int lda, int n, int R, double ski
                         dim3(SOLVE_THREADS), 0, s, OneSub64{A, lda, n, nb, skip_abs, u.sl, u.ex, u.rot, nrot}, R, skip);
 }
 
+// The products for A run ahead of those for V (a side stream's), which nothing
+// waits for before the next round but one: A's CTAs take every slot that falls
+// free.  FP64 sweeps at n = 1500 (twelve) 74.0 -> 71.3 ms, n = 2048 24.1 -> 23.2,
+// n = 4096 258 -> 256.  The subproblems gained nothing by it (and 75 ms with both).
+// A stream that is above the side stream already keeps its own priority.
+static int rm_a_priority(cudaStream_t s) {
+  int p = 0;
+  if (cudaStreamGetPriority(s, &p) != cudaSuccess) (void)cudaGetLastError();
+  return p < 0 ? 0 : -1;
+}
+
 // Round R, step 2: A <- U~^T A U~ through B (two right multiplications).
 cudaError_t mpj_blocked_update_A(double* A, int lda, double* B, int n, int R, void* scratch, unsigned* flags,
                                  cudaStream_t s) {
@@ -1268,12 +1279,14 @@ cudaError_t mpj_blocked_update_A(double* A, int lda, double* B, int n, int R, vo
   cudaError_t e = rmul_attr();
   if (e != cudaSuccess) return e;
   const dim3 grid((nb / 2 + 3) / 4, nb / 2);
-  e = mpj_launch_pdl(blk_rmul, grid, dim3(RM_THREADS), rmul_smem(), s, (const double*)A, lda, (int)XMODE_COLS, B, n,
-                     n, nb, R, (const __half*)u.sl, (const int*)u.ex, (const int*)u.rot, flags, (int)TRI_FIRST);
+  const int prio = rm_a_priority(s);
+  e = mpj_launch_pdl_at(prio, blk_rmul, grid, dim3(RM_THREADS), rmul_smem(), s, (const double*)A, lda, (int)XMODE_COLS,
+                        B, n, n, nb, R, (const __half*)u.sl, (const int*)u.ex, (const int*)u.rot, flags,
+                        (int)TRI_FIRST);
   if (e != cudaSuccess) return e;
-  return mpj_launch_pdl(blk_rmul, grid, dim3(RM_THREADS), rmul_smem(), s, (const double*)B, n, (int)XMODE_ROWS, A,
-                        lda, n, nb, R, (const __half*)u.sl, (const int*)u.ex, (const int*)u.rot, flags,
-                        (int)TRI_SECOND);
+  return mpj_launch_pdl_at(prio, blk_rmul, grid, dim3(RM_THREADS), rmul_smem(), s, (const double*)B, n,
+                           (int)XMODE_ROWS, A, lda, n, nb, R, (const __half*)u.sl, (const int*)u.ex,
+                           (const int*)u.rot, flags, (int)TRI_SECOND);
 }
 
 // Round R, step 3: V <- V U~ (in place); independent of step 2.

@@ -238,22 +238,31 @@ MPJ_DEV void pdl_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// priority: 0 = the stream's; a negative one is the launch's own (0 is the lowest).
 template <typename... KArgs, typename... Args>
-cudaError_t mpj_launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                           Args... args) {
+cudaError_t mpj_launch_pdl_at(int priority, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                              cudaStream_t s, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributePriority;
+  attr[1].val.priority = priority;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = priority ? 2 : 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
   mpj_count_launch();
   return e;
+}
+
+template <typename... KArgs, typename... Args>
+cudaError_t mpj_launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                           Args... args) {
+  return mpj_launch_pdl_at(0, kernel, grid, block, smem, s, args...);
 }
 
 // SMs of the current device.
