@@ -273,10 +273,18 @@ __global__ void oz_rowmax_warp(const double* __restrict__ X, long long rs, long 
 }
 
 // The 8 slices of 8 consecutive k values of one row per thread, written as
-// one 16-byte core-matrix row per slice.  rows_fast: consecutive threads take
-// consecutive rows (coalesced reads of column-major rows).
+// one 16-byte core-matrix row per slice.  ROWS: consecutive threads take
+// consecutive rows (coalesced reads of column-major rows).  Otherwise a warp takes
+// 8 rows of 32 k: it reads 256 contiguous bytes of each (in 16-byte loads where k
+// runs along memory and the address allows) and writes 512 contiguous bytes per
+// slice.  With 32 k groups of one row per warp the writes were 16-byte pieces of
+// 32-byte sectors: 219 us for a 4096 x 4096 operand (DRAM 267 + 339 MB), now 79
+// (134 + 209 MB; column-major rows 90-102; 400 MB at the copy rate: 59).  Two
+// instances, since the wide loads' 80 registers cost the other form its occupancy
+// (122 us).
+template <bool ROWS>
 __global__ void oz_slice(const double* __restrict__ X, long long rs, long long ks, long long sx, int R, int K, int Rp,
-                         int Kp, int rows_fast, const unsigned long long* __restrict__ mx, int* __restrict__ exps,
+                         int Kp, const unsigned long long* __restrict__ mx, int* __restrict__ exps,
                          __nv_bfloat16* __restrict__ S, long long sop) {
   X += blockIdx.z * sx;
   mx = (const unsigned long long*)((const char*)mx + blockIdx.z * sop);
@@ -287,22 +295,34 @@ __global__ void oz_slice(const double* __restrict__ X, long long rs, long long k
   for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
        idx += (long long)gridDim.x * blockDim.x) {
     int r, g;
-    if (rows_fast) {
+    if (ROWS) {
       r = (int)(idx % Rp);
       g = (int)(idx / Rp);
     } else {
-      g = (int)(idx % (Kp / 8));
-      r = (int)(idx / (Kp / 8));
+      const long long w = idx >> 5;
+      g = 4 * (int)(w % (Kp / OZ_KS)) + (int)(idx & 3);
+      r = 8 * (int)(w / (Kp / OZ_KS)) + (int)((idx >> 2) & 7);
     }
     const int k0 = g * 8;
     const int e = r < R ? oz_exp_of(mx[r]) : 0;  // every |x(r, k)| < 2^e
     if (g == 0) exps[r] = e;
     uint32_t d[8][OZ_S];
+    const double* x0 = X + (long long)r * rs + (long long)k0 * ks;
+    if (!ROWS && ks == 1 && r < R && k0 + 8 <= K && ((size_t)x0 & 15) == 0) {
+      double2 v[4];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int k = k0 + j;
-      const double x = (r < R && k < K) ? X[(long long)r * rs + (long long)k * ks] : 0.0;
-      oz_digits(x, e, d[j]);
+      for (int j = 0; j < 4; ++j) v[j] = reinterpret_cast<const double2*>(x0)[j];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        oz_digits(v[j].x, e, d[2 * j]);
+        oz_digits(v[j].y, e, d[2 * j + 1]);
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const double x = (r < R && k0 + j < K) ? x0[(long long)j * ks] : 0.0;
+        oz_digits(x, e, d[j]);
+      }
     }
     const long long tile = (long long)(k0 / OZ_KS) * (Rp / 64) + r / 64;
     const long long off = tile * OZ_TILE64 + (kmaj16(r & 63, k0 & 31) >> 1);
@@ -634,8 +654,8 @@ cudaError_t mpj_oz_prepare(const double* X, long long rs, long long ks, int R, i
   }
   const long long total = (long long)Rp * (Kp / 8);
   const int blocks = (int)((total + 255) / 256 > 8192 ? 8192 : (total + 255) / 256);
-  oz_slice<<<dim3(blocks, 1, batch), 256, 0, s>>>(X, rs, ks, sx, R, K, Rp, Kp, rs == 1 ? 1 : 0, mx, exps, S,
-                                                  (long long)ob);
+  (rs == 1 ? oz_slice<true> : oz_slice<false>)<<<dim3(blocks, 1, batch), 256, 0, s>>>(X, rs, ks, sx, R, K, Rp, Kp, mx,
+                                                                                     exps, S, (long long)ob);
   mpj_count_launch();
   e = cudaGetLastError();
   if (e != cudaSuccess) {
