@@ -33,9 +33,9 @@
  *
  * Environment switches (read once per process):
  *   MPJ_JACOBI_OVERLAP=0  keep the V updates of the FP32 stage-1 rounds and
- *                         of the FP64 sweeps on `stream` (by default they
- *                         run on a private side stream joined back into
- *                         `stream`);
+ *                         of the FP64 sweeps, and the stage-1 updates of A, on
+ *                         `stream` (by default they run on private side
+ *                         streams joined back into `stream`);
  *   MPJ_STAGE1_GRAPH=0    enqueue the stage-1 sweeps kernel by kernel (by
  *                         default one sweep is captured once per workspace
  *                         as a CUDA graph and replayed);

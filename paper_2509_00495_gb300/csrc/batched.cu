@@ -1,7 +1,8 @@
 // batched.cu -- many independent symmetric eigenproblems (sizes 1..256): the C
 // entry point, and the solve with one thread group per matrix in one persistent
-// launch that MPJ_BATCHED_GROUP selects (the default is batched_rounds.cu).  Not in the paper: each matrix runs the mixed method of
-// Algorithm 9 (Sec. 5.1) on its own, inside one thread group.
+// launch that MPJ_BATCHED_GROUP selects (the default is batched_rounds.cu).  Not
+// in the paper: each matrix runs the mixed method of Algorithm 9 (Sec. 5.1) on
+// its own, inside one thread group.
 //
 // A CTA of 1024 threads holds 1024/G groups of G threads (G = 256, 512 or
 // 1024, picked by the autotuner below); each group pulls matrix indices from
@@ -25,7 +26,7 @@
 // 2 FP64 FMA per clock per SM, so the batch costs at least its total FP64
 // work over 152 SMs; barrier-separated rounds add latency on top.
 //
-// Planning and replay: the first call for a given batch (sizes, pointer
+// Planning and replay (of this form): the first call for a given batch (sizes, pointer
 // arrays, tolerance) allocates the workspace, sorts the queue, picks G (timed
 // on the batch itself unless a cached choice exists for its size histogram)
 // and captures [queue reset, kernel, result copies] in a CUDA graph; later
@@ -648,7 +649,7 @@ extern "C" int mpj_syev_batched(int batch, const int* n_host, const double* cons
   for (int i = 0; i < batch; ++i)
     if (n_host[i] < 1 || n_host[i] > NMAX) return MPJ_EINVAL;
   // One thread group per matrix only on request: the round-by-round solve is
-  // faster for large batches (2048 matrices of 8 .. 256: 141 against 446 ms) and
+  // faster for large batches (2048 matrices of 8 .. 256: 125 against 446 ms) and
   // level for the smallest (200 of 8 .. 48: 1.8 ms both), where it needs no
   // tuning runs before the first solve.
   if (!getenv("MPJ_BATCHED_GROUP")) return mpj_batched_rounds(batch, n_host, A_dev, W_dev, Q_dev, tol, sweeps_host, s);

@@ -9,9 +9,10 @@
 // disjoint block pairs P = (I, J) each run one inner round-robin sweep (31
 // inner rounds of 16 disjoint pairs) over the 32 indices of I u J on their
 // 32 x 32 diagonal subproblem A[P, P] in shared memory, accumulating U_P,
-// which is then made orthogonal to FP64 precision (blk_solve).  This is the rotation sequence of the block
-// round-robin ordering one rotation at a time: the subproblem's rotations
-// depend only on its own entries, and the pairs of one round are disjoint.
+// which is then made orthogonal to FP64 precision (blk_solve).  This is the
+// rotation sequence of the block round-robin ordering one rotation at a time:
+// the subproblem's rotations depend only on its own entries, and the pairs of
+// one round are disjoint.
 // The rest of the matrix then receives the round's rotations as products
 //   A <- U~^T A U~,  V <- V U~,   U~ = blockdiag(U_P) (in index-set order),
 // run as three block-diagonal right multiplications, each panel
@@ -54,8 +55,8 @@ constexpr int NSL = 7;                 // 8-bit digits per value
 constexpr int NLEV = 7;                // levels 0..6 kept
 constexpr int TM = 128;                // rows per CTA of the right multiplication
 constexpr uint32_t TMEM_COLS = 256;    // >= NLEV * 32
-constexpr int USL_BYTES = W2 * W2 * 2;          // one 32 x 32 bf16 digit tile
-constexpr int XSL_BYTES = TM * W2 * 2;          // one 128 x 32 bf16 digit tile
+constexpr int USL_BYTES = W2 * W2 * 2;          // one 32 x 32 binary16 digit tile
+constexpr int XSL_BYTES = TM * W2 * 2;          // one 128 x 32 binary16 digit tile
 constexpr long long WAIT_CYCLES = 4000000000LL;
 
 MPJ_DEV uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }

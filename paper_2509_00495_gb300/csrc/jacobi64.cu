@@ -25,7 +25,7 @@
 //    paper's row update, then column update, then vector update, with the
 //    paper's formulas.  The sweep runs as 2n - 3 wavefronts of mutually
 //    independent rotations (pairs with equal p + q), which is the same
-//    rotation sequence (see cyc_wave_update).
+//    rotation sequence (see cyc_wave).
 //
 // off(A) (Sec. 3.1, direct form) is reduced after every sweep with a fixed
 // reduction order, so repeated runs are bitwise identical.

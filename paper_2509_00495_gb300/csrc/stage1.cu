@@ -15,9 +15,9 @@
 //   A[P,Q] <- U_P^T A[P,Q] U_Q,   V[:,Q] <- V[:,Q] U_Q
 // (P, Q = index sets of block pairs) gives the same iterates as applying them
 // one by one.  Each round is the subproblem solves and two block products
-// (FP32 FMA, rmul32): V <- V U~ and A <- U~^T A U~ (the lower tiles, each
-// formed once and mirrored), so that A32 and V32 are touched once per round
-// instead of once per pair step.  off(A32) is reduced after each sweep; stop
+// (FP32 FMA, rmul32 or rmul32_pipe): V <- V U~ and A <- U~^T A U~ (the lower
+// tiles, each formed once and mirrored), so that A32 and V32 are touched once
+// per round instead of once per pair step.  off(A32) is reduced after each sweep; stop
 // at off(A32) <= tol32 or the sweep cap.
 #include <memory>
 #include <mutex>
