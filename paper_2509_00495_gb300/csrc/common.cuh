@@ -59,6 +59,16 @@ MPJ_DEV bool jacobi_pair(T app, T aqq, T apq, T skip, T& t, T& cm1, T& s, T skip
   return true;
 }
 
+// The skip test of Algorithm 4, |a_pq| > skip sqrt|a_pp a_qq|: in squares where
+// a_pq^2 is well inside the range (no root in the chain), as it stands below
+// 2^-450, where the squares would underflow and the pair would never rotate.
+// The range is read off the high word (an FP64 compare issues on the FP64 pipe).
+MPJ_DEV bool above_skip(double app, double aqq, double apq, double skip) {
+  const double a2 = apq * apq, d = fabs(app * aqq);
+  if ((__double2hiint(a2) & 0x7FF00000) >= (1023 - 900) << 20) return a2 > (skip * skip) * d;
+  return fabs(apq) > skip * sqrt(d);
+}
+
 // Special functions without subnormal handling: 19 cycles of latency on this
 // GPU against 41.
 MPJ_DEV float rcp_ftz(float x) {

@@ -556,7 +556,7 @@ struct WaveRec {
   int rot, pad;
 };
 
-// Rotation of a pair from its entries (skip rule of Algorithm 4, compared in squares).
+// Rotation of a pair from its entries (skip rule of Algorithm 4).
 MPJ_DEV WaveRec wave_rec(double app, double aqq, double apq, double skip, double skip_abs, int* __restrict__ rotated) {
   WaveRec r;
   r.c = 1.0;
@@ -566,7 +566,7 @@ MPJ_DEV WaveRec wave_rec(double app, double aqq, double apq, double skip, double
   r.apq = apq;
   r.rot = 0;
   r.pad = 0;
-  if (apq * apq > (skip * skip) * fabs(app * aqq) && fabs(apq) > skip_abs) {
+  if (above_skip(app, aqq, apq, skip) && fabs(apq) > skip_abs) {
     double t;
     jacobi_angle(aqq - app, apq, t, r.c);
     r.s = t * r.c;
