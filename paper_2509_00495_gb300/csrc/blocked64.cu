@@ -1238,16 +1238,14 @@ size_t rmul_smem() {
   // that the 512 TMEM columns hold (256 each), so no CTA waits in tcgen05.alloc
   return sizeof(RmulSmem) + 1024 > 80 * 1024 ? sizeof(RmulSmem) + 1024 : 80 * 1024;
 }
-cudaError_t rmul_attr() {
-  static bool done = false;
-  if (done) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(blk_rmul, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rmul_smem());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(blk_rmul_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rmul_smem());
-  if (e == cudaSuccess) done = true;
-  return e;
+cudaError_t rmul_attr(const void* kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rmul_smem());
 }
 }  // namespace
+
+// Before the sweeps of a call: the kernels' shared-memory limit, which belongs to
+// the current device (a limit set on one device says nothing about another).
+cudaError_t mpj_blocked_prepare() { return rmul_attr((const void*)blk_rmul); }
 
 // Round R, step 1: the subproblems of the block pairs, U_P into set R mod 2;
 // *nrot (if not null) counts the block pairs that rotated.
@@ -1277,13 +1275,11 @@ cudaError_t mpj_blocked_update_A(double* A, int lda, double* B, int n, int R, vo
   const int N = (n + 2 * BS - 1) / (2 * BS) * (2 * BS);
   const int nb = N / BS;
   const USet u = uset(scratch, n, R & 1);
-  cudaError_t e = rmul_attr();
-  if (e != cudaSuccess) return e;
   const dim3 grid((nb / 2 + 3) / 4, nb / 2);
   const int prio = rm_a_priority(s);
-  e = mpj_launch_pdl_at(prio, blk_rmul, grid, dim3(RM_THREADS), rmul_smem(), s, (const double*)A, lda, (int)XMODE_COLS,
-                        B, n, n, nb, R, (const __half*)u.sl, (const int*)u.ex, (const int*)u.rot, flags,
-                        (int)TRI_FIRST);
+  const cudaError_t e = mpj_launch_pdl_at(prio, blk_rmul, grid, dim3(RM_THREADS), rmul_smem(), s, (const double*)A,
+                                          lda, (int)XMODE_COLS, B, n, n, nb, R, (const __half*)u.sl,
+                                          (const int*)u.ex, (const int*)u.rot, flags, (int)TRI_FIRST);
   if (e != cudaSuccess) return e;
   return mpj_launch_pdl_at(prio, blk_rmul, grid, dim3(RM_THREADS), rmul_smem(), s, (const double*)B, n,
                            (int)XMODE_ROWS, A, lda, n, nb, R, (const __half*)u.sl, (const int*)u.ex,
@@ -1295,8 +1291,6 @@ cudaError_t mpj_blocked_update_V(double* V, int ldv, int n, int R, void* scratch
   const int N = (n + 2 * BS - 1) / (2 * BS) * (2 * BS);
   const int nb = N / BS;
   const USet u = uset(scratch, n, R & 1);
-  cudaError_t e = rmul_attr();
-  if (e != cudaSuccess) return e;
   const dim3 grid((nb / 2 + 3) / 4, nb / 2);
   return mpj_launch_pdl(blk_rmul, grid, dim3(RM_THREADS), rmul_smem(), s, (const double*)V, ldv, (int)XMODE_COLS, V,
                         ldv, n, nb, R, (const __half*)u.sl, (const int*)u.ex, (const int*)u.rot, flags,
@@ -1310,7 +1304,7 @@ cudaError_t mpj_batch_sweep64_round(const BatchShape& b, int R, double* A, doubl
   const int lo = batch_lowest_class(R);
   const long long subs = batch_blocks(b, lo, [](int np) { return np; });
   if (subs == 0) return cudaSuccess;
-  cudaError_t e = rmul_attr();
+  cudaError_t e = rmul_attr((const void*)blk_rmul_batch);
   if (e != cudaSuccess) return e;
   __half* sl = (__half*)digits;
   int* ex = (int*)((char*)digits + al256((size_t)pairs * NSL * USL_BYTES));

@@ -926,6 +926,7 @@ int mpj_jacobi64_run(int n, double* A, int lda, double* V, int ldv, double tol, 
     unsigned* nrot = (unsigned*)(iscal + 2);
     unsigned hflags = 0, hnrot = 0;
     MPJ_CUDA_TRY(cudaMemsetAsync(bflags, 0, 2 * sizeof(unsigned), s));
+    MPJ_CUDA_TRY(mpj_blocked_prepare());
     const int rounds = mpj_blocked_rounds_per_sweep(n);
     // V <- V U~ of round R runs on a private side stream, overlapping round
     // R+1's subproblems and A update; the U_P sets alternate between rounds,

@@ -17,6 +17,7 @@ size_t mpj_jacobi64_scratch_bytes_ordering(int n, int ordering);
 // the two updates independent of each other; the scratch they need, rounds
 // per sweep, and the end-of-sweep symmetrization.
 size_t mpj_blocked_scratch_bytes(int n);
+cudaError_t mpj_blocked_prepare();  // once before the sweeps of a call
 cudaError_t mpj_blocked_solve(const double* A, int lda, int n, int R, double skip, double skip_abs, void* scratch,
                               unsigned* nrot, cudaStream_t s);
 cudaError_t mpj_blocked_update_A(double* A, int lda, double* B, int n, int R, void* scratch, unsigned* flags,
