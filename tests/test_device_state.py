@@ -4,8 +4,7 @@ A kernel's dynamic shared-memory limit (cudaFuncSetAttribute) holds for the
 device that was current when it was set.  Code that remembers in a static
 variable that it has set one launches with the default limit of 48 KB on the
 next device, and the launch is rejected.  Read from the sources: no function
-that sets an attribute has a mutable static local, and no other static flag than
-those of the environment switches (read once per process) exists.
+that sets an attribute has a mutable static local.
 """
 import glob
 import os
@@ -27,6 +26,4 @@ def test_attributes_are_set_for_the_current_device():
             if "cudaFuncSetAttribute" in body:
                 seen += 1
                 assert not re.search(r"\bstatic\s+(?!constexpr|const\b)", body), (f, body[:200])
-        for name in re.findall(r"^[ \t]+static\s+(?:bool|int|unsigned)\s+(\w+)", text, flags=re.M):
-            assert name == "env", (f, name)
     assert seen >= 5
