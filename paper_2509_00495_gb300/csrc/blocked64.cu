@@ -310,7 +310,7 @@ MPJ_DEV void df_angle(float2 a, float2 d, float tie, float2& t, float2& c, float
 // orthogonal to 2^-59.  (The digits the products use have 2^-57.)  Entries
 // whose range does not fit pairs (more than 2^70 between the couplings, or
 // 2^100 between a coupling and the diagonal: graded matrices) run the same
-// sweep in FP64 instructions instead.
+// sweep in FP64 instructions instead (solve_wide).
 //
 // What bounds it: the chain coupling -> angle -> record -> next coupling, and
 // beside it the number of instructions a warp has to get through per round.
@@ -338,14 +338,20 @@ struct SolveSmem {
       float2 U[W2][LDS];           // U[column][row]
       float2 gap[W2 - 1][W2 / 2];  // starting a_yy - a_xx of each round's slots
     } p;
-    double U64[W2][LDS];  // FP64 form: U[column][row]
+    struct {                      // FP64 form (solve_wide)
+      double U[W2][LDS];          // U~[column][row]
+      double cs[2][W2 / 2][2];    // mx, my
+      double dg[2][W2 / 2][2];    // the pair's new true diagonal
+      double d[W2], e[W2];        // scales and their reciprocals
+      int p[2][W2 / 2], q[2][W2 / 2], rot[2][W2 / 2];
+      int slot_of[2][W2];         // pair slot of each index in the round
+    } w;
     struct {
       int u1[W2][UFL], u0[W2][UFL];  // U = (u1 + u0 2^-30) 2^-30, [column][row]
       float Ef[W2][UFL];             // E = U^T U - I
     } f;
   };
   double A[W2][LDS];      // the subproblem as loaded; FP64 form: in place
-  double cs[W2 / 2][2];   // FP64 form: c - 1, s
   float4 rec[2][W2 / 2];  // c, s oriented to the slot's (x, y)
   unsigned emax_off, emin_off, emax_dg, any;
 };
@@ -368,6 +374,130 @@ MPJ_DEV int pos_at(int i, int j) {
   const int si = i < 16 ? i : 31 - i, sj = j < 16 ? j : 31 - j;
   const int a = min(si, sj), b = max(si, sj), ea = si < sj ? i > 15 : j > 15, eb = si < sj ? j > 15 : i > 15;
   return (2 * ea + eb) * SSTR + (a * (31 - a)) / 2 + (b - a - 1);
+}
+
+// The same sweep in FP64 instructions on sm.A (both triangles), for entries whose
+// range does not fit pairs; U_P into sm.w.U, sm.any set when a pair rotates.
+// Scaled rotations: off the diagonal S = D S~ D and U = U~ D with one scale vector
+// d (and e = 1 / d), the diagonal holds the true values, so a rotation (t, c) of
+// pair p < q costs one FMA per entry and side:
+//   x_p <- x_p - mx x_q,  x_q <- x_q + my x_p  (old values),
+//   mx = t d_q / d_p,  my = t d_p / d_q,  d_p, d_q <- c d_p, c d_q.
+// Warp 0 updates the blocks that hold a pair of the next round and forms that
+// round's rotations while the other warps update the remaining blocks and U~: one
+// barrier per inner round.  An FP64 instruction is 65 cycles here, so the length
+// of warp 0's chain is the time.  Microseconds per round (with the products), n =
+// 1024, D B D with D = 2^-60 .. 1: 125; with c - 1 carried, two FMAs an entry and
+// side, divisions and roots and no looking ahead 145; this form with divisions and
+// roots 138.  (Rounds of pairs: 50.)
+MPJ_DEV void solve_wide(SolveSmem& sm, double skip, double skip_abs) {
+  auto& w = sm.w;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  for (int e = tid; e < W2 * W2; e += SOLVE_THREADS) w.U[e / W2][e % W2] = (e / W2 == e % W2) ? 1.0 : 0.0;
+  if (tid < W2) w.d[tid] = w.e[tid] = 1.0;
+  __syncthreads();
+  // the rotation of the pair in slot k of inner round rho; the pair's scales are
+  // updated here (no one else touches them this round)
+  auto rotation = [&](int rho, int k, int buf) {
+    int x, y;
+    rr_slot(W2, rho, k, x, y);
+    const int p = min(x, y), q = max(x, y);
+    const double app = sm.A[p][p], aqq = sm.A[q][q], dp = w.d[p], dq = w.d[q], apq = sm.A[p][q] * dp * dq;
+    double mx = 0.0, my = 0.0;
+    const bool rot = above_skip(app, aqq, apq, skip) && fabs(apq) > skip_abs;
+    if (rot) {
+      double t, c;
+      jacobi_angle(aqq - app, apq, t, c);
+      const double h = fma(t, t, 1.0) * c, ep = w.e[p], eq = w.e[q];  // h = 1 / c
+      mx = t * dq * ep;
+      my = t * dp * eq;
+      w.d[p] = dp * c;
+      w.d[q] = dq * c;
+      w.e[p] = ep * h;
+      w.e[q] = eq * h;
+      w.dg[buf][k][0] = app - t * apq;
+      w.dg[buf][k][1] = aqq + t * apq;
+      sm.any = 1u;
+    }
+    w.cs[buf][k][0] = mx;
+    w.cs[buf][k][1] = my;
+    w.rot[buf][k] = rot;
+    w.p[buf][k] = p;
+    w.q[buf][k] = q;
+    w.slot_of[buf][p] = k;
+    w.slot_of[buf][q] = k;
+  };
+  // the 2 x 2 block between slots a and b: rows by a's rotation, columns by b's,
+  // the mirror block the same values
+  auto block = [&](int a, int b, int buf) {
+    if (!w.rot[buf][a] && !w.rot[buf][b]) return;
+    const int pa = w.p[buf][a], qa = w.q[buf][a], pb = w.p[buf][b], qb = w.q[buf][b];
+    const double mxa = w.cs[buf][a][0], mya = w.cs[buf][a][1], mxb = w.cs[buf][b][0], myb = w.cs[buf][b][1];
+    const double b00 = sm.A[pa][pb], b01 = sm.A[pa][qb], b10 = sm.A[qa][pb], b11 = sm.A[qa][qb];
+    const double t00 = fma(-mxa, b10, b00), t10 = fma(mya, b00, b10);
+    const double t01 = fma(-mxa, b11, b01), t11 = fma(mya, b01, b11);
+    sm.A[pa][pb] = sm.A[pb][pa] = fma(-mxb, t01, t00);
+    sm.A[pa][qb] = sm.A[qb][pa] = fma(myb, t00, t01);
+    sm.A[qa][pb] = sm.A[pb][qa] = fma(-mxb, t11, t10);
+    sm.A[qa][qb] = sm.A[qb][qa] = fma(myb, t10, t11);
+  };
+  if (warp == 0 && lane < W2 / 2) rotation(0, lane, 0);
+  __syncthreads();
+#pragma unroll 1
+  for (int rho = 0; rho < W2 - 1; ++rho) {
+    const int cur = rho & 1;
+    const bool more = rho + 1 < W2 - 1;
+    if (warp == 0) {
+      if (lane < W2 / 2) {  // the pairs' own blocks: new diagonal, no coupling
+        if (w.rot[cur][lane]) {
+          const int p = w.p[cur][lane], q = w.q[cur][lane];
+          sm.A[p][p] = w.dg[cur][lane][0];
+          sm.A[q][q] = w.dg[cur][lane][1];
+          sm.A[p][q] = sm.A[q][p] = 0.0;
+        }
+      } else if (more) {  // the block that holds the next round's pair lane - 16
+        int x, y;
+        rr_slot(W2, rho + 1, lane - W2 / 2, x, y);
+        if (w.slot_of[cur][x] > w.slot_of[cur][y]) {
+          const int t = x;
+          x = y;
+          y = t;
+        }
+        const int a = w.slot_of[cur][x], b = w.slot_of[cur][y];
+        // two next pairs may share a block: the smaller index of a takes it
+        const int o = w.p[cur][a] == x ? w.q[cur][a] : w.p[cur][a];
+        const bool twice = w.slot_of[cur][rr_partner(W2, rho + 1, o)] == b;
+        if (a != b && (!twice || x < o)) block(a, b, cur);
+      }
+      __syncwarp();
+      if (more && lane < W2 / 2) rotation(rho + 1, lane, cur ^ 1);
+    } else {
+      for (int task = tid - 32; task < 120 + (W2 / 2) * W2; task += SOLVE_THREADS - 32) {
+        if (task < 120) {
+          int a = 0, rem = task;
+          while (rem >= 15 - a) {
+            rem -= 15 - a;
+            ++a;
+          }
+          const int b = a + 1 + rem;
+          // a block that holds a pair of the next round is warp 0's
+          if (more && (w.slot_of[cur][rr_partner(W2, rho + 1, w.p[cur][a])] == b ||
+                       w.slot_of[cur][rr_partner(W2, rho + 1, w.q[cur][a])] == b))
+            continue;
+          block(a, b, cur);
+        } else {
+          const int k = (task - 120) / W2, j = (task - 120) % W2;
+          if (!w.rot[cur][k]) continue;
+          double &up = w.U[w.p[cur][k]][j], &uq = w.U[w.q[cur][k]][j];
+          const double u0 = up, u1 = uq;
+          up = fma(-w.cs[cur][k][0], u1, u0);
+          uq = fma(w.cs[cur][k][1], u0, u1);
+        }
+      }
+    }
+    __syncthreads();
+  }
+  for (int e = tid; e < W2 * W2; e += SOLVE_THREADS) w.U[e / W2][e % W2] *= w.d[e / W2];
 }
 
 // One subproblem: pair P of round R of a matrix, and where its digits,
@@ -641,58 +771,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS, CTAS) blk_solve(Src src, int R,
   } else {
     __syncthreads();
     if (tid == 0) sm.any = 0u;  // read by all above
-    // the same sweep in FP64 instructions (c - 1 carried separately)
-    for (int e = tid; e < W2 * W2; e += SOLVE_THREADS) sm.U64[e / W2][e % W2] = (e / W2 == e % W2) ? 1.0 : 0.0;
-    __syncthreads();
-#pragma unroll 1
-    for (int rho = 0; rho < W2 - 1; ++rho) {
-      if (tid < W2 / 2) {
-        int x, y;
-        rr_slot(W2, rho, tid, x, y);
-        double t, cm1, s;
-        const int pi = min(x, y), qi = max(x, y);
-        const double apq = sm.A[pi][qi];
-        const bool rot = jacobi_pair<double>(sm.A[pi][pi], sm.A[qi][qi], apq, skip, t, cm1, s, skip_abs);
-        if (rot) {
-          sm.any = 1u;
-          sm.A[pi][pi] -= t * apq;
-          sm.A[qi][qi] += t * apq;
-          sm.A[pi][qi] = 0.0;
-          sm.A[qi][pi] = 0.0;
-        }
-        sm.cs[tid][0] = cm1;
-        sm.cs[tid][1] = x < y ? s : -s;
-      }
-      __syncthreads();
-      for (int task = tid; task < 120 + (W2 / 2) * W2; task += SOLVE_THREADS) {
-        if (task < 120) {
-          int a = 0, rem = task;
-          while (rem >= 15 - a) {
-            rem -= 15 - a;
-            ++a;
-          }
-          const int b = a + 1 + rem;
-          int xa, ya, xb, yb;
-          rr_slot(W2, rho, a, xa, ya);
-          rr_slot(W2, rho, b, xb, yb);
-          double v00 = sm.A[xa][xb], v01 = sm.A[xa][yb], v10 = sm.A[ya][xb], v11 = sm.A[ya][yb];
-          rot_apply(sm.cs[a][0], sm.cs[a][1], v00, v10);
-          rot_apply(sm.cs[a][0], sm.cs[a][1], v01, v11);
-          rot_apply(sm.cs[b][0], sm.cs[b][1], v00, v01);
-          rot_apply(sm.cs[b][0], sm.cs[b][1], v10, v11);
-          sm.A[xa][xb] = sm.A[xb][xa] = v00;
-          sm.A[xa][yb] = sm.A[yb][xa] = v01;
-          sm.A[ya][xb] = sm.A[xb][ya] = v10;
-          sm.A[ya][yb] = sm.A[yb][ya] = v11;
-        } else {
-          const int e = task - 120, k = e / W2, j = e % W2;
-          int x, y;
-          rr_slot(W2, rho, k, x, y);
-          rot_apply(sm.cs[k][0], sm.cs[k][1], sm.U64[x][j], sm.U64[y][j]);
-        }
-      }
-      __syncthreads();
-    }
+    solve_wide(sm, skip, skip_abs);
   }
   __syncthreads();
   if (!sm.any) {
@@ -715,7 +794,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS, CTAS) blk_solve(Src src, int R,
       u1[it] = ah + al + carry;
       u0[it] = b - (carry << 30);
     } else {
-      const long long F = __double2ll_rn(sm.U64[col][row] * 0x1p60);
+      const long long F = __double2ll_rn(sm.w.U[col][row] * 0x1p60);
       const long long t = (F + (1LL << 29)) >> 30;
       u1[it] = (int)t;
       u0[it] = (int)(F - (t << 30));

@@ -26,7 +26,7 @@ def m():
 
 
 @pytest.mark.parametrize("p,q", list(itertools.combinations(range(5), 2)))
-@pytest.mark.parametrize("ordering", ["cyclic", "round_robin"])
+@pytest.mark.parametrize("ordering", ["cyclic", "round_robin", "block"])
 def test_small_pair_rotates(m, ordering, p, q):
     i, j, k = (x for x in range(5) if x not in (p, q))
     A = np.zeros((5, 5))
