@@ -176,11 +176,11 @@ int mpj_syev_ex(int n, const double* A_dev, int lda, double* W_dev, double* Q_de
  * matrix.
  * All matrices go through the rounds of a stage together, one launch per step
  * of a round; those that have converged drop out.  The first call for a list
- * of sizes plans: it orders the matrices by decreasing size and allocates a
- * workspace with cudaMalloc (at most about 6 GB: larger batches run in
- * several parts).  Later calls with the same sizes reuse it, whatever the
- * pointers.  Up to 4 plans are kept (mpj_release_plans frees them); calls
- * from several threads run one after the other.  Synchronizes `stream` (once
+ * of sizes plans on the host (it orders the matrices by decreasing size).  The
+ * workspace, at most about 6 GB, comes from cudaMalloc, grows to the largest
+ * batch so far and is kept, one per device, until mpj_release_plans; larger
+ * batches, and those for which that memory cannot be had, run in several parts.
+ * Calls from several threads run one after the other.  Synchronizes `stream` (once
  * per sweep, to read how many matrices still need one, and at the end), so it
  * cannot be stream-captured.
  * With MPJ_BATCHED_GROUP set, one thread group solves each matrix in one
@@ -193,7 +193,7 @@ int mpj_syev_ex(int n, const double* A_dev, int lda, double* W_dev, double* Q_de
 int mpj_syev_batched(int batch, const int* n_host, const double* const* A_dev, double* const* W_dev,
                      double* const* Q_dev, double tol, int* sweeps_host, void* stream);
 
-/* Frees the workspaces and graphs of all cached batched plans and returns the
+/* Frees the workspaces and graphs of the batched solves and returns the
  * memory that the library's pools keep between calls. */
 void mpj_release_plans(void);
 

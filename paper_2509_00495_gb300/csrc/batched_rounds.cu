@@ -185,27 +185,54 @@ Layout layout(const Chunk& c) {
   return L;
 }
 
+// How a list of sizes is solved: places by decreasing size, cut into chunks.
 struct Plan {
-  int device = -1;
-  std::vector<int> sizes;
+  std::vector<int> sizes, order, n_place;
   std::vector<Chunk> chunks;
-  void* work = nullptr;
-  void* small = nullptr;
+  size_t work = 0;  // bytes of the largest chunk
+};
+// What a device keeps between calls, which run one after the other: the last
+// plan, and memory grown to the largest one so far (a workspace of at most
+// kChunkBytes or one matrix, and some words per matrix).  Calls with changing
+// lists of sizes plan again on the host but allocate nothing once it is grown.
+struct Device {
+  int id = -1;
+  Plan plan;
+  bool uploaded = false;  // plan.order and plan.n_place are in `small`
+  void *work = nullptr, *small = nullptr;
   int* pinned = nullptr;  // count, flags, then the sweeps by matrix
-  size_t small_bytes = 0;
+  size_t work_bytes = 0, small_bytes = 0, pinned_bytes = 0;
 };
 std::mutex g_mu;
-std::vector<Plan*>& plans() {  // most recent last; never destroyed (no CUDA calls at process exit)
-  static auto* p = new std::vector<Plan*>();
-  return *p;
+std::vector<Device*>& devices() {  // never destroyed (no CUDA calls at process exit)
+  static auto* d = new std::vector<Device*>();
+  return *d;
 }
-constexpr size_t kMaxPlans = 4;
 
-void free_plan(Plan* p) {
-  if (p->work) cudaFree(p->work);
-  if (p->small) cudaFree(p->small);
-  if (p->pinned) cudaFreeHost(p->pinned);
-  delete p;
+void give_back(Device* d) {
+  if (d->work) cudaFree(d->work);
+  if (d->small) cudaFree(d->small);
+  if (d->pinned) cudaFreeHost(d->pinned);
+  delete d;
+}
+
+// *p of at least `need` bytes; what it held is lost when it has to grow.
+template <class Alloc, class Free>
+cudaError_t grow(void** p, size_t* have, size_t need, Alloc alloc, Free release) {
+  if (*have >= need) return cudaSuccess;
+  if (*p) release(*p);
+  *p = nullptr;
+  *have = 0;
+  const cudaError_t e = alloc(p, need);
+  mpj_count_alloc();
+  if (e == cudaSuccess)
+    *have = need;
+  else
+    (void)cudaGetLastError();
+  return e;
+}
+cudaError_t grow_device(void** p, size_t* have, size_t need) {
+  return grow(p, have, need, [](void** q, size_t b) { return cudaMalloc(q, b); }, [](void* q) { cudaFree(q); });
 }
 
 // The small area: order, n by place, then the state by place, count and flags,
@@ -240,39 +267,37 @@ Small small_ptrs(char* b, int batch) {
 
 int class_of(int n) { return (n + 31) / 32 - 1; }
 
-int make_plan(int dev, int batch, const int* n_host, Plan** out) {
-  Plan* p = new Plan;
-  p->device = dev;
+// The plan of a list of sizes with chunks of at most `limit` bytes (at least one
+// matrix each).
+void make_plan(int batch, const int* n_host, size_t limit, Plan* p) {
   p->sizes.assign(n_host, n_host + batch);
+  p->order.resize(batch);
+  p->n_place.resize(batch);
+  p->chunks.clear();
+  p->work = 0;
   // decreasing size class, then decreasing n (counting sort), ties by index
-  std::vector<int> order(batch), n_place(batch);
-  {
-    std::vector<int> start(BATCH_NMAX + 2, 0);
-    int cnt[BATCH_NMAX + 1] = {0};
-    for (int i = 0; i < batch; ++i) cnt[n_host[i]]++;
-    int acc = 0;
-    for (int v = BATCH_NMAX; v >= 1; --v) {
-      start[v] = acc;
-      acc += cnt[v];
-    }
-    for (int i = 0; i < batch; ++i) order[start[n_host[i]]++] = i;
-    for (int i = 0; i < batch; ++i) n_place[i] = n_host[order[i]];
+  int start[BATCH_NMAX + 1], cnt[BATCH_NMAX + 1] = {0};
+  for (int i = 0; i < batch; ++i) cnt[n_host[i]]++;
+  for (int v = BATCH_NMAX, acc = 0; v >= 1; --v) {
+    start[v] = acc;
+    acc += cnt[v];
   }
-  size_t work = 0;
+  for (int i = 0; i < batch; ++i) p->order[start[n_host[i]]++] = i;
+  for (int i = 0; i < batch; ++i) p->n_place[i] = n_host[p->order[i]];
   for (int p0 = 0; p0 < batch;) {
     Chunk c;
     memset(&c, 0, sizeof c);
     c.p0 = p0;
-    c.cmax = class_of(n_place[p0]);
+    c.cmax = class_of(p->n_place[p0]);
     int cls = -1;
     for (int i = p0; i < batch; ++i) {
-      const int k = class_of(n_place[i]), N = 32 * (k + 1);
+      const int k = class_of(p->n_place[i]), N = 32 * (k + 1);
       Chunk d = c;
       d.count += 1;
       d.el += (long long)N * N;
       d.oz += 8LL * batch_rp(N) * N;
       d.pairs += k + 1;
-      if (c.count > 0 && layout(d).total > kChunkBytes) break;
+      if (c.count > 0 && layout(d).total > limit) break;
       if (k != cls) {
         cls = k;
         d.shape.first[k] = i - p0;
@@ -284,41 +309,55 @@ int make_plan(int dev, int batch, const int* n_host, Plan** out) {
       c = d;
     }
     const size_t t = layout(c).total;
-    if (t > work) work = t;
+    if (t > p->work) p->work = t;
     p->chunks.push_back(c);
     p0 += c.count;
   }
-  p->small_bytes = small_ptrs(nullptr, batch).total;
-  cudaError_t e = cudaMalloc(&p->work, work);
-  mpj_count_alloc();
-  if (e == cudaSuccess) e = cudaMalloc(&p->small, p->small_bytes);
-  mpj_count_alloc();
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&p->pinned, sizeof(int) * ((size_t)batch + 2));
-  mpj_count_alloc();
-  if (e != cudaSuccess) {
-    mpj_set_cuda_error(e, "batched plan allocation", __LINE__);
-    (void)cudaGetLastError();
-    free_plan(p);
-    return MPJ_ENOMEM;
+}
+
+// The plan and its memory on the device.  Where the memory for chunks of
+// kChunkBytes cannot be had, the batch is cut into smaller ones (until other
+// sizes are planned or the memory is given back), down to single matrices.
+int prepare(Device* d, int batch, const int* n_host, cudaStream_t s) {
+  const bool same = (int)d->plan.sizes.size() == batch &&
+                    memcmp(d->plan.sizes.data(), n_host, sizeof(int) * (size_t)batch) == 0;
+  if (!same || !d->uploaded) {
+    d->uploaded = false;
+    cudaError_t e = cudaSuccess;
+    for (size_t limit = kChunkBytes;; limit = d->plan.work / 2) {
+      make_plan(batch, n_host, limit, &d->plan);
+      e = grow_device(&d->work, &d->work_bytes, d->plan.work);
+      if (e != cudaErrorMemoryAllocation || (int)d->plan.chunks.size() == batch) break;
+    }
+    const size_t small = small_ptrs(nullptr, batch).total, pinned = sizeof(int) * ((size_t)batch + 2);
+    if (e == cudaSuccess) e = grow_device(&d->small, &d->small_bytes, small);
+    if (e == cudaSuccess)
+      e = grow((void**)&d->pinned, &d->pinned_bytes, pinned, [](void** q, size_t b) { return cudaMallocHost(q, b); },
+               [](void* q) { cudaFreeHost(q); });
+    if (e != cudaSuccess) {
+      mpj_set_cuda_error(e, "batched plan allocation", __LINE__);
+      return MPJ_ENOMEM;
+    }
+    const Small sm = small_ptrs((char*)d->small, batch);
+    e = cudaMemcpyAsync(sm.order, d->plan.order.data(), sizeof(int) * (size_t)batch, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(sm.n, d->plan.n_place.data(), sizeof(int) * (size_t)batch, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) {
+      mpj_set_cuda_error(e, "batched plan upload", __LINE__);
+      return MPJ_ECUDA;
+    }
+    for (Chunk& c : d->plan.chunks) c.shape.n = sm.n + c.p0;
+    d->uploaded = true;
   }
-  const Small sm = small_ptrs((char*)p->small, batch);
-  e = cudaMemcpy(sm.order, order.data(), sizeof(int) * (size_t)batch, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(sm.n, n_place.data(), sizeof(int) * (size_t)batch, cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) {
-    mpj_set_cuda_error(e, "batched plan upload", __LINE__);
-    free_plan(p);
-    return MPJ_ECUDA;
-  }
-  for (Chunk& c : p->chunks) c.shape.n = sm.n + c.p0;
-  *out = p;
   return MPJ_OK;
 }
 
 // One chunk on stream s; *not_converged is set when a sweep cap was reached
 // with a matrix above its tolerance.
-int run_chunk(const Plan& p, const Chunk& c, const double* const* A, double* const* W, double* const* Q, double tol,
+int run_chunk(const Device& d, const Chunk& c, const double* const* A, double* const* W, double* const* Q, double tol,
               bool* not_converged, cudaStream_t s) {
-  const Small sm0 = small_ptrs((char*)p.small, (int)p.sizes.size());
+  const Small sm0 = small_ptrs((char*)d.small, (int)d.plan.sizes.size());
   State st = sm0.st;
   st.active += c.p0;
   st.sweeps += c.p0;
@@ -327,7 +366,7 @@ int run_chunk(const Plan& p, const Chunk& c, const double* const* A, double* con
   st.skip_abs += c.p0;
   const int* order = sm0.order + c.p0;
   const Layout L = layout(c);
-  char* w = (char*)p.work;
+  char* w = (char*)d.work;
   double *X = (double*)(w + L.X), *M = (double*)(w + L.M), *Y = (double*)(w + L.Y);
   float *A32 = (float*)(w + L.A32), *V32 = (float*)(w + L.V32), *S = (float*)(w + L.S), *U = (float*)(w + L.U);
   const BatchOperand o0{(__nv_bfloat16*)(w + L.oz[0]), (int*)(w + L.ozx[0])};
@@ -336,7 +375,7 @@ int run_chunk(const Plan& p, const Chunk& c, const double* const* A, double* con
   all.active = nullptr;
   act.active = st.active;
   const int rounds = 2 * c.cmax + 1;
-  int* h_count = p.pinned;
+  int* h_count = d.pinned;
   // the number of matrices that need another sweep
   auto count = [&](auto check) -> cudaError_t {
     cudaError_t e = cudaMemsetAsync(sm0.count, 0, sizeof(int), s);
@@ -401,47 +440,41 @@ int run_chunk(const Plan& p, const Chunk& c, const double* const* A, double* con
 
 void mpj_batched_rounds_release() {
   std::lock_guard<std::mutex> lock(g_mu);
-  for (Plan* p : plans()) free_plan(p);
-  plans().clear();
+  for (Device* d : devices()) give_back(d);
+  devices().clear();
 }
 
 int mpj_batched_rounds(int batch, const int* n_host, const double* const* A_dev, double* const* W_dev,
                        double* const* Q_dev, double tol, int* sweeps_host, cudaStream_t s) {
   int dev = 0;
   MPJ_CUDA_TRY(cudaGetDevice(&dev));
-  std::lock_guard<std::mutex> lock(g_mu);  // the plan's workspace serves one call at a time
-  Plan* plan = nullptr;
-  auto& reg = plans();
-  for (size_t i = 0; i < reg.size(); ++i)
-    if (reg[i]->device == dev && (int)reg[i]->sizes.size() == batch &&
-        memcmp(reg[i]->sizes.data(), n_host, sizeof(int) * (size_t)batch) == 0)
-      plan = reg[i];
-  if (!plan) {
-    const int st = make_plan(dev, batch, n_host, &plan);
-    if (st != MPJ_OK) return st;
-    if (reg.size() >= kMaxPlans) {
-      free_plan(reg.front());
-      reg.erase(reg.begin());
-    }
-    reg.push_back(plan);
+  std::lock_guard<std::mutex> lock(g_mu);  // a device's memory serves one call at a time
+  Device* d = nullptr;
+  for (Device* x : devices())
+    if (x->id == dev) d = x;
+  if (!d) {
+    d = new Device;
+    d->id = dev;
+    devices().push_back(d);
   }
-  const Small sm = small_ptrs((char*)plan->small, batch);
+  int st = prepare(d, batch, n_host, s);
+  if (st != MPJ_OK) return st;
+  const Small sm = small_ptrs((char*)d->small, batch);
   MPJ_CUDA_TRY(cudaMemsetAsync(sm.flags, 0, sizeof(unsigned), s));
   bool not_converged = false;
-  int st = MPJ_OK;
-  for (const Chunk& c : plan->chunks) {
-    st = run_chunk(*plan, c, A_dev, W_dev, Q_dev, tol, &not_converged, s);
+  for (const Chunk& c : d->plan.chunks) {
+    st = run_chunk(*d, c, A_dev, W_dev, Q_dev, tol, &not_converged, s);
     if (st != MPJ_OK) break;
   }
   if (st != MPJ_OK) {
     (void)cudaStreamSynchronize(s);  // nothing of this call may still use the workspace
     return st;
   }
-  MPJ_CUDA_TRY(cudaMemcpyAsync(plan->pinned + 1, sm.flags, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
-  MPJ_CUDA_TRY(cudaMemcpyAsync(plan->pinned + 2, sm.sweeps_out, sizeof(int) * (size_t)batch, cudaMemcpyDeviceToHost, s));
+  MPJ_CUDA_TRY(cudaMemcpyAsync(d->pinned + 1, sm.flags, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+  MPJ_CUDA_TRY(cudaMemcpyAsync(d->pinned + 2, sm.sweeps_out, sizeof(int) * (size_t)batch, cudaMemcpyDeviceToHost, s));
   MPJ_CUDA_TRY(cudaStreamSynchronize(s));
-  if (sweeps_host) memcpy(sweeps_host, plan->pinned + 2, sizeof(int) * (size_t)batch);
-  const unsigned flags = (unsigned)plan->pinned[1];
+  if (sweeps_host) memcpy(sweeps_host, d->pinned + 2, sizeof(int) * (size_t)batch);
+  const unsigned flags = (unsigned)d->pinned[1];
   if (flags & MPJ_FLAG_NONFINITE) return MPJ_ENONFINITE;
   if (flags & MPJ_FLAG_TIMEOUT) return MPJ_ETIMEOUT;
   return not_converged ? MPJ_NOT_CONVERGED : MPJ_OK;
