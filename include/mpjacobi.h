@@ -175,7 +175,9 @@ int mpj_syev_ex(int n, const double* A_dev, int lda, double* W_dev, double* Q_de
  * the FP64 sweep count per matrix.  tol <= 0 selects n_i 2^-53 ||A_i||_F per
  * matrix.
  * All matrices go through the rounds of a stage together, one launch per step
- * of a round; those that have converged drop out.  The first call for a list
+ * of a round, and those that have converged drop out; batches of small matrices
+ * (all n_i <= 64, by an estimate of both) are solved with one thread group per
+ * matrix in one launch.  The first call for a list
  * of sizes plans on the host (it orders the matrices by decreasing size).  The
  * workspace, at most about 6 GB, comes from cudaMalloc, grows to the largest
  * batch so far and is kept, one per device, until mpj_release_plans; larger
@@ -183,8 +185,8 @@ int mpj_syev_ex(int n, const double* A_dev, int lda, double* W_dev, double* Q_de
  * Calls from several threads run one after the other.  Synchronizes `stream` (once
  * per sweep, to read how many matrices still need one, and at the end), so it
  * cannot be stream-captured.
- * With MPJ_BATCHED_GROUP set, one thread group solves each matrix in one
- * persistent launch instead; its plan also keeps the pointer arrays, the
+ * With MPJ_BATCHED_GROUP set, one thread group solves each matrix whatever the
+ * sizes; the plan then also keeps its workspace, the pointer arrays, the
  * group size (fixed, or picked by timing 256, 512 and 1024 threads on this
  * batch unless the size histogram was tuned before, see MPJ_AUTOTUNE_CACHE)
  * and a CUDA graph of the launch.

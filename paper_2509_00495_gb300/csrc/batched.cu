@@ -1,8 +1,8 @@
 // batched.cu -- many independent symmetric eigenproblems (sizes 1..256): the C
 // entry point, and the solve with one thread group per matrix in one persistent
-// launch that MPJ_BATCHED_GROUP selects (the default is batched_rounds.cu).  Not
-// in the paper: each matrix runs the mixed method of Algorithm 9 (Sec. 5.1) on
-// its own, inside one thread group.
+// launch, taken for batches of small matrices (the others go round by round, see
+// batched_rounds.cu) and for all when MPJ_BATCHED_GROUP is set.  Not in the paper:
+// each matrix runs the mixed method of Algorithm 9 (Sec. 5.1) on its own.
 //
 // A CTA of 1024 threads holds 1024/G groups of G threads (G = 256, 512 or
 // 1024, picked by the autotuner below); each group pulls matrix indices from
@@ -26,7 +26,7 @@
 // 2 FP64 FMA per clock per SM, so the batch costs at least its total FP64
 // work over 152 SMs; barrier-separated rounds add latency on top.
 //
-// Planning and replay (of this form): the first call for a given batch (sizes, pointer
+// Planning and replay (with MPJ_BATCHED_GROUP): the first call for a given batch (sizes, pointer
 // arrays, tolerance) allocates the workspace, sorts the queue, picks G (timed
 // on the batch itself unless a cached choice exists for its size histogram)
 // and captures [queue reset, kernel, result copies] in a CUDA graph; later
@@ -357,15 +357,17 @@ MPJ_DEV double grp_off2(const Grp& g, int n, const T* A, double* red) {
   return group_sum(g, s, red);
 }
 
-size_t group_bytes() {
-  return 2 * (size_t)NMAX * NMAX * sizeof(float) + 3 * (size_t)NMAX * NMAX * sizeof(double);
-}
+// Elements of a group's buffer for one matrix (order at most nmax), and the bytes
+// of a group's five buffers.
+size_t group_cap(int nmax) { return ((size_t)nmax * nmax + 31) & ~(size_t)31; }
+size_t group_bytes(int nmax) { return group_cap(nmax) * (2 * sizeof(float) + 3 * sizeof(double)); }
 
+// order, nvec: matrix and size by place in the queue; cap: elements per buffer.
 template <int G>
 __global__ void __launch_bounds__(NTH, 1)
     batched_syev(const int* __restrict__ order, const int* __restrict__ nvec, const double* const* __restrict__ Aptr,
                  double* const* __restrict__ Wptr, double* const* __restrict__ Qptr, int batch, double tol_in,
-                 int max32, int max64, int ns_steps, char* __restrict__ work, size_t per_group,
+                 int max32, int max64, int ns_steps, char* __restrict__ work, size_t cap,
                  int* __restrict__ counter, int* __restrict__ sweeps_out, unsigned* __restrict__ flags,
                  int region) {
   constexpr int NG = NTH / G;
@@ -383,13 +385,13 @@ __global__ void __launch_bounds__(NTH, 1)
   g.t = threadIdx.x % G;
   g.n = G;
   g.bar = 1 + g.id;
-  char* base = work + ((size_t)blockIdx.x * NG + g.id) * per_group;
+  char* base = work + ((size_t)blockIdx.x * NG + g.id) * cap * (2 * sizeof(float) + 3 * sizeof(double));
   Bufs B;
   B.A32 = (float*)base;
-  B.V32 = B.A32 + NMAX * NMAX;
-  B.X = (double*)(base + 2 * (size_t)NMAX * NMAX * sizeof(float));
-  B.M = B.X + NMAX * NMAX;
-  B.Y = B.M + NMAX * NMAX;
+  B.V32 = B.A32 + cap;
+  B.X = (double*)(base + 2 * cap * sizeof(float));
+  B.M = B.X + cap;
+  B.Y = B.M + cap;
   const int tid = g.t;
   for (;;) {
     if (tid == 0) job[g.id] = atomicAdd(counter, 1);
@@ -398,7 +400,7 @@ __global__ void __launch_bounds__(NTH, 1)
     gsync(g);
     if (jb >= batch) break;
     const int idx = order[jb];
-    const int n = nvec[idx];
+    const int n = nvec[jb];
     const double* A = Aptr[idx];
     double* W = Wptr[idx];
     double* Q = Qptr[idx];
@@ -599,14 +601,25 @@ struct Layout {
 
 Layout layout_for(int batch, int grid) {
   Layout L;
-  size_t per_group = group_bytes();
-  L.groups_bytes = per_group * (size_t)grid * MAXG;  // enough for the smallest group size
+  L.groups_bytes = group_bytes(NMAX) * (size_t)grid * MAXG;  // enough for the smallest group size
   L.order = L.groups_bytes;
   L.nvec = L.order + (((size_t)batch * sizeof(int) + 255) & ~(size_t)255);
   L.sweeps = L.nvec + (((size_t)batch * sizeof(int) + 255) & ~(size_t)255);
   L.counter = L.sweeps + (((size_t)batch * sizeof(int) + 255) & ~(size_t)255);
   L.total = L.counter + 256;
   return L;
+}
+
+cudaError_t launch_groups(int G, int grid, int nmax, const int* order, const int* n, const double* const* A,
+                          double* const* W, double* const* Q, int batch, double tol, void* work, int* counter,
+                          int* sweeps, unsigned* flags, cudaStream_t s) {
+  int region = 0;
+  size_t dyn = 0;
+  const cudaError_t e = stage1_smem(kernel_for(G), G, &region, &dyn);
+  if (e != cudaSuccess) return e;
+  kernel_for(G)<<<grid, NTH, dyn, s>>>(order, n, A, W, Q, batch, tol, 15, 30, 2, (char*)work, group_cap(nmax), counter,
+                                       sweeps, flags, region);
+  return cudaGetLastError();
 }
 
 cudaError_t enqueue(const Plan* p, const Layout& L, const double* const* A, double* const* W, double* const* Q,
@@ -616,15 +629,9 @@ cudaError_t enqueue(const Plan* p, const Layout& L, const double* const* A, doub
   unsigned* d_flags = (unsigned*)(d_counter + 1);
   cudaError_t e = cudaMemsetAsync(d_counter, 0, 2 * sizeof(int), s);
   if (e != cudaSuccess) return e;
-  int region = 0;
-  size_t dyn = 0;
-  e = stage1_smem(kernel_for(G), G, &region, &dyn);
-  if (e != cudaSuccess) return e;
-  kernel_for(G)<<<p->grid, NTH, dyn, s>>>((const int*)(base + L.order), (const int*)(base + L.nvec), A, W, Q, p->batch,
-                                          p->tol, 15, 30, 2, base, group_bytes(), d_counter, (int*)(base + L.sweeps),
-                                          d_flags, region);
+  e = launch_groups(G, p->grid, NMAX, (const int*)(base + L.order), (const int*)(base + L.nvec), A, W, Q, p->batch,
+                    p->tol, base, d_counter, (int*)(base + L.sweeps), d_flags, s);
   if (count) mpj_count_launch();
-  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   e = cudaMemcpyAsync(p->h_sweeps, base + L.sweeps, sizeof(int) * p->batch, cudaMemcpyDeviceToHost, s);
   if (e != cudaSuccess) return e;
@@ -632,6 +639,15 @@ cudaError_t enqueue(const Plan* p, const Layout& L, const double* const* A, doub
 }
 
 }  // namespace
+
+size_t mpj_batched_groups_bytes(int G, int grid, int nmax) { return group_bytes(nmax) * (size_t)grid * (NTH / G); }
+
+cudaError_t mpj_batched_groups(int G, int grid, int nmax, const int* order, const int* n, const double* const* A,
+                               double* const* W, double* const* Q, int batch, double tol, void* work, int* counter,
+                               int* sweeps, unsigned* flags, cudaStream_t s) {
+  mpj_count_launch();
+  return launch_groups(G, grid, nmax, order, n, A, W, Q, batch, tol, work, counter, sweeps, flags, s);
+}
 
 extern "C" void mpj_release_plans(void) {
   mpj_release_pools();
@@ -648,10 +664,8 @@ extern "C" int mpj_syev_batched(int batch, const int* n_host, const double* cons
   if (batch == 0) return MPJ_OK;
   for (int i = 0; i < batch; ++i)
     if (n_host[i] < 1 || n_host[i] > NMAX) return MPJ_EINVAL;
-  // One thread group per matrix only on request: the round-by-round solve is
-  // faster for large batches (2048 matrices of 8 .. 256: 125 against 446 ms) and
-  // level for the smallest (200 of 8 .. 48: 1.8 ms both), where it needs no
-  // tuning runs before the first solve.
+  // Which form: by the sizes (choose_group in batched_rounds.cu) unless the
+  // environment asks for the thread groups with their tuning and their graph.
   if (!getenv("MPJ_BATCHED_GROUP")) return mpj_batched_rounds(batch, n_host, A_dev, W_dev, Q_dev, tol, sweeps_host, s);
   int dev = 0, sms = 0;
   MPJ_CUDA_TRY(cudaGetDevice(&dev));
@@ -687,7 +701,7 @@ extern "C" int mpj_syev_batched(int batch, const int* n_host, const double* cons
       return MPJ_ENOMEM;
     }
     // longest job first: order by decreasing n (counting sort), ties by index
-    std::vector<int> order(batch);
+    std::vector<int> order(batch), n_place(batch);
     {
       int cnt[NMAX + 2] = {0}, start[NMAX + 2];
       for (int i = 0; i < batch; ++i) cnt[n_host[i]]++;
@@ -697,10 +711,11 @@ extern "C" int mpj_syev_batched(int batch, const int* n_host, const double* cons
         acc += cnt[v];
       }
       for (int i = 0; i < batch; ++i) order[start[n_host[i]]++] = i;
+      for (int i = 0; i < batch; ++i) n_place[i] = n_host[order[i]];
     }
     char* base = (char*)plan->work;
     e = cudaMemcpy(base + L.order, order.data(), sizeof(int) * (size_t)batch, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(base + L.nvec, n_host, sizeof(int) * (size_t)batch, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(base + L.nvec, n_place.data(), sizeof(int) * (size_t)batch, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
       mpj_set_cuda_error(e, "batched plan upload", __LINE__);
       free_plan(plan);

@@ -17,9 +17,11 @@
 // and SM), bound by that pipe and by the latency of the rounds; here a sweep
 // is at most 15 rounds whose subproblems of all matrices run side by side, and
 // the FP64 work is on the tensor cores.  2048 matrices, n uniform in [8, 256]:
-// 453 ms with one group per matrix, 125 ms here.
+// 453 ms with one group per matrix, 125 ms here.  Small matrices do better in
+// groups: see choose_group.
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 #include <vector>
 
@@ -189,7 +191,8 @@ Layout layout(const Chunk& c) {
 struct Plan {
   std::vector<int> sizes, order, n_place;
   std::vector<Chunk> chunks;
-  size_t work = 0;  // bytes of the largest chunk
+  size_t work = 0;         // bytes of the largest chunk
+  int group = 0, grid = 0; // one thread group of that size per matrix instead, in so many CTAs
 };
 // What a device keeps between calls, which run one after the other: the last
 // plan, and memory grown to the largest one so far (a workspace of at most
@@ -235,8 +238,8 @@ cudaError_t grow_device(void** p, size_t* have, size_t need) {
   return grow(p, have, need, [](void** q, size_t b) { return cudaMalloc(q, b); }, [](void* q) { cudaFree(q); });
 }
 
-// The small area: order, n by place, then the state by place, count and flags,
-// the sweeps by matrix.
+// The small area: order, n by place, then the state by place, then count, flags
+// and the sweeps by matrix (copied to the pinned words in one piece).
 struct Small {
   int *order, *n, *sweeps_out, *count;
   unsigned* flags;
@@ -253,19 +256,64 @@ Small small_ptrs(char* b, int batch) {
   };
   s.order = (int*)take(sizeof(int) * (size_t)batch);
   s.n = (int*)take(sizeof(int) * (size_t)batch);
-  s.sweeps_out = (int*)take(sizeof(int) * (size_t)batch);
   s.st.active = (int*)take(sizeof(int) * (size_t)batch);
   s.st.sweeps = (int*)take(sizeof(int) * (size_t)batch);
   s.st.tol = (double*)take(sizeof(double) * (size_t)batch);
   s.st.tol32 = (double*)take(sizeof(double) * (size_t)batch);
   s.st.skip_abs = (double*)take(sizeof(double) * (size_t)batch);
-  s.count = (int*)take(2 * sizeof(int));
+  s.count = (int*)take(sizeof(int) * ((size_t)batch + 2));
   s.flags = (unsigned*)(s.count + 1);
+  s.sweeps_out = s.count + 2;
   s.total = o;
   return s;
 }
 
 int class_of(int n) { return (n + 31) / 32 - 1; }
+
+// Round by round (0) or one thread group per matrix (its threads), by an estimate
+// of the milliseconds of each, for 152 SMs:
+//   a group of G threads   a n + c n^3 per matrix, a = 0.018 .. 0.0195 (the rounds' latency, their
+//                          work), as long as the slowest matrix and all of them
+//                          over the resident groups take;
+//   round by round         0.67 ms for one block pair per matrix and 0.36 for each
+//                          class more, or 0.42 and 0.23 and for each matrix 2.2 us
+//                          (n <= 32), 5.2 (n <= 64): a matrix is padded to whole
+//                          classes.
+// Batches with a matrix above n = 64 go by rounds: a group alone takes longer than
+// they do.  Measured (ms; 256, 512, 1024 threads, rounds), the coefficients fitted
+// to 110 such rows, the choice within 10 % of the best:
+//   1 x 8         0.15  0.16  0.17   0.61     152 x 24      0.86  0.63  0.54   0.76
+//   608 x 8       0.20  0.35  0.66   1.58     2048 x 24     3.19  4.08  7.00   5.08
+//   2048 x 8      0.68  1.09  2.15   4.80     200 x [8,48]  2.73  2.21  1.49   1.36
+//   1 x 32        0.72  0.70  0.72   0.68     608 x [8,48]  3.31  2.22  2.92   2.78
+//   2048 x 32     4.76  5.99  9.69   5.12     2048 x [8,48] 4.46  6.07  9.43   7.67
+//   1 x 48        1.87  1.64  1.54   0.96     2048 x [8,64] 8.33  10.4  14.7   8.80
+//   2048 x 48     13.0  15.1  20.5   11.9     2048 x [8,96] 23.2  25.3  32.6   16.4
+constexpr int kGroupMax = 64;
+int choose_group(const std::vector<int>& n_place, int sms) {
+  const int nmax = n_place.front(), cmax = class_of(nmax);
+  if (nmax > kGroupMax) return 0;
+  double work = 0.0;
+  for (int n : n_place) work += n <= 32 ? 0.0022 : 0.0052;
+  work *= 152.0 / sms;
+  double best = std::max(0.67 + 0.36 * cmax, 0.42 + 0.23 * cmax + work);
+  int form = 0;
+  const struct {
+    int threads;
+    double a, c;
+  } groups[3] = {{256, 0.018, 2.3e-5}, {512, 0.019, 1.1e-5}, {1024, 0.0195, 6e-6}};
+  for (const auto& g : groups) {
+    auto ms = [&](int n) { return g.a * n + g.c * n * n * n; };
+    double sum = 0.0;
+    for (int n : n_place) sum += ms(n);
+    const double t = std::max(ms(nmax), sum / ((double)sms * (1024 / g.threads)));
+    if (t < best) {
+      best = t;
+      form = g.threads;
+    }
+  }
+  return form;
+}
 
 // The plan of a list of sizes with chunks of at most `limit` bytes (at least one
 // matrix each).
@@ -284,6 +332,13 @@ void make_plan(int batch, const int* n_host, size_t limit, Plan* p) {
   }
   for (int i = 0; i < batch; ++i) p->order[start[n_host[i]]++] = i;
   for (int i = 0; i < batch; ++i) p->n_place[i] = n_host[p->order[i]];
+  const int sms = sm_count();
+  p->group = choose_group(p->n_place, sms);
+  if (p->group) {
+    p->grid = sms;  // also for fewer matrices: they then spread over the SMs
+    p->work = mpj_batched_groups_bytes(p->group, p->grid, p->n_place.front());
+    return;
+  }
   for (int p0 = 0; p0 < batch;) {
     Chunk c;
     memset(&c, 0, sizeof c);
@@ -327,7 +382,7 @@ int prepare(Device* d, int batch, const int* n_host, cudaStream_t s) {
     for (size_t limit = kChunkBytes;; limit = d->plan.work / 2) {
       make_plan(batch, n_host, limit, &d->plan);
       e = grow_device(&d->work, &d->work_bytes, d->plan.work);
-      if (e != cudaErrorMemoryAllocation || (int)d->plan.chunks.size() == batch) break;
+      if (e != cudaErrorMemoryAllocation || d->plan.group || (int)d->plan.chunks.size() == batch) break;
     }
     const size_t small = small_ptrs(nullptr, batch).total, pinned = sizeof(int) * ((size_t)batch + 2);
     if (e == cudaSuccess) e = grow_device(&d->small, &d->small_bytes, small);
@@ -460,8 +515,11 @@ int mpj_batched_rounds(int batch, const int* n_host, const double* const* A_dev,
   int st = prepare(d, batch, n_host, s);
   if (st != MPJ_OK) return st;
   const Small sm = small_ptrs((char*)d->small, batch);
-  MPJ_CUDA_TRY(cudaMemsetAsync(sm.flags, 0, sizeof(unsigned), s));
+  MPJ_CUDA_TRY(cudaMemsetAsync(sm.count, 0, 2 * sizeof(int), s));  // and the flags
   bool not_converged = false;
+  if (d->plan.group)
+    MPJ_CUDA_TRY(mpj_batched_groups(d->plan.group, d->plan.grid, d->plan.n_place.front(), sm.order, sm.n, A_dev, W_dev,
+                                    Q_dev, batch, tol, d->work, sm.count, sm.sweeps_out, sm.flags, s));
   for (const Chunk& c : d->plan.chunks) {
     st = run_chunk(*d, c, A_dev, W_dev, Q_dev, tol, &not_converged, s);
     if (st != MPJ_OK) break;
@@ -470,12 +528,11 @@ int mpj_batched_rounds(int batch, const int* n_host, const double* const* A_dev,
     (void)cudaStreamSynchronize(s);  // nothing of this call may still use the workspace
     return st;
   }
-  MPJ_CUDA_TRY(cudaMemcpyAsync(d->pinned + 1, sm.flags, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
-  MPJ_CUDA_TRY(cudaMemcpyAsync(d->pinned + 2, sm.sweeps_out, sizeof(int) * (size_t)batch, cudaMemcpyDeviceToHost, s));
+  MPJ_CUDA_TRY(cudaMemcpyAsync(d->pinned, sm.count, sizeof(int) * ((size_t)batch + 2), cudaMemcpyDeviceToHost, s));
   MPJ_CUDA_TRY(cudaStreamSynchronize(s));
   if (sweeps_host) memcpy(sweeps_host, d->pinned + 2, sizeof(int) * (size_t)batch);
   const unsigned flags = (unsigned)d->pinned[1];
   if (flags & MPJ_FLAG_NONFINITE) return MPJ_ENONFINITE;
-  if (flags & MPJ_FLAG_TIMEOUT) return MPJ_ETIMEOUT;
+  if (flags & MPJ_FLAG_TIMEOUT) return d->plan.group ? MPJ_NOT_CONVERGED : MPJ_ETIMEOUT;
   return not_converged ? MPJ_NOT_CONVERGED : MPJ_OK;
 }
