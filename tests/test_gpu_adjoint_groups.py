@@ -78,3 +78,20 @@ def test_leading_dimensions(m):
     assert np.isnan(got[:, :, n:]).all()
     for b, p in enumerate(ps):
         check(got[b, :, :n].T, oracle.eigh_backward(*p))
+
+
+def test_groups_of_a_ragged_size(m):
+    """n = 300: an operand is padded to 384 x 512, 3.1 MB, so 85 matrices fit in half
+    a GB and 91 split into two groups of unequal size."""
+    n, batch = 300, 91
+    ps = [problem(n, 70 + i) for i in range(4)]
+    W, Q, dW, dQ = (torch.from_numpy(np.stack([ps[b % 4][k] for b in range(batch)])).cuda() for k in range(4))
+    before = m.lib().mpj_kernel_launches()
+    m.syev_backward(W[:4], Q[:4], dW[:4], dQ[:4])
+    one = m.lib().mpj_kernel_launches() - before
+    dA = m.syev_backward(W, Q, dW, dQ)
+    assert m.lib().mpj_kernel_launches() - before == 3 * one  # one group, then two
+    for b in range(batch):
+        assert torch.equal(dA[b], dA[b % 4]), b
+    for i in range(4):
+        check(dA[i].cpu().numpy(), oracle.eigh_backward(*ps[i]))
