@@ -372,17 +372,19 @@ void make_plan(int batch, const int* n_host, size_t limit, Plan* p) {
 
 // The plan and its memory on the device.  Where the memory for chunks of
 // kChunkBytes cannot be had, the batch is cut into smaller ones (until other
-// sizes are planned or the memory is given back), down to single matrices.
+// sizes are planned or the memory is given back), down to the largest matrix alone.
 int prepare(Device* d, int batch, const int* n_host, cudaStream_t s) {
   const bool same = (int)d->plan.sizes.size() == batch &&
                     memcmp(d->plan.sizes.data(), n_host, sizeof(int) * (size_t)batch) == 0;
   if (!same || !d->uploaded) {
     d->uploaded = false;
     cudaError_t e = cudaSuccess;
-    for (size_t limit = kChunkBytes;; limit = d->plan.work / 2) {
+    for (size_t limit = kChunkBytes, last = ~(size_t)0;; limit = last / 2) {
       make_plan(batch, n_host, limit, &d->plan);
-      e = grow_device(&d->work, &d->work_bytes, d->plan.work);
-      if (e != cudaErrorMemoryAllocation || d->plan.group || (int)d->plan.chunks.size() == batch) break;
+      if (d->plan.work >= last) break;  // one matrix needs that much
+      last = d->plan.work;
+      e = grow_device(&d->work, &d->work_bytes, last);
+      if (e != cudaErrorMemoryAllocation) break;
     }
     const size_t small = small_ptrs(nullptr, batch).total, pinned = sizeof(int) * ((size_t)batch + 2);
     if (e == cudaSuccess) e = grow_device(&d->small, &d->small_bytes, small);
