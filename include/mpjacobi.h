@@ -45,9 +45,10 @@
  *                         the FP64 DMMA kernel instead of the tensor cores
  *                         (the exact bf16-slice products of mpj_dgemm_tc, the
  *                         default);
+ *                         (the batched solve heeds neither of these two);
  *   MPJ_BATCHED_GROUP=g   batched solve with one thread group per matrix (256,
- *                         512 or 1024 threads, anything else: autotuned)
- *                         instead of round by round (read on each call);
+ *                         512 or 1024 threads, anything else: autotuned) for
+ *                         all sizes (read on each call);
  *   MPJ_AUTOTUNE_CACHE=f  file that keeps the autotuned group-size choices.
  */
 #ifndef MPJACOBI_H
@@ -177,14 +178,14 @@ int mpj_syev_ex(int n, const double* A_dev, int lda, double* W_dev, double* Q_de
  * All matrices go through the rounds of a stage together, one launch per step
  * of a round, and those that have converged drop out; batches of small matrices
  * (all n_i <= 64, by an estimate of both) are solved with one thread group per
- * matrix in one launch.  The first call for a list
- * of sizes plans on the host (it orders the matrices by decreasing size).  The
- * workspace, at most about 6 GB, comes from cudaMalloc, grows to the largest
- * batch so far and is kept, one per device, until mpj_release_plans; larger
- * batches, and those for which that memory cannot be had, run in several parts.
- * Calls from several threads run one after the other.  Synchronizes `stream` (once
- * per sweep, to read how many matrices still need one, and at the end), so it
- * cannot be stream-captured.
+ * matrix in one launch.  A call with another list of sizes than the last plans
+ * on the host (it orders the matrices by decreasing size).  The workspace, at
+ * most about 6 GB, comes from cudaMalloc, grows to the largest batch so far and
+ * is kept, one per device, until mpj_release_plans; larger batches, and those
+ * for which that memory cannot be had, run in several parts.  Calls from several
+ * threads run one after the other.  Synchronizes `stream` (round by round once
+ * per sweep, to read how many matrices still need one; at the end), so it cannot
+ * be stream-captured.
  * With MPJ_BATCHED_GROUP set, one thread group solves each matrix whatever the
  * sizes; the plan then also keeps its workspace, the pointer arrays, the
  * group size (fixed, or picked by timing 256, 512 and 1024 threads on this

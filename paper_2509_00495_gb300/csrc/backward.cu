@@ -9,7 +9,7 @@
 // slices, ozaki.cu), each step one launch over a group of matrices: one n = 512
 // product has 32 output tiles for 152 SMs, and 18 launches per matrix over side
 // streams were bound by the host (64 matrices: 6.4 ms, 5.3 ms with the faster
-// products; grouped 4.9 ms).  With MPJ_GEMM_TC=0 they run on the FP64 DMMA
+// products; grouped 4.9 ms, 3.4 ms with kept scratch and whole-line slicing).  With MPJ_GEMM_TC=0 they run on the FP64 DMMA
 // kernel, batched over blockIdx.z (the last one as a lower-tile product).
 #include "common.cuh"
 #include "gemm64.cuh"

@@ -1,5 +1,5 @@
 // batch.cuh -- how the kernels of the single-matrix stages address a batch of
-// matrices with n <= 256 that go through their rounds together (batched.cu).
+// matrices with n <= 256 that go through their rounds together (batched_rounds.cu).
 //
 // The matrices are ordered by decreasing padded size N (n rounded up to a
 // multiple of 32, so there are eight classes); every buffer holds them one

@@ -297,7 +297,7 @@ MPJ_DEV void df_angle(float2 a, float2 d, float tie, float2& t, float2& c, float
 // method, 31 rounds of 16 disjoint pairs, Algorithm 2 with the skip test of
 // Algorithm 4) on the 32 x 32 subproblem, then one Newton-Schulz correction of
 // U_P and U_P's columns cut into digits for the tensor products.  Writes per
-// block pair: NSL digit tiles (32 x 32 bf16, K-major over the rows of U_P, one
+// block pair: NSL digit tiles (32 x 32 binary16, K-major over the rows of U_P, one
 // "row" per column of U_P), 32 column exponents, and whether any rotation
 // happened (when none did, U_P = I and only that flag is written).
 //
@@ -538,10 +538,10 @@ struct BatchSub64 {  // the block pairs of a batch
     return true;
   }
 };
-// CTAS: resident CTAs per SM the registers are limited for.  One (78 registers)
-// has the shorter latency and is taken when every subproblem of a round finds
-// its own SM; beyond that two (48 registers) have the higher rate: 16 against 21
-// us per subproblem and SM.
+// CTAS: resident CTAs per SM the registers are limited for.  One (80 registers, 82
+// in a batch) has the shorter latency and is taken when every subproblem of a round
+// finds its own SM; beyond that two (48 registers, two of them spilled for a single
+// matrix) have the higher rate: 16 against 21 us per subproblem and SM.
 template <int CTAS, class Src>
 __global__ void __launch_bounds__(SOLVE_THREADS, CTAS) blk_solve(Src src, int R, double skip) {
   __shared__ __align__(16) SolveSmem sm;

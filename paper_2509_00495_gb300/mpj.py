@@ -326,6 +326,7 @@ class BatchedSolver:
         return self.W, [q.T for q in self.Qt], list(sweeps), st
 
     def group_size(self) -> int:
+        """The group size that tuning chose for these sizes (MPJ_BATCHED_GROUP), 0 if none was tuned."""
         return int(lib().mpj_batched_group_size(len(self.sizes), self.ns))
 
 
