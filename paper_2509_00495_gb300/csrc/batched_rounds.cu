@@ -53,7 +53,11 @@ struct State {  // by place
   int* sweeps;
 };
 
-// ||A||_F, tolerances, A32 = fl32(A) and V32 = I padded to N
+// ||A||_F, tolerances, A32 = fl32(A 2^-e) and V32 = I padded to N.  e = 0 unless
+// ||A||_F is below 2^-24 or above 2^24: the FP32 sweeps compare squares of entries,
+// which leave FP32's range for matrices of 1e-23 and 1e19 (entries themselves
+// beyond 1e-38 and 1e38); e = log2 ||A||_F there.  The FP32 rotations do not depend
+// on a power of two.
 __global__ void __launch_bounds__(BT) batch_init(BatchShape b, const double* const* __restrict__ Aptr,
                                                  const int* __restrict__ order, double tol_in, float* __restrict__ A32,
                                                  float* __restrict__ V32, State st, unsigned* __restrict__ flags) {
@@ -74,10 +78,19 @@ __global__ void __launch_bounds__(BT) batch_init(BatchShape b, const double* con
   }
   if (bad) atomicOr(flags, MPJ_FLAG_NONFINITE);
   s = cta_sum(s, red);
+  const double norm = sqrt(s);
+  double scale = 1.0;
+  if (norm > 0.0 && isfinite(norm) && (norm < 0x1p-24 || norm > 0x1p24)) {
+    scale = __hiloint2double((2046 - ((__double2hiint(norm) >> 20) & 0x7FF)) << 20, 0);
+    for (int e = threadIdx.x; e < N * N; e += BT) {
+      const int i = e % N, j = e / N;
+      if (i < n && j < n) A32[t.el + e] = (float)(A[(size_t)j * n + i] * scale);
+    }
+  }
   if (threadIdx.x == 0) {
-    const double norm = sqrt(s), tol = tol_in > 0 ? tol_in : (double)n * 0x1p-53 * norm;
+    const double tol = tol_in > 0 ? tol_in : (double)n * 0x1p-53 * norm;
     st.tol[t.place] = tol;
-    st.tol32[t.place] = (double)n * 0x1p-24 * norm;
+    st.tol32[t.place] = (double)n * 0x1p-24 * (norm * scale);
     st.skip_abs[t.place] = tol / n;
     st.sweeps[t.place] = 0;
   }

@@ -76,3 +76,16 @@ def test_new_buffers_on_a_kept_plan_and_a_nonfinite_neighbour(m):
         solver.solve([torch.from_numpy(a).cuda() for a in bad])
     assert e.value.status == m.MPJ_ENONFINITE
     check([mats[0], mats[2]], [solver.W[0], solver.W[2]], [solver.Qt[0].T, solver.Qt[2].T])
+
+
+@pytest.mark.parametrize("e", [-400, -126, -75, -30, 30, 60, 126, 400])
+def test_scales(m, e):
+    """2^e A rotates as A does, also where FP32 (or its squares) cannot hold 2^e: the
+    same sweeps and the same vectors, the eigenvalues times 2^e."""
+    rng = np.random.default_rng(11)
+    mats = [goe(n, rng) for n in (40, 70, 130, 250)]
+    W, Q, sweeps, st = m.syev_batched([torch.from_numpy(a).cuda() for a in mats])
+    W2, Q2, sweeps2, st2 = m.syev_batched([torch.from_numpy(a * 2.0 ** e).cuda() for a in mats])
+    assert st == 0 and st2 == 0 and sweeps == sweeps2
+    assert all(torch.equal(a, b) for a, b in zip(Q, Q2))
+    assert all(torch.equal(a * 2.0 ** e, b) for a, b in zip(W, W2))
